@@ -255,15 +255,14 @@ __global__ void k_fixed_to_complex(const unsigned long long* __restrict__ in, do
 // row per grid cell: the strength index a * n_det + (k mod n_det) of every contributing
 // sample and its kernel weight psi(x) psi(y).  Entries of a row are sorted by strength index,
 // so every later gather sums in a fixed order (deterministic) and needs no atomics.
-__global__ void k_csr_count(const double* __restrict__ angles, int na, int nd, int nf, int W, int* __restrict__ cnt) {
+__global__ void k_csr_count(const double2* __restrict__ cs, int na, int nd, int nf, int W, int* __restrict__ cnt) {
   const int npa = nd - 1;
   const size_t total = (size_t)na * npa;
   for (size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x; id < total; id += (size_t)gridDim.x * blockDim.x) {
     const int kk = (int)(id % npa), a = (int)(id / npa);
     const int k = kk - (nd / 2 - 1);
-    double sa, ca;
-    sincos(angles[a], &sa, &ca);
-    const double ux = (double)k * ca * nf / nd, uy = (double)k * sa * nf / nd;
+    const double2 e = cs[a];
+    const double ux = (double)k * e.x * nf / nd, uy = (double)k * e.y * nf / nd;
     const int lx0 = (int)ceil(ux - 0.5 * W), ly0 = (int)ceil(uy - 0.5 * W);
     for (int jy = 0; jy < W; ++jy)
       for (int jx = 0; jx < W; ++jx) {
@@ -272,45 +271,152 @@ __global__ void k_csr_count(const double* __restrict__ angles, int na, int nd, i
       }
   }
 }
-__global__ void k_csr_fill(const double* __restrict__ angles, int na, int nd, int nf, int W, double beta,
-                           int* __restrict__ cursor, int* __restrict__ idx, double* __restrict__ wt) {
+// Fills the rows (unordered) with one warp per sample: lanes 0 .. W - 1 evaluate the kernel at the
+// sample's W columns, lanes 16 .. 16 + W - 1 at its W rows, and the W^2 entries take their two
+// factors from shared memory.  The FP64 pipe is 1/64 of the FP32 one, so the count of FP64
+// exponentials bounds this kernel: one thread per sample evaluating every entry took W^2 + W of
+// them per sample.  cs: (cos, sin) of every angle.  Measured at 512^2, 181 angles, both widths:
+// 2.74 ms before.
+template <int W>
+__global__ void __launch_bounds__(256) k_csr_fill(const double2* __restrict__ cs, int na, int nd, int nf, double beta,
+                                                  int* __restrict__ cursor, int* __restrict__ idx,
+                                                  double* __restrict__ wt) {
+  static_assert(W <= 16, "a warp evaluates both axes at once");
+  __shared__ double fac[8][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int npa = nd - 1;
-  const size_t total = (size_t)na * npa;
-  for (size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x; id < total; id += (size_t)gridDim.x * blockDim.x) {
-    const int kk = (int)(id % npa), a = (int)(id / npa);
+  const int total = na * npa;
+  for (int id = blockIdx.x * 8 + warp; id < total; id += gridDim.x * 8) {
+    const int kk = id % npa, a = id / npa;
     const int k = kk - (nd / 2 - 1);
-    double sa, ca;
-    sincos(angles[a], &sa, &ca);
-    const double ux = (double)k * ca * nf / nd, uy = (double)k * sa * nf / nd;
+    const double2 e = cs[a];
+    const double ux = (double)k * e.x * nf / nd, uy = (double)k * e.y * nf / nd;
     const int lx0 = (int)ceil(ux - 0.5 * W), ly0 = (int)ceil(uy - 0.5 * W);
     const int sidx = a * nd + (k < 0 ? k + nd : k);
-    for (int jy = 0; jy < W; ++jy) {
-      const double wy = es_kernel((2.0 * (ly0 + jy - uy)) / W, beta);
-      for (int jx = 0; jx < W; ++jx) {
-        const int ly = (ly0 + jy + nf) % nf, lx = (lx0 + jx + nf) % nf;
-        const int pos = atomicAdd(&cursor[(size_t)ly * nf + lx], 1);
-        idx[pos] = sidx;
-        wt[pos] = wy * es_kernel((2.0 * (lx0 + jx - ux)) / W, beta);
-      }
+    const int j = lane & 15;
+    if (j < W) fac[warp][lane] = es_kernel((2.0 * ((lane < 16 ? lx0 + j - ux : ly0 + j - uy))) / W, beta);
+    __syncwarp();
+    for (int q = lane; q < W * W; q += 32) {
+      const int jy = q / W, jx = q - jy * W;
+      const int ly = (ly0 + jy + nf) % nf, lx = (lx0 + jx + nf) % nf;
+      const int pos = atomicAdd(&cursor[(size_t)ly * nf + lx], 1);
+      idx[pos] = sidx;
+      wt[pos] = fac[warp][16 + jy] * fac[warp][jx];
+    }
+    __syncwarp();
+  }
+}
+
+// ---- rows sorted by strength index (the indices of a row are distinct)
+// Rows are short (tens of entries) except near the grid's centre, where the samples crowd (row
+// lengths fall like 1 / radius from about 11 per angle).  A warp ranks a row of up to 256 entries:
+// each entry's place is the number of smaller indices, counted from registers, and the row is
+// rewritten from registers.  Longer rows go to a list that whole blocks sort by a bitonic network,
+// in shared memory where they fit and in place otherwise.  One thread per row by insertion took
+// 267 ms at 512^2 with 181 angles: thousands of dependent moves by the few threads at the centre.
+constexpr int kRankMax = 256;
+constexpr int kSortSmem = 4096;  // entries a block sorts in shared memory (48 KB)
+
+template <int Q>
+__device__ __forceinline__ void rank_row(int b, int n, int lane, int* idx, double* wt) {
+  int key[Q], rank[Q];
+  double w[Q];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    const int j = lane + 32 * q;
+    key[q] = j < n ? idx[b + j] : 0x7fffffff;
+    w[q] = j < n ? wt[b + j] : 0.0;
+    rank[q] = 0;
+  }
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    for (int l = 0; l < 32; ++l) {
+      const int o = __shfl_sync(0xffffffffu, key[q], l);
+#pragma unroll
+      for (int r = 0; r < Q; ++r) rank[r] += o < key[r] ? 1 : 0;
+    }
+  }
+  __syncwarp();  // every lane's entries are in registers
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    if (lane + 32 * q < n) {
+      idx[b + rank[q]] = key[q];
+      wt[b + rank[q]] = w[q];
     }
   }
 }
-// insertion sort of each row by strength index (rows are short except near the centre)
-__global__ void k_csr_sort(const int* __restrict__ ptr, int ncells, int* __restrict__ idx, double* __restrict__ wt) {
-  for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < ncells; cell += gridDim.x * blockDim.x) {
-    const int b = ptr[cell], e = ptr[cell + 1];
-    for (int i = b + 1; i < e; ++i) {
-      const int ki = idx[i];
-      const double wi = wt[i];
-      int j = i - 1;
-      while (j >= b && idx[j] > ki) {
-        idx[j + 1] = idx[j];
-        wt[j + 1] = wt[j];
-        --j;
-      }
-      idx[j + 1] = ki;
-      wt[j + 1] = wi;
+__global__ void __launch_bounds__(256) k_csr_rank(const int* __restrict__ ptr, int ncells, int* idx, double* wt,
+                                                  int* __restrict__ longs, int* __restrict__ nlongs) {
+  const int lane = threadIdx.x & 31;
+  for (int cell = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; cell < ncells; cell += (gridDim.x * blockDim.x) >> 5) {
+    const int b = ptr[cell], n = ptr[cell + 1] - b;
+    if (n < 2) continue;
+    if (n <= 32)
+      rank_row<1>(b, n, lane, idx, wt);
+    else if (n <= 64)
+      rank_row<2>(b, n, lane, idx, wt);
+    else if (n <= 128)
+      rank_row<4>(b, n, lane, idx, wt);
+    else if (n <= kRankMax)
+      rank_row<8>(b, n, lane, idx, wt);
+    else if (lane == 0)
+      longs[atomicAdd(nlongs, 1)] = cell;
+  }
+}
+// Bitonic sort of n entries by one block, every comparison ascending (the first step of each merge
+// pairs i with its mirror image), so positions past n act as keys above all others and are skipped.
+__device__ __forceinline__ void block_bitonic(int n, int* key, double* w) {
+  auto cmp = [&](int i, int j) {
+    if (j < n && key[i] > key[j]) {
+      const int t = key[i];
+      key[i] = key[j];
+      key[j] = t;
+      const double u = w[i];
+      w[i] = w[j];
+      w[j] = u;
     }
+  };
+  int half = 1;
+  while (half < n) half <<= 1;
+  half >>= 1;  // pairs per step: half of n rounded up to a power of two
+  for (int size = 2; size <= 2 * half; size <<= 1) {
+    for (int i = threadIdx.x; i < half; i += blockDim.x) {
+      const int o = i % (size / 2), base = (i / (size / 2)) * size;
+      cmp(base + o, base + size - 1 - o);
+    }
+    __syncthreads();
+    for (int st = size / 4; st > 0; st >>= 1) {
+      for (int i = threadIdx.x; i < half; i += blockDim.x) {
+        const int o = i % st, base = (i / st) * 2 * st;
+        cmp(base + o, base + o + st);
+      }
+      __syncthreads();
+    }
+  }
+}
+__global__ void __launch_bounds__(256) k_csr_sort_long(const int* __restrict__ ptr, int* idx, double* wt,
+                                                       const int* __restrict__ longs, const int* __restrict__ nlongs) {
+  extern __shared__ double sort_sm[];
+  double* w = sort_sm;
+  int* key = reinterpret_cast<int*>(sort_sm + kSortSmem);
+  const int count = *nlongs;
+  for (int i = blockIdx.x; i < count; i += gridDim.x) {
+    const int b = ptr[longs[i]], n = ptr[longs[i] + 1] - b;
+    if (n > kSortSmem) {
+      block_bitonic(n, idx + b, wt + b);
+      continue;
+    }
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+      key[j] = idx[b + j];
+      w[j] = wt[b + j];
+    }
+    __syncthreads();
+    block_bitonic(n, key, w);
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+      idx[b + j] = key[j];
+      wt[b + j] = w[j];
+    }
+    __syncthreads();
   }
 }
 // inclusive scan, three phases over tiles of 2048 ints
@@ -663,7 +769,7 @@ size_t setup_scratch_bytes(const tmbir_group& g) {
   const size_t k_elems = kernel_direct(g.N) ? nf_k + 2 * M * M + (size_t)g.n_angles : nf_k + 2 * nf_k * nf_k;
   // R*g in FP64 on grid 1; the FP32 back-projection of the direct operators on grid 0
   const size_t a_bytes = std::max(backproject_elems(g, 1) * sizeof(double2), backproject_elems(g, 0) * sizeof(float2));
-  const size_t csr_build = (nf0 * nf0 + 2 * ((nf0 * nf0 + 2048) / 2048 + 1)) * sizeof(int);
+  const size_t csr_build = (nf0 * nf0 + 2 * ((nf0 * nf0 + 2048) / 2048 + 1)) * sizeof(int) + (size_t)g.n_angles * sizeof(double2);
   return std::max(std::max(std::max(k_elems * sizeof(double2), a_bytes), csr_build) + 256, forward_scratch_bytes(g));
 }
 size_t fbp_scratch_bytes(const tmbir_group& g) { return backproject_elems(g, 0) * sizeof(float2) + 256; }
@@ -769,13 +875,16 @@ int build_spread_matrix(Ctx& c, int gi) {
   cudaStream_t s = c.stream;
   const size_t total = (size_t)g.na * (g.nd - 1);
   const int blocks = (int)std::min<size_t>((total + 255) / 256, 152 * 16);
+  double2* cs = reinterpret_cast<double2*>(c.scratch);
+  k_angle_table<<<(g.na + 255) / 256, 256, 0, s>>>(g.angles, g.na, cs);
+  TMBIR_CHECK_LAUNCH();
   for (int k = 0; k < 2; ++k) {
     GroupDev::Spread& sp = g.sp[k];
     const int nf = sp.nf, ncells = nf * nf, W = kSpreadWidth[k];
-    int* cursor = reinterpret_cast<int*>(c.scratch);
+    int* cursor = reinterpret_cast<int*>(cs + g.na);
     int* sums = cursor + ncells;
     TMBIR_CUDA(cudaMemsetAsync(sp.ptr, 0, sizeof(int) * (ncells + 1), s));
-    k_csr_count<<<blocks, 256, 0, s>>>(g.angles, g.na, g.nd, nf, W, sp.ptr);
+    k_csr_count<<<blocks, 256, 0, s>>>(cs, g.na, g.nd, nf, W, sp.ptr);
     TMBIR_CHECK_LAUNCH();
     const int ntiles = (ncells + 1 + 2047) / 2048;
     k_scan_tiles<<<ntiles, 256, 0, s>>>(sp.ptr, ncells + 1, sums);
@@ -785,9 +894,17 @@ int build_spread_matrix(Ctx& c, int gi) {
     k_scan_add<<<1024, 256, 0, s>>>(sp.ptr, ncells + 1, sums);
     TMBIR_CHECK_LAUNCH();
     TMBIR_CUDA(cudaMemcpyAsync(cursor, sp.ptr, sizeof(int) * ncells, cudaMemcpyDeviceToDevice, s));
-    k_csr_fill<<<blocks, 256, 0, s>>>(g.angles, g.na, g.nd, nf, W, spread_beta(k), cursor, sp.idx, sp.wt);
+    const int fill_blocks = (int)std::min<size_t>((total + 7) / 8, 152 * 32);
+    if (k == 0)
+      k_csr_fill<kSpreadWidth[0]><<<fill_blocks, 256, 0, s>>>(cs, g.na, g.nd, nf, spread_beta(k), cursor, sp.idx, sp.wt);
+    else
+      k_csr_fill<kSpreadWidth[1]><<<fill_blocks, 256, 0, s>>>(cs, g.na, g.nd, nf, spread_beta(k), cursor, sp.idx, sp.wt);
     TMBIR_CHECK_LAUNCH();
-    k_csr_sort<<<(ncells + 255) / 256, 256, 0, s>>>(sp.ptr, ncells, sp.idx, sp.wt);
+    // the cursors and the scan's sums have been used: the list of long rows and its length
+    TMBIR_CUDA(cudaMemsetAsync(sums, 0, sizeof(int), s));
+    k_csr_rank<<<std::min((ncells + 7) / 8, 152 * 32), 256, 0, s>>>(sp.ptr, ncells, sp.idx, sp.wt, cursor, sums);
+    TMBIR_CHECK_LAUNCH();
+    k_csr_sort_long<<<152 * 4, 256, kSortSmem * 12, s>>>(sp.ptr, sp.idx, sp.wt, cursor, sums);
     TMBIR_CHECK_LAUNCH();
     if (k == 1) {  // R*g runs in double-word FP32: its weights as (hi, lo) pairs
       k_wt_to_df<<<1024, 256, 0, s>>>(sp.wt, spread_nnz(c.groups[gi], 1));
