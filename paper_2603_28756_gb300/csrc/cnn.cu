@@ -39,7 +39,8 @@ constexpr int kStageAPad = (kStageA + 127) / 128 * 128;
 constexpr int kWElems = 9 * 4 * kC * 8;           // packed 32 -> 32 weights [tap][chunk][n][8]
 constexpr int kConvSmem = kStageAPad + kWElems * 2;  // staged rows + weights
 constexpr uint32_t kMmaPolls = 1u << 22;          // bound of every wait on an MMA completion
-constexpr int kWgradBlocks = 304;      // blocks of the weight-gradient reductions
+constexpr int kWgradBlocks = 304;      // most blocks of the weight-gradient reductions: two per SM
+constexpr int kPartRow = kW1 + kB1;    // one block's partial sums
 
 struct CnnNet {
   cudaStream_t stream;
@@ -62,7 +63,7 @@ struct CnnNet {
   float* out;           // [B][H][W] network output
   float* gout;          // [B][H][W]
   float* sig;           // [B] per-image scale
-  float* wpart;         // [kWgradBlocks][kW1] weight-gradient partials
+  float* wpart;         // [kWgradBlocks][kPartRow] weight-gradient partials
   double* dpart;        // scalar partials
   int step;
 };
@@ -278,13 +279,17 @@ __global__ void __launch_bounds__(256) k_conv_first(const float* __restrict__ x,
 // with T[q][tap] = sum_ci w3[ci][tap] a2[q][ci]: a block computes T once per pixel of its 8 x 32
 // tile plus a one-pixel halo (each activation vector read once) and sums the nine shifted
 // entries from shared memory.
+// DGRAD: the data gradient of layer 0, gin[p] = sum_{tap, co} w0[co][tap] g0[p - tap][co]: the same
+// sums with layer 0's weights, the taps flipped and no bias.
 constexpr int kLH = 8, kLW = 32;
+template <bool DGRAD>
 __global__ void __launch_bounds__(256, 2) k_conv_last(const __nv_bfloat16* __restrict__ a2, int B, int H, int W,
                                                       const float* __restrict__ master, float* __restrict__ out) {
   __shared__ __align__(16) float w[kC][12];  // w3[ci][tap], rows padded to 12 for 16-byte vector reads
   __shared__ float T[(kLH + 2) * (kLW + 2)][9];
-  for (int i = threadIdx.x; i < kC * 9; i += blockDim.x) w[i / 9][i % 9] = master[kOff3 + i];
-  const float b3 = master[kOff3 + kW3];
+  for (int i = threadIdx.x; i < kC * 9; i += blockDim.x)
+    w[i / 9][DGRAD ? 8 - i % 9 : i % 9] = master[(DGRAD ? kOff0 : kOff3) + i];
+  const float b3 = DGRAD ? 0.f : master[kOff3 + kW3];
   const int tiles_x = (W + kLW - 1) / kLW, tiles_y = (H + kLH - 1) / kLH;
   const int tpi = tiles_x * tiles_y;
   for (int tile = blockIdx.x; tile < B * tpi; tile += gridDim.x) {
@@ -368,141 +373,259 @@ __global__ void k_last_dgrad(const float* __restrict__ gout, const __nv_bfloat16
 }
 
 // ---------------------------------------------------------------- weight gradients (fixed-order block partials)
-// Layer 1/2: dW[co][ci][tap] = sum_p g[p][co] in[p + tap][ci]; thread t owns co = t / 8 and
-// ci = 4 (t % 8) .. +3 for all 9 taps (36 sums); pixels in a fixed grid-stride order.
-__global__ void __launch_bounds__(256) k_wgrad32(const __nv_bfloat16* __restrict__ g, const __nv_bfloat16* __restrict__ in,
-                                                 int B, int H, int W, float* __restrict__ part) {
-  const int co = threadIdx.x >> 3, ci0 = (threadIdx.x & 7) * 4;
-  float s[4][9];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int t = 0; t < 9; ++t) s[i][t] = 0.f;
-  const size_t total = (size_t)B * H * W;
-  for (size_t p = blockIdx.x; p < total; p += gridDim.x) {
-    const int xx = (int)(p % W), yy = (int)((p / W) % H);
-    const size_t b = p / ((size_t)H * W);
-    const float gv = __bfloat162float(g[p * kC + co]);
-#pragma unroll
-    for (int t = 0; t < 9; ++t) {
-      const int gy = yy + t / 3 - 1, gx = xx + t % 3 - 1;
-      if (gy < 0 || gy >= H || gx < 0 || gx >= W) continue;
-      const __nv_bfloat162* a = reinterpret_cast<const __nv_bfloat162*>(in + ((b * H + gy) * W + gx) * kC + ci0);
-      const float2 v0 = __bfloat1622float2(a[0]), v1 = __bfloat1622float2(a[1]);
-      s[0][t] = fmaf(gv, v0.x, s[0][t]);
-      s[1][t] = fmaf(gv, v0.y, s[1][t]);
-      s[2][t] = fmaf(gv, v1.x, s[2][t]);
-      s[3][t] = fmaf(gv, v1.y, s[3][t]);
-    }
-  }
-  float* o = part + (size_t)blockIdx.x * kW1;
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int t = 0; t < 9; ++t) o[(co * kC + ci0 + i) * 9 + t] = s[i][t];
-}
+// Layers 1, 2: dW[co][ci][tap] = sum_p g[p][co] in[p + tap][ci] and db[co] = sum_p g[p][co], as a
+// GEMM over the pixels on the tensor cores.  The images' channel-last layout makes the channels of a
+// pixel contiguous and the pixels the contraction index, which is the MMA's MN-major operand layout
+// with the staging of the forward convolution ([row][8-channel chunk][pixel][8]):
+//   A (M = 128): the 32 channels of four consecutive rows of g, rows y - 1 .. y + 2 against input
+//      row y: three of the four are the taps dy = +1, 0, -1 (the fourth is not used);
+//   B (N = 32):  input row y shifted by dx pixels (16 bytes), one MMA per dx; the centre one takes
+//      N = 48 with 16 further columns of ones, whose products are the bias gradient.
+// A tile is kGRows input rows x 128 pixels (8 K-steps of 16 pixels per row), accumulated in TMEM and
+// then added to FP32 registers, thread = (dy, co), 96 sums: the tensor core's accumulator is not
+// rounded to nearest, so its chains are kept to 32 K-steps, which leaves the sums nearer to 64 bits
+// than one FP32 chain per thread over all pixels.
+// Bound by the operand reads from shared memory (4 KB of A per MMA) and by the two activation
+// streams (128 B per pixel); the CUDA-core form this replaced read every pixel's nine neighbours
+// in every thread: 76 ms at 8 x 1024^2.
+constexpr int kGRows = 4;
+constexpr int kGRowB = 4 * kTM * 16;               // bytes of one staged row of g
+constexpr int kGInB = 6 * kChunkB;                 // one staged input row: four chunks, ones, zeros
+constexpr int kGSmemG = (kGRows + 3) * kGRowB;     // rows y0 - 1 .. y0 + kGRows + 1 (the last stays zero)
+constexpr int kGradSmem = kGSmemG + kGRows * kGInB;
+constexpr int kGCols = 112;                        // D columns: dx 0 | dx 1, ones | dx 2
 
-// Layer 0: dW0[co][tap] = sum_p g0[p][co] xin[p + tap], db0[co] = sum_p g0[p][co];
-// thread t: co = t % 32, taps 3 (t / 32) .. +2 for t < 96, bias for 96 <= t < 128.
-// Partial row layout: [0, 288) dW0, [288, 320) db0.
-__global__ void __launch_bounds__(128) k_wgrad_first(const __nv_bfloat16* __restrict__ g0, const float* __restrict__ xin,
-                                                     int B, int H, int W, float* __restrict__ part) {
-  const int co = threadIdx.x & 31, role = threadIdx.x >> 5;
-  float acc[3] = {0.f, 0.f, 0.f};
-  const size_t total = (size_t)B * H * W;
-  for (size_t p = blockIdx.x; p < total; p += gridDim.x) {
-    const float gv = __bfloat162float(g0[p * kC + co]);
-    if (role == 3) {
-      acc[0] += gv;
-      continue;
-    }
-    const int xx = (int)(p % W), yy = (int)((p / W) % H);
-    const size_t b = p / ((size_t)H * W);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const int t = role * 3 + j;
-      const int gy = yy + t / 3 - 1, gx = xx + t % 3 - 1;
-      if (gy >= 0 && gy < H && gx >= 0 && gx < W) acc[j] = fmaf(gv, xin[(b * H + gy) * W + gx], acc[j]);
-    }
+__global__ void __launch_bounds__(128) k_wgrad32(const __nv_bfloat16* __restrict__ g, const __nv_bfloat16* __restrict__ in,
+                                                 int B, int H, int W, float* __restrict__ part, int* err) {
+  namespace tc = tc05;
+  extern __shared__ __align__(128) unsigned char smraw[];
+  unsigned char* sg = smraw;
+  unsigned char* si = smraw + kGSmemG;
+  __shared__ uint64_t bar;
+  __shared__ uint32_t tmem_base;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp == 0) tc::tmem_alloc<128>(&tmem_base);
+  if (threadIdx.x == 0) {
+    tc::mbar_init(&bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  float* o = part + (size_t)blockIdx.x * kW1;
-  if (role < 3) {
-#pragma unroll
-    for (int j = 0; j < 3; ++j) o[co * 9 + role * 3 + j] = acc[j];
-  } else {
-    o[288 + co] = acc[0];
+  // the parts that staging never writes: the ones and zeros of every input row, the last row of g
+  for (int i = threadIdx.x; i < kGRows * 2 * kTX; i += blockDim.x) {
+    const int r = i / (2 * kTX), c = (i / kTX) & 1, px = i % kTX;
+    const uint32_t one2 = 0x3f803f80u;
+    const uint4 v = c == 0 ? make_uint4(one2, one2, one2, one2) : make_uint4(0, 0, 0, 0);
+    *reinterpret_cast<uint4*>(si + r * kGInB + (4 + c) * kChunkB + px * 16) = v;
   }
-}
-// Hidden-layer bias: db[co] = sum_p g[p][co]; partial row [0, 32)
-__global__ void __launch_bounds__(32) k_bias_grad(const __nv_bfloat16* __restrict__ g, size_t total, float* __restrict__ part) {
-  float acc = 0.f;
-  for (size_t p = blockIdx.x; p < total; p += gridDim.x) acc += __bfloat162float(g[p * kC + threadIdx.x]);
-  part[(size_t)blockIdx.x * kW1 + threadIdx.x] = acc;
-}
-// Layer 3: dW3[ci][tap] = sum_p gout[p] a2[p + tap][ci], db3 = sum_p gout[p];
-// thread t < 32: ci = t, all taps; thread 32: bias.  Partial row [0, 288) dW3, [288] db3.
-__global__ void __launch_bounds__(64) k_wgrad_last(const float* __restrict__ gout, const __nv_bfloat16* __restrict__ a2,
-                                                   int B, int H, int W, float* __restrict__ part) {
-  const int ci = threadIdx.x;
-  float acc[9];
-#pragma unroll
-  for (int t = 0; t < 9; ++t) acc[t] = 0.f;
-  const size_t total = (size_t)B * H * W;
-  for (size_t p = blockIdx.x; p < total; p += gridDim.x) {
-    const float gv = gout[p];
-    if (ci == 32) {
-      acc[0] += gv;
-      continue;
-    }
-    if (ci > 32) continue;
-    const int xx = (int)(p % W), yy = (int)((p / W) % H);
-    const size_t b = p / ((size_t)H * W);
-#pragma unroll
-    for (int t = 0; t < 9; ++t) {
-      const int gy = yy + t / 3 - 1, gx = xx + t % 3 - 1;
-      if (gy >= 0 && gy < H && gx >= 0 && gx < W)
-        acc[t] = fmaf(gv, __bfloat162float(a2[((b * H + gy) * W + gx) * kC + ci]), acc[t]);
-    }
-  }
-  float* o = part + (size_t)blockIdx.x * kW1;
-  if (ci < 32) {
-#pragma unroll
-    for (int t = 0; t < 9; ++t) o[ci * 9 + t] = acc[t];
-  } else if (ci == 32) {
-    o[288] = acc[0];
-  }
-}
-// gin[p] = sum_{tap, co} w0[co][tap] g0[p - tap][co]
-__global__ void k_first_dgrad(const __nv_bfloat16* __restrict__ g0, int B, int H, int W, const float* __restrict__ master,
-                              float* __restrict__ gin) {
-  __shared__ float w[kW0];
-  for (int i = threadIdx.x; i < kW0; i += blockDim.x) w[i] = master[kOff0 + i];
+  for (int i = threadIdx.x; i < kGRowB / 16; i += blockDim.x)
+    *reinterpret_cast<uint4*>(sg + (kGRows + 2) * kGRowB + i * 16) = make_uint4(0, 0, 0, 0);
+  tc::fence_before_sync();
   __syncthreads();
-  const size_t total = (size_t)B * H * W;
-  for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < total; p += (size_t)gridDim.x * blockDim.x) {
-    const int xx = (int)(p % W), yy = (int)((p / W) % H);
-    const size_t b = p / ((size_t)H * W);
-    float s = 0.f;
-#pragma unroll 1
-    for (int t = 0; t < 9; ++t) {
-      const int gy = yy - (t / 3 - 1), gx = xx - (t % 3 - 1);
-      if (gy < 0 || gy >= H || gx < 0 || gx >= W) continue;
-      const __nv_bfloat162* gg = reinterpret_cast<const __nv_bfloat162*>(g0 + ((b * H + gy) * W + gx) * kC);
+  tc::fence_after_sync();
+  const uint32_t tmem = tmem_base;
+  // MN-major: M (N) chunks of 8 channels lie sbo apart, groups of 8 pixels lbo = 128 bytes apart
+  const uint64_t a_desc = tc::smem_desc(tc::smem_addr(sg), 128, kTM * 16);
+  const uint64_t b_desc = tc::smem_desc(tc::smem_addr(si), 128, kChunkB);
+  constexpr uint32_t ID32 = tc::idesc_bf16_f32_mn<128, 32>(), ID48 = tc::idesc_bf16_f32_mn<128, 48>();
+  const int tiles_x = (W + kTM - 1) / kTM, tiles_y = (H + kGRows - 1) / kGRows;
+  const int ntiles = B * tiles_y * tiles_x;
+  float acc[3 * kC], accb = 0.f;
 #pragma unroll
-      for (int c = 0; c < kC; c += 2) {
-        const float2 v = __bfloat1622float2(gg[c / 2]);
-        s = fmaf(w[c * 9 + t], v.x, s);
-        s = fmaf(w[(c + 1) * 9 + t], v.y, s);
+  for (int i = 0; i < 3 * kC; ++i) acc[i] = 0.f;
+  uint32_t parity = 0;
+  bool failed = false;
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int tx = tile % tiles_x, ty = (tile / tiles_x) % tiles_y, b = tile / (tiles_x * tiles_y);
+    const int y0 = ty * kGRows, x0 = tx * kTM;
+    {
+      const int gx = x0 + threadIdx.x;
+#pragma unroll
+      for (int r = 0; r < kGRows + 2; ++r) {
+        const int gy = y0 - 1 + r;
+        const bool v = gx < W && gy >= 0 && gy < H;
+        const __nv_bfloat16* src = v ? g + (((size_t)b * H + gy) * W + gx) * kC : g;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          tc::cp_async16(sg + r * kGRowB + j * (kTM * 16) + threadIdx.x * 16, v ? src + 8 * j : g, v);
       }
     }
-    gin[p] = s;
+    for (int px = threadIdx.x; px < kTX; px += blockDim.x) {
+      const int gx = x0 - 1 + px;
+#pragma unroll
+      for (int r = 0; r < kGRows; ++r) {
+        const int gy = y0 + r;
+        const bool v = gx >= 0 && gx < W && gy < H;
+        const __nv_bfloat16* src = v ? in + (((size_t)b * H + gy) * W + gx) * kC : in;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) tc::cp_async16(si + r * kGInB + j * kChunkB + px * 16, v ? src + 8 * j : in, v);
+      }
+    }
+    tc::cp_async_wait_all();
+    tc::fence_async_shared();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      tc::fence_after_sync();
+#pragma unroll 1
+      for (int r = 0; r < kGRows; ++r) {
+#pragma unroll
+        for (int s = 0; s < kTM / 16; ++s) {
+          const uint64_t ad = a_desc + (uint64_t)((r * kGRowB + s * 256) >> 4);
+          const uint64_t bd = b_desc + (uint64_t)((r * kGInB + s * 256) >> 4);
+          const uint32_t more = (r | s) ? 1u : 0u;
+          tc::mma_bf16(tmem, ad, bd, ID32, more);
+          tc::mma_bf16(tmem + 32, ad, bd + 1, ID48, more);
+          tc::mma_bf16(tmem + 80, ad, bd + 2, ID32, more);
+        }
+      }
+      tc::mma_commit(&bar);
+    }
+    const bool ok = tc::mbar_wait(&bar, parity, kMmaPolls);
+    parity ^= 1u;
+    if (__syncthreads_or(!ok)) {
+      failed = true;
+      break;
+    }
+    tc::fence_after_sync();
+    if (warp < 3) {  // warp = row of g relative to the input row: tap row 2 - warp
+      const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16);
+#pragma unroll
+      for (int dx = 0; dx < 3; ++dx) {
+        float v[32];
+        tc::tmem_ld32(base + (dx == 2 ? 80 : 32 * dx), v);
+#pragma unroll
+        for (int c = 0; c < kC; ++c) acc[dx * kC + c] += v[c];
+      }
+      if (warp == 1) accb += tc::tmem_ld1(base + 64);
+    }
+    tc::fence_before_sync();
+    __syncthreads();  // TMEM and the staged rows are reused by the next tile
+  }
+  if (failed) {
+    // give the outstanding MMAs a second bounded chance to finish before freeing their TMEM
+    tc::mbar_wait(&bar, parity ^ 1u, kMmaPolls);
+    if (threadIdx.x == 0) atomicExch(err, 1);
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == 0) tc::tmem_dealloc<128>(tmem);
+  float* o = part + (size_t)blockIdx.x * kPartRow;
+  if (warp < 3) {
+#pragma unroll
+    for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+      for (int c = 0; c < kC; ++c) o[(lane * kC + c) * 9 + (2 - warp) * 3 + dx] = acc[dx * kC + c];
+    if (warp == 1) o[kW1 + lane] = accb;
   }
 }
-// dst[i] += sum over blocks (fixed order) of part[b][i], i < n
-__global__ void k_reduce_parts(const float* __restrict__ part, int nblocks, int n, float* __restrict__ dst) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += part[(size_t)b * kW1 + i];
+
+// Layers 0 and 3, FP32 on the CUDA cores: dW[c][tap] = sum_q h[q][c] f[q + s tap] with 32 BF16
+// channels h and one FP32 image f.  FIRST: h = g0, f = xin, s = +1, bias db[c] = sum_q h[q][c];
+// otherwise h = a2, f = gout, s = -1 (dW3[ci][tap] = sum_p gout[p] a2[p + tap][ci]) and
+// db = sum_q f[q].  A block takes tiles of 8 rows x 128 pixels, one row per warp; a lane owns a
+// channel pair (packed FP32 FMAs), the two half-warps walk the two halves of the row, and the nine
+// values of f slide along x, so a step costs one 4-byte load of h and three shared loads of f for
+// 18 sums.  Partial row layout: [0, 288) dW, then the bias.  The form this replaced read h once
+// per tap and pixel from 64 to 128 threads a block: 23.5 ms (first) and 36.9 ms (last) at 8 x 1024^2.
+constexpr int kEH = 8, kEW = 128;
+template <bool FIRST>
+__global__ void __launch_bounds__(256) k_wgrad_edge(const __nv_bfloat16* __restrict__ h, const float* __restrict__ f,
+                                                    int B, int H, int W, float* __restrict__ part) {
+  __shared__ float ft[kEH + 2][kEW + 2];
+  __shared__ float2 red[8][10][16];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, half = lane >> 4, cp = lane & 15;
+  float2 acc[9], accb = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int t = 0; t < 9; ++t) acc[t] = make_float2(0.f, 0.f);
+  const int tiles_x = (W + kEW - 1) / kEW, tiles_y = (H + kEH - 1) / kEH;
+  const int ntiles = B * tiles_x * tiles_y;
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int tx = tile % tiles_x, ty = (tile / tiles_x) % tiles_y, b = tile / (tiles_x * tiles_y);
+    const int y0 = ty * kEH, x0 = tx * kEW;
+    __syncthreads();
+    for (int q = threadIdx.x; q < (kEH + 2) * (kEW + 2); q += blockDim.x) {
+      const int gy = y0 - 1 + q / (kEW + 2), gx = x0 - 1 + q % (kEW + 2);
+      ft[q / (kEW + 2)][q % (kEW + 2)] =
+          (gy >= 0 && gy < H && gx >= 0 && gx < W) ? __ldg(f + ((size_t)b * H + gy) * W + gx) : 0.f;
+    }
+    __syncthreads();
+    const int y = y0 + warp;
+    if (y < H) {
+      const int xs = half * (kEW / 2);
+      const __nv_bfloat162* hp = reinterpret_cast<const __nv_bfloat162*>(h) + (((size_t)b * H + y) * W + x0 + xs) * (kC / 2) + cp;
+      const int n = min(kEW / 2, W - x0 - xs);  // this half's pixels (may be <= 0)
+      const float* fr = &ft[warp][xs];
+      // window win[i][j] = f at row y + i - 1, column x + j - 1
+      float win[3][3];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        win[i][0] = 0.f;
+        win[i][1] = fr[i * (kEW + 2)];
+        win[i][2] = fr[i * (kEW + 2) + 1];
+      }
+#pragma unroll 8
+      for (int k = 0; k < kEW / 2; ++k) {
+        __nv_bfloat162 hv = __floats2bfloat162_rn(0.f, 0.f);
+        if (k < n) hv = hp[(size_t)k * (kC / 2)];
+        const float2 v = __bfloat1622float2(hv);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          win[i][0] = win[i][1];
+          win[i][1] = win[i][2];
+          win[i][2] = fr[i * (kEW + 2) + k + 2];
+        }
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+          const float fv = FIRST ? win[t / 3][t % 3] : win[2 - t / 3][2 - t % 3];
+          acc[t] = __ffma2_rn(v, make_float2(fv, fv), acc[t]);
+        }
+        if constexpr (FIRST)
+          accb = __fadd2_rn(accb, v);
+        else if (k < n)
+          accb.x += win[1][1];  // every lane of the half holds the half's sum
+      }
+    }
+  }
+  // the two halves, then the eight warps in order
+#pragma unroll
+  for (int t = 0; t < 10; ++t) {
+    float2 v = t < 9 ? acc[t < 9 ? t : 0] : accb;
+    v.x += __shfl_down_sync(0xffffffffu, v.x, 16);
+    v.y += __shfl_down_sync(0xffffffffu, v.y, 16);
+    if (half == 0) red[warp][t][cp] = v;
+  }
+  __syncthreads();
+  float* o = part + (size_t)blockIdx.x * kPartRow;
+  for (int q = threadIdx.x; q < 160; q += blockDim.x) {
+    const int t = q / 16, c = q % 16;
+    float2 s = make_float2(0.f, 0.f);
+    for (int w = 0; w < 8; ++w) {
+      s.x += red[w][t][c].x;
+      s.y += red[w][t][c].y;
+    }
+    if (t < 9) {
+      o[(2 * c) * 9 + t] = s.x;
+      o[(2 * c + 1) * 9 + t] = s.y;
+    } else if (FIRST) {
+      o[288 + 2 * c] = s.x;
+      o[288 + 2 * c + 1] = s.y;
+    } else if (c == 0) {
+      o[288] = s.x;
+    }
+  }
+}
+// dst[i] += sum over blocks of part[b][i], i < n, in FP64: eight threads per element take every
+// eighth block, then their sums in order
+__global__ void __launch_bounds__(256) k_reduce_parts(const float* __restrict__ part, int nblocks, int n,
+                                                      float* __restrict__ dst) {
+  __shared__ double sh[8][32];
+  const int i = blockIdx.x * 32 + (threadIdx.x & 31), r = threadIdx.x >> 5;
+  double s = 0.0;
+  if (i < n)
+    for (int b = r; b < nblocks; b += 8) s += part[(size_t)b * kPartRow + i];
+  sh[r][threadIdx.x & 31] = s;
+  __syncthreads();
+  if (r == 0 && i < n) {
+#pragma unroll
+    for (int k = 1; k < 8; ++k) s += sh[k][threadIdx.x];
     dst[i] += (float)s;
   }
 }
@@ -601,7 +724,7 @@ static size_t cnn_bytes(int B, int H, int W, size_t* offs) {
   for (int i = 0; i < 5; ++i) offs[8 + i] = take(P * kC * 2);           // a0 a1 a2 g1 g2
   for (int i = 0; i < 3; ++i) offs[13 + i] = take(P * 4);               // xin out gout
   offs[16] = take((size_t)B * 4);                                        // sig
-  offs[17] = take((size_t)kWgradBlocks * kW1 * 4);                       // wpart
+  offs[17] = take((size_t)kWgradBlocks * kPartRow * 4);                  // wpart
   offs[18] = take(std::max<size_t>(4096, (size_t)B * kNormBlocks) * 8);  // dpart (loss / norm partials)
   offs[19] = take(256);                                                  // err
   return (off + 255) / 256 * 256;
@@ -644,7 +767,23 @@ static int net_forward(CnnNet& n, int B) {
   TMBIR_CHECK_LAUNCH();
   if (int e = conv32(n, n.a0, B, n.wg1, n.master + kOffB1, nullptr, n.a1, true)) return e;
   if (int e = conv32(n, n.a1, B, n.wg2, n.master + kOffB2, nullptr, n.a2, true)) return e;
-  k_conv_last<<<blocks, 256, 0, n.stream>>>(n.a2, B, n.H, n.W, n.master, n.out);
+  k_conv_last<false><<<blocks, 256, 0, n.stream>>>(n.a2, B, n.H, n.W, n.master, n.out);
+  TMBIR_CHECK_LAUNCH();
+  return TMBIR_OK;
+}
+
+// dW and db of a 32 -> 32 layer into n.grad at `off` (weights, then the bias)
+static int wgrad32(CnnNet& n, int B, const __nv_bfloat16* g, const __nv_bfloat16* in, int off) {
+  static bool attr = false;
+  if (!attr) {
+    TMBIR_CUDA(cudaFuncSetAttribute(k_wgrad32, cudaFuncAttributeMaxDynamicSharedMemorySize, kGradSmem));
+    attr = true;
+  }
+  const int tiles = B * ((n.H + kGRows - 1) / kGRows) * ((n.W + kTM - 1) / kTM);
+  const int blocks = std::min(tiles, kWgradBlocks);
+  k_wgrad32<<<blocks, 128, kGradSmem, n.stream>>>(g, in, B, n.H, n.W, n.wpart, n.err);
+  TMBIR_CHECK_LAUNCH();
+  k_reduce_parts<<<(kPartRow + 31) / 32, 256, 0, n.stream>>>(n.wpart, blocks, kPartRow, n.grad + off);
   TMBIR_CHECK_LAUNCH();
   return TMBIR_OK;
 }
@@ -653,42 +792,29 @@ static int net_forward(CnnNet& n, int B) {
 static int net_backward(CnnNet& n, int B, float* gin) {
   const size_t P = (size_t)B * n.H * n.W;
   const int blocks = (int)std::min<size_t>((P + 255) / 256, 152 * 16);
-  const int rb = (kW1 + 255) / 256;
+  const int etiles = B * ((n.H + kEH - 1) / kEH) * ((n.W + kEW - 1) / kEW);
+  const int eblocks = std::min(etiles, kWgradBlocks);
   // layer 3
-  k_wgrad_last<<<kWgradBlocks, 64, 0, n.stream>>>(n.gout, n.a2, B, n.H, n.W, n.wpart);
+  k_wgrad_edge<false><<<eblocks, 256, 0, n.stream>>>(n.a2, n.gout, B, n.H, n.W, n.wpart);
   TMBIR_CHECK_LAUNCH();
-  k_reduce_parts<<<2, 256, 0, n.stream>>>(n.wpart, kWgradBlocks, kW3 + kB3, n.grad + kOff3);
+  k_reduce_parts<<<(kW3 + kB3 + 31) / 32, 256, 0, n.stream>>>(n.wpart, eblocks, kW3 + kB3, n.grad + kOff3);
   TMBIR_CHECK_LAUNCH();
   k_last_dgrad<<<blocks, 256, 0, n.stream>>>(n.gout, n.a2, B, n.H, n.W, n.master, n.g2);
   TMBIR_CHECK_LAUNCH();
   // layer 2: weights from (g2, a1), then g1 = mask(a1) conv(g2, W2 flipped transposed)
-  k_wgrad32<<<kWgradBlocks, 256, 0, n.stream>>>(n.g2, n.a1, B, n.H, n.W, n.wpart);
-  TMBIR_CHECK_LAUNCH();
-  k_reduce_parts<<<rb, 256, 0, n.stream>>>(n.wpart, kWgradBlocks, kW1, n.grad + kOff2);
-  TMBIR_CHECK_LAUNCH();
-  k_bias_grad<<<kWgradBlocks, 32, 0, n.stream>>>(n.g2, P, n.wpart);
-  TMBIR_CHECK_LAUNCH();
-  k_reduce_parts<<<1, 32, 0, n.stream>>>(n.wpart, kWgradBlocks, kB1, n.grad + kOffB2);
-  TMBIR_CHECK_LAUNCH();
+  if (int e = wgrad32(n, B, n.g2, n.a1, kOff2)) return e;
   if (int e = conv32(n, n.g2, B, n.wt2, nullptr, n.a1, n.g1, false)) return e;
   // layer 1: weights from (g1, a0), then g0 = mask(a0) conv(g1, W1 flipped transposed) into g2's buffer
-  k_wgrad32<<<kWgradBlocks, 256, 0, n.stream>>>(n.g1, n.a0, B, n.H, n.W, n.wpart);
-  TMBIR_CHECK_LAUNCH();
-  k_reduce_parts<<<rb, 256, 0, n.stream>>>(n.wpart, kWgradBlocks, kW1, n.grad + kOff1);
-  TMBIR_CHECK_LAUNCH();
-  k_bias_grad<<<kWgradBlocks, 32, 0, n.stream>>>(n.g1, P, n.wpart);
-  TMBIR_CHECK_LAUNCH();
-  k_reduce_parts<<<1, 32, 0, n.stream>>>(n.wpart, kWgradBlocks, kB1, n.grad + kOffB1);
-  TMBIR_CHECK_LAUNCH();
+  if (int e = wgrad32(n, B, n.g1, n.a0, kOff1)) return e;
   __nv_bfloat16* g0 = n.g2;
   if (int e = conv32(n, n.g1, B, n.wt1, nullptr, n.a0, g0, false)) return e;
   // layer 0
-  k_wgrad_first<<<kWgradBlocks, 128, 0, n.stream>>>(g0, n.xin, B, n.H, n.W, n.wpart);
+  k_wgrad_edge<true><<<eblocks, 256, 0, n.stream>>>(g0, n.xin, B, n.H, n.W, n.wpart);
   TMBIR_CHECK_LAUNCH();
-  k_reduce_parts<<<2, 256, 0, n.stream>>>(n.wpart, kWgradBlocks, kW0 + kB0, n.grad + kOff0);
+  k_reduce_parts<<<(kW0 + kB0 + 31) / 32, 256, 0, n.stream>>>(n.wpart, eblocks, kW0 + kB0, n.grad + kOff0);
   TMBIR_CHECK_LAUNCH();
   if (gin) {
-    k_first_dgrad<<<blocks, 256, 0, n.stream>>>(g0, B, n.H, n.W, n.master, gin);
+    k_conv_last<true><<<blocks, 256, 0, n.stream>>>(g0, B, n.H, n.W, n.master, gin);
     TMBIR_CHECK_LAUNCH();
   }
   return TMBIR_OK;

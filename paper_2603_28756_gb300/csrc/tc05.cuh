@@ -82,6 +82,13 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32() {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// The same with both operands MN-major (the transpose bits 15 and 16): element (row r, k) of an
+// operand sits at start + (r % 8) * 2 + (r / 8) * sbo + (k % 8) * 16 + (k / 8) * lbo bytes.
+template <int M, int N>
+__host__ __device__ constexpr uint32_t idesc_bf16_f32_mn() {
+  return idesc_bf16_f32<M, N>() | (1u << 15) | (1u << 16);
+}
+
 // D (TMEM) (+)= A * B^T; accumulate = 0 overwrites D.  Issued by a single thread.
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                          uint32_t accumulate) {
@@ -114,6 +121,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// one 32-bit column
+__device__ __forceinline__ float tmem_ld1(uint32_t taddr) {
+  uint32_t r;
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr) : "memory");
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  return __uint_as_float(r);
 }
 
 // ---------------------------------------------------------------- asynchronous 16-byte copies
