@@ -1,0 +1,84 @@
+"""Kernels and dispatch rules at the sizes where they change route, against the FP64 oracle or against
+the same work done another way.  Tolerances are those of the operators' own parity tests: 1e-5
+relative L2 for FP32 operators, bitwise where only the order of launches differs."""
+import math
+
+import numpy as np
+import pytest
+
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+import paper_2603_28756_gb300 as tm  # noqa: E402
+
+PRIOR = dict(p=1.2, q=2.0, c=0.01, sigma=0.1, lam=1.0)
+
+
+def rel(a, b):
+    return float(np.linalg.norm(np.asarray(a, np.float64) - b) / np.linalg.norm(b))
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a, dtype=np.float32).ravel()).cuda()
+
+
+def host(t, shape):
+    torch.cuda.synchronize()
+    return t.double().cpu().numpy().reshape(shape)
+
+
+# odd sides (scalar accesses), sides that end a thread's column pair, a block's 256 columns and a walk
+# of 8 or 32 rows, and enough slices for the long walks
+@pytest.mark.parametrize("S,Nc", [(1, 1), (2, 5), (1, 33), (1, 257), (2, 258), (305, 64), (330, 63)])
+def test_upsample_routes(orc, S, Nc):
+    c = np.random.default_rng(S + Nc).standard_normal((S, Nc, Nc)).astype(np.float32)
+    ctx = tm.Context([tm.Group(N=64, angles=[0.0], n_slices=1)])
+    f = host(ctx.upsample_lanczos3(dev(c), S, Nc), (S, 2 * Nc, 2 * Nc))
+    ref = orc.lanczos_up(c.astype(np.float64))
+    assert np.array_equal(f[:, ::2, ::2], c.astype(np.float64))
+    assert np.max(np.abs(f - ref)) < 1e-5 * np.max(np.abs(ref))
+
+
+# rows of the spreading matrix at the grid's centre: about 5 (FP32 paths) and 11 (R*g) entries per
+# angle, so 40 angles end in the rows a warp ranks, 200 in those a block sorts in shared memory and
+# 1000 in those it sorts in place
+@pytest.mark.parametrize("na", [1, 40, 200, 1000])
+def test_spreading_matrix_rows(orc, na):
+    N = 64
+    p = synth.volume(S=1, N=N, n_angles=na, n_ellipsoids=4, seed=na)
+    outs = []
+    for _ in range(2):  # the fill order differs from run to run, the sorted rows must not
+        ctx = tm.Context([tm.Group(N=N, angles=list(p.theta), n_slices=1)])
+        outs.append((ctx.adjoint(dev(p.sino)), ctx.build_operator(dev(p.sino))))
+    ref = orc.adjoint(p.sino.astype(np.float64), N, p.theta)
+    assert rel(host(outs[0][0], ref.shape), ref) < 1e-5
+    assert rel(host(outs[0][1], ref.shape), ref) < 1e-6
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+
+
+def test_many_groups_reduce_like_one(orc):
+    # more groups than the finalize kernel reduces between two barriers
+    specs = [(64, 1 + k % 3, 9 + k) for k in range(18)]
+    groups, sinos = [], []
+    for k, (N, S, na) in enumerate(specs):
+        p = synth.volume(S=S, N=N, n_angles=na, n_ellipsoids=3, seed=70 + k)
+        groups.append(tm.Group(N=N, angles=list(p.theta), n_slices=S))
+        sinos.append(p.sino.ravel())
+    big = tm.Context(groups)
+    atg = big.build_operator(dev(np.concatenate(sinos)))
+    x = torch.zeros_like(atg)
+    big.reconstruct(x, atg, tm.Params(**PRIOR, max_iter=6))
+    off = 0
+    for k, (N, S, na) in enumerate(specs):
+        n = S * N * N
+        ctx = tm.Context([groups[k]])
+        x1 = torch.zeros(n, dtype=torch.float32, device="cuda")
+        ctx.reconstruct(x1, ctx.build_operator(dev(sinos[k])), tm.Params(**PRIOR, max_iter=6))
+        torch.cuda.synchronize()
+        assert torch.equal(x[off:off + n], x1), k
+        off += n
