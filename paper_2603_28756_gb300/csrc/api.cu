@@ -825,12 +825,15 @@ int tmbir_get_log(tmbir_ctx* ctx, double* h_log, int max_entries, int* n_out) {
   return TMBIR_OK;
 }
 
-// one pass-1/2/3 sequence per group with explicit arguments, then the partial sums to the host
+// one pass-1/2/3 sequence per group with explicit arguments, then the partial sums to the host (in
+// Apply mode, whose result pass 3a writes, pass 3b only forms partial sums and is left out when
+// nobody asks for them)
 static int run_explicit(Ctx& c, const StepArgs& a, Pass3Mode m, const PriorC& pc, double* h_parts) {
   int off = 0;
   for (size_t i = 0; i < c.gdev.size(); ++i) {
     const GroupDev& g = c.gdev[i];
     if (int e = launch_convolution(g, a, m, pc, c.stream)) return e;
+    if (m == Pass3Mode::Apply && !h_parts) continue;
     if (int e = launch_pass3(g, a, m, pc, c.partials, off, c.stream, false, 2)) return e;
     off += blocks_pass3(g);
   }

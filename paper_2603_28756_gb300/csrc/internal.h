@@ -279,16 +279,29 @@ GroupDev chunk_view(const GroupDev& g, int c0, int n);
 int launch_convolution(const GroupDev& g, const StepArgs& a, Pass3Mode mode, const PriorC& pc, cudaStream_t s,
                        bool bf16 = false);
 int conv_launches(const GroupDev& g);
-// Pass-3b blocks per slice chunk: bands of 4 rows times column blocks of up to 512 columns
-// (eight warps of 64 columns).
-constexpr int pass3_row_blocks(int N) { return (N / 4) * (N / (64 * (N / 64 < 8 ? N / 64 : 8))); }
-// Slices each pass-3 block marches through: enough blocks for about four waves of two
-// blocks per SM on 152 SMs, longer marches when the volume has slices to spare.
+// Pass-3b blocks: two bands of pass3_band(N) rows times column blocks of pass3_warps(N) warps of 32
+// columns.  Four-warp blocks, four per SM, finish and restart at a finer grain than eight-warp ones
+// (1.36 against 1.47 ms at 32 x 2048^2).  Bands of eight rows evaluate 14.1 pairs per voxel, bands of
+// four 15.3 (1.29 against 1.41 ms), but twice the rows per lane is twice the latency of a small
+// image's only wave of blocks, so the sides up to 256 keep four.
+constexpr int pass3_warps(int N) { return N / 32 < 4 ? N / 32 : 4; }
+constexpr int pass3_band(int N) { return N >= 512 ? 8 : 4; }
+constexpr int pass3_row_blocks(int N) { return (N / (2 * pass3_band(N))) * (N / (32 * pass3_warps(N))); }
+// Slices each pass-3 block marches through: the march with the least work per SM slot, counting
+// whole waves of four blocks per SM on 152 SMs and, per march, the pairs into its first slice,
+// which are evaluated once more (about 0.7 of a slice).
 inline int pass3_slices_per_block(int S, int row_blocks) {
-  int chunks = (1216 + row_blocks / 2) / row_blocks;
-  if (chunks < 1) chunks = 1;
-  if (chunks > S) chunks = S;
-  return (S + chunks - 1) / chunks;
+  int best = S;
+  double best_cost = 1e300;
+  for (int c = 1; c <= S && c <= 256; ++c) {
+    const int zc = (S + c - 1) / c, chunks = (S + zc - 1) / zc;
+    const double cost = (double)(((long long)chunks * row_blocks + 607) / 608) * (zc + 0.7);
+    if (cost < best_cost * 0.999) {
+      best_cost = cost;
+      best = zc;
+    }
+  }
+  return best;
 }
 // slices whose gradient pass 3b computes
 inline int pass3_slices(const GroupDev& g) { return g.zn > 0 ? g.zn : g.S; }

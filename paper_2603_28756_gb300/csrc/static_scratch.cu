@@ -80,15 +80,23 @@ extern "C" int tmbir_normal_apply_static(tmbir_ctx* ctx, const float* d_x, float
   Ctx& c = ctx->c;
   if (!d_x || !d_z || ((uintptr_t)d_x & 15u) || ((uintptr_t)d_z & 15u) || d_x == d_z)
     return set_error(TMBIR_ERR_ARG, "normal_apply_static: bad buffers");
-  // the groups one after another, each in spectrum chunks that fit the static array
-  int blocks = 0;
+  // the groups one after another, each in spectrum chunks that fit the static array.  The block
+  // budget counts bands of 4 rows x 512 columns and marches of about four waves per 1216 blocks; the
+  // launches below march through whole groups and never write more rows than that.
+  auto budget = [](const GroupDev& g) {
+    const int nb = (g.N / 4) * (g.N / (64 * std::min(g.N / 64, 8)));
+    const int chunks = std::max(1, std::min(g.S, (1216 + nb / 2) / nb));
+    const int zc = g.zc > 0 ? std::min(g.zc, g.S) : (g.S + chunks - 1) / chunks;
+    return nb * ((g.S + zc - 1) / zc);
+  };
+  long long blocks = 0;
   for (const GroupDev& g : c.gdev) {
     const size_t per = (size_t)(g.N + 1) * g.N;
     if (per > kStaticSpecElems)
       return set_error(TMBIR_ERR_SHAPE, "normal_apply_static: one slice needs " + std::to_string(per) +
                                             " complex scratch values, the static array holds " +
                                             std::to_string(kStaticSpecElems));
-    blocks += blocks_pass3(g);
+    blocks += budget(g);
   }
   if ((size_t)blocks * kParts > kStaticPartElems)
     return set_error(TMBIR_ERR_SHAPE, "normal_apply_static: too many reducing blocks for the static array");
@@ -105,6 +113,7 @@ extern "C" int tmbir_normal_apply_static(tmbir_ctx* ctx, const float* d_x, float
   for (const GroupDev& g0 : c.gdev) {
     GroupDev g = g0;
     g.spec = spec;
+    g.zc = g.S;
     g.sc = std::min(spec_chunk(g0), (int)(kStaticSpecElems / ((size_t)(g.N + 1) * g.N)));
     if (int e = launch_convolution(g, a, Pass3Mode::Apply, pc, c.stream)) return e;
     if (int e = launch_pass3(g, a, Pass3Mode::Apply, pc, parts, boff, c.stream, false, 2)) return e;

@@ -138,51 +138,6 @@ __device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) { return _
 __device__ __forceinline__ float2 f2mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 f2add(float2 a, float2 b) { return __fadd2_rn(a, b); }
 
-// Constants of the qGGMRF potential in the form the packed neighbour term uses.
-struct PriorK {
-  float2 half_qp;  // (q - p) / 2
-  float2 qp_l2;    // (q - p) log2(1 / (c sigma))
-  float2 p, qmp;   // p, q - p
-  float2 half_q2;  // (q - 2) / 2
-  float2 q2_l2;    // (q - 2) log2(1 / sigma)
-};
-__device__ __forceinline__ PriorK prior_k(const PriorC& c) {
-  PriorK k;
-  k.half_qp = f2(0.5f * c.qp);
-  k.qp_l2 = f2(c.qp_l2_inv_csig);
-  k.p = f2(c.p);
-  k.qmp = f2(c.qp);
-  k.half_q2 = f2(0.5f * (c.q - 2.0f));
-  k.q2_l2 = f2((c.q - 2.0f) * c.l2_inv_sig);
-  return k;
-}
-
-// One neighbour term of the qGGMRF potential for two voxels at once (the two lanes):
-//   rho(d)  = |d/sigma|^q / (1 + u),  u = |d/(c sigma)|^(q-p),  r = 1 / (1 + u)
-//   rho'(d) = d/sigma^2 |d/sigma|^(q-2) (q + p u) / (1 + u)^2
-//           = d/sigma^2 |d/sigma|^(q-2) r (p + (q - p) r)
-// g += sigma^2 rho'(d) and, when phi, ph += sigma^2 rho(d) (the caller folds 1/sigma^2 into
-// the neighbour weight).  u comes from log2(d^2 + 1e-30), which stays finite at d = 0 (there
-// r = 1 and both terms vanish).  Three special-function operations per lane (log2, exp2,
-// reciprocal), four for q != 2.
-template <bool Q2>
-__device__ __forceinline__ void nbr2(float2 y, float2 nb, const PriorK& k, float2& g, float2& ph, bool phi) {
-  const float2 d = f2fma(nb, f2(-1.f), y);
-  const float2 sq = f2fma(d, d, f2(1e-30f));
-  const float2 la = make_float2(lg2a(sq.x), lg2a(sq.y));
-  const float2 s = f2fma(k.half_qp, la, k.qp_l2);
-  const float2 e = f2add(make_float2(ex2a(s.x), ex2a(s.y)), f2(1.f));
-  const float2 r = make_float2(rcpa(e.x), rcpa(e.y));
-  const float2 t = f2fma(k.qmp, r, k.p);
-  float2 dr = f2mul(d, r);
-  if constexpr (!Q2) {
-    const float2 s2 = f2fma(k.half_q2, la, k.q2_l2);
-    dr = f2mul(dr, make_float2(ex2a(s2.x), ex2a(s2.y)));
-  }
-  g = f2fma(dr, t, g);
-  if (phi) ph = f2fma(d, dr, ph);
-}
-
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -824,151 +779,196 @@ __global__ void __launch_bounds__(64 * RB, 8 / RB) k_pass3a_q(const __grid_const
 // pair is evaluated once, from its lexicographically smaller end (13 forward offsets), and
 // the value is handed to the other end instead of being recomputed there.
 //
-// A block owns R = 4 rows (a band) by BC columns of one group and marches through a chunk of
-// its slices.  Warp w owns 64 columns; lane l owns the voxel pair a = 2l, b = 2l + 1 of every
-// row of the band as the two lanes of packed FP32 pairs, so the pair (a, b) stays in the
-// thread, the pairs with columns a - 1 and b + 1 go to the neighbouring lanes by shuffle, and
-// the pairs that cross a warp's outer columns are evaluated once more by the receiving warp
-// (nine per row, spread over the lanes before the row walk).  Rows are walked top to bottom
-// with the halo rows -1 and R as sources of pairs into the band; slice z is the source of
-// the pairs into slice z + 1, whose contributions wait in shared memory (one entry per
-// thread) for the next step.  A chunk starting at z0 > 0 first evaluates the pairs between
-// slices z0 - 1 and z0 (the only pairs evaluated twice, once per chunk).  Shared memory holds
-// y for slices z and z + 1 (rows -1 .. R, columns c0 - 4 .. c0 + BC + 3), each beside a copy
-// shifted by one column so that the neighbour pairs (a - 1, a) and (b, b + 1) are aligned 8-byte
-// loads like (a, b); x and x_prev of slice z + 2, arriving by asynchronous copies while slice
-// z is worked on; the carried contributions; and K (*) y, R*g and x_k at each thread's voxels,
-// copied asynchronously one slice ahead.  Neighbours outside the volume read the voxel itself
-// (d = 0 adds nothing).
+// A block owns two bands of R rows by BC columns of one group, one below the other, and marches
+// through a chunk of its slices.  A lane owns one column; the two lanes of its packed FP32 pairs
+// are the rows r0 + t and r0 + R + t, so every neighbour offset is the same for both halves: the
+// ring in shared memory interleaves the two bands (float2 per column) and a neighbour pair is one
+// aligned 8-byte load at any column offset, without shifted copies and without exchanges between
+// the halves.  (With two neighbouring columns in a pair, as this kernel was first built, the
+// offsets dx = +-1 need a copy shifted by one column and scalar hand-overs between the halves.)
+//
+// Rows are walked by the target row u: the pairs that end in row u of slice zs (from rows u - 1 and
+// u) and in row u of slice zs + 1 (from rows u - 1, u, u + 1).  A target row's contributions are
+// then complete after one step, its loads are used at once, and what stays in registers between
+// steps is three centre values and two gradient rows: 6 shared loads per voxel pair and row
+// instead of 14.  The walk is a loop, not unrolled: the unrolled bodies of the four boundary
+// variants are 130 KB of instructions and measured slower (1.50 against 1.29 ms at 32 x 2048^2).
+// The shares of the pairs with dx = +-1 go to the neighbouring lanes by shuffle once per row.
+// Across a warp's outer columns the pairs within a slice are evaluated once more by the receiving
+// warp (three per row, one evaluation for all rows), and those into slice zs + 1 are handed over
+// through shared memory.  The halo rows -1 and R are sources or targets only.  Slice zs is the
+// source of the pairs into slice zs + 1, whose contributions wait in shared memory (one entry per
+// thread and row) for the next step.  A chunk starting at z0 > 0 first evaluates the pairs between
+// slices z0 - 1 and z0 (evaluated twice, once per chunk).  x and x_prev of slice z + 2 arrive by
+// asynchronous copies while slice z is worked on; K (*) y, R*g and x_k of a row are loaded into
+// registers one row ahead of their use.  A neighbour outside the volume is masked to d = 0.
+//
+// What bounds it: the special-function unit, then FP32 issue.  Per packed pair the unit spends 16
+// cycles of an SM quarter on two log2, 8 on two exp2 and 8 on one reciprocal (measured rates: 16
+// log2, 32 exp2 and 16 reciprocals per clock and SM), the FMA pipe about 25.  The two halves share
+// one reciprocal (r_x = e_y / (e_x e_y)); with one each the kernel ran at the unit's rate (40 cycles a
+// pair).  Measured at 32 x 2048^2: 1.64 ms with neighbouring columns in a pair, 1.36 with the two
+// bands, 1.29 with the shared reciprocal and eight-row bands; at 64 x 1024^2 0.87, 0.77 and 0.69 ms.
 template <int N>
 struct GeoP {
-  static_assert(N % 64 == 0, "a warp owns 64 columns");
-  static constexpr int R = 4;                             // rows of a band
-  static constexpr int WPB = N / 64 < 8 ? N / 64 : 8;     // warps per block
+  static_assert(N % 64 == 0, "a warp owns 32 columns, a block at least two warps");
+  static constexpr int R = pass3_band(N);                 // rows of a band
+  static constexpr int ROWS = 2 * R;                      // rows of a block
+  static constexpr int WPB = pass3_warps(N);              // warps per block
   static constexpr int THREADS = 32 * WPB;
-  static constexpr int BC = 64 * WPB;                     // columns of a block
-  static constexpr int CB = N / BC;                       // column blocks per band
-  static constexpr int NB = N / R;                        // bands per slice
-  static constexpr int LDR = BC + 8;                      // ring row stride (floats)
-  static constexpr int RING = (R + 2) * LDR;              // y of one slice (the shifted copy follows)
-  static constexpr int NEDGE = 9 * R;                     // cross-warp pairs per warp and step
-  static constexpr int FIN = 3 * R * THREADS;            // K (*) y, R*g, x_k of the band (float2)
-  // ring (2 slices of y and shifted y) | staging (x, x_prev of one slice) | carry | cross-warp
-  // pair values | the next slice's K (*) y, R*g and x_k at each thread's voxels
-  static constexpr size_t SM = (size_t)(6 * RING + R * BC + WPB * NEDGE) * sizeof(float) + (size_t)FIN * 8;
-  static_assert(N % BC == 0, "column blocks");
+  static constexpr int BC = 32 * WPB;                     // columns of a block
+  static constexpr int CB = N / BC;                       // column blocks per band pair
+  static constexpr int NB = N / ROWS;                     // band pairs per slice
+  static constexpr int LDR = BC + 8;                      // row stride of ring and staging: columns c0 - 4 .. c0 + BC + 3
+  static constexpr int RING = (R + 2) * LDR;              // float2 entries of one slice
+  static constexpr int STG = (ROWS + 2) * LDR;            // floats of one staged array
+  static constexpr int EDGE = 4 * R;                      // a warp's outer sums: left, right, outside the block, zeros
+  static constexpr int XCH = 2 * (WPB + 2) * R;           // shares handed from warp to warp (one parity)
+  // ring (2 slices) | carry | warps' outer sums | warp-to-warp shares (2 parities) | staged x, x_prev
+  static constexpr size_t SM = (size_t)(2 * RING + R * THREADS + WPB * EDGE + 2 * XCH) * 8 + (size_t)2 * STG * 4;
+  static_assert(3 * R <= 32 && WPB >= 2, "outer pairs of a warp in one evaluation per target slice");
+  static_assert(N % BC == 0 && N % ROWS == 0, "blocks");
 };
 
-// y = x + beta (x - x_prev) of one slice, rows r0 - 1 .. r0 + R, columns c0 - 4 .. c0 + BC + 3,
-// into a ring slot (zero outside the image)
+// y = x + beta (x - x_prev) of one slice into a ring slot: ring row i, column q of the float4
+// grid, holds rows r0 - 1 + i (first halves) and r0 - 1 + i + R (second halves) at columns
+// c0 - 4 + 4 q .. + 3.  ld(row index 0 .. 2R + 1, q, which) gives the float4 of x (0) or x_prev (1).
+// A thread keeps its column and takes every fourth row; the two halo columns of all rows go to the
+// first threads.
+template <int N, class Ld>
+__device__ __forceinline__ void fill_ring(float2* slot, float beta, Ld&& ld) {
+  using GP = GeoP<N>;
+  constexpr int QB = GP::BC / 4;
+  const float2 b2 = f2(beta);
+  auto yv = [&](float2 x, float2 p) { return f2fma(b2, make_float2(x.x - p.x, x.y - p.y), x); };
+  auto put = [&](int i, int q) {
+    const float4 xa = ld(i, q, 0), pa = ld(i, q, 1), xb = ld(i + GP::R, q, 0), pb = ld(i + GP::R, q, 1);
+    const float2 y0 = yv(make_float2(xa.x, xb.x), make_float2(pa.x, pb.x));
+    const float2 y1 = yv(make_float2(xa.y, xb.y), make_float2(pa.y, pb.y));
+    const float2 y2 = yv(make_float2(xa.z, xb.z), make_float2(pa.z, pb.z));
+    const float2 y3 = yv(make_float2(xa.w, xb.w), make_float2(pa.w, pb.w));
+    float4* d = reinterpret_cast<float4*>(slot + i * GP::LDR + 4 * q);
+    d[0] = make_float4(y0.x, y0.y, y1.x, y1.y);
+    d[1] = make_float4(y2.x, y2.y, y3.x, y3.y);
+  };
+  const int q = threadIdx.x % QB + 1, i0 = threadIdx.x / QB;
+#pragma unroll
+  for (int h = 0; h < (GP::R + 2 + 3) / 4; ++h)
+    if (i0 + 4 * h < GP::R + 2) put(i0 + 4 * h, q);
+  // (from the other end of the block, whose threads have fewer rows)
+  const int e = GP::THREADS - 1 - threadIdx.x;
+  if (e < 2 * (GP::R + 2)) put(e >> 1, (e & 1) * (QB + 1));
+}
+// from global memory (zero outside the image)
 template <int N>
-__device__ __forceinline__ void load_ring_p(float* slot, const float* x, const float* xp, float beta,
+__device__ __forceinline__ void load_ring_p(float2* slot, const float* x, const float* xp, float beta,
                                             size_t off_slice, int r0, int c0) {
+  fill_ring<N>(slot, beta, [&](int i, int q, int which) {
+    const int rr = r0 - 1 + i, cc = c0 - 4 + 4 * q;
+    if (rr < 0 || rr >= N || cc < 0 || cc >= N) return make_float4(0.f, 0.f, 0.f, 0.f);
+    return __ldg(reinterpret_cast<const float4*>((which ? xp : x) + off_slice + (size_t)rr * N + cc));
+  });
+}
+// x and x_prev of one slice (rows r0 - 1 .. r0 + 2R, the ring's columns) into the staging area by
+// asynchronous 16-byte copies, zero-filled outside the image.  A thread copies one array and one
+// column, every second row, from one pointer at fixed offsets; the halo columns go to the first
+// threads.
+template <int N>
+struct Stager {
   using GP = GeoP<N>;
-  constexpr int Q = GP::LDR / 4;
-  for (int e = threadIdx.x; e < (GP::R + 2) * Q; e += GP::THREADS) {
-    const int q = e % Q, rowi = e / Q;
-    const int rr = r0 - 1 + rowi, cc = c0 - 4 + 4 * q;
-    float4 yv = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (rr >= 0 && rr < N && cc >= 0 && cc < N) {
-      const size_t off = off_slice + (size_t)rr * N + cc;
-      const float4 xv = __ldg(reinterpret_cast<const float4*>(x + off));
-      const float4 pv = __ldg(reinterpret_cast<const float4*>(xp + off));
-      yv = make_float4(fmaf(beta, xv.x - pv.x, xv.x), fmaf(beta, xv.y - pv.y, xv.y), fmaf(beta, xv.z - pv.z, xv.z),
-                       fmaf(beta, xv.w - pv.w, xv.w));
+  static constexpr int QB = GP::BC / 4, ITEMS = (GP::ROWS + 2) / 2;
+  static_assert(4 * (GP::ROWS + 2) <= GP::THREADS, "halo items");
+  const float* src;    // first item in slice 0
+  const float* hsrc;   // halo item in slice 0
+  float *dst, *hdst;
+  bool first, last, halo, hok;
+  __device__ __forceinline__ Stager(float* stg, const float* x, const float* xp, int r0, int c0) {
+    const int q = threadIdx.x % QB, arr = (threadIdx.x / QB) & 1, row = threadIdx.x / (2 * QB);
+    src = (arr ? xp : x) + (ptrdiff_t)(r0 - 1 + row) * N + c0 + 4 * q;
+    dst = stg + arr * GP::STG + row * GP::LDR + 4 * (q + 1);
+    first = row > 0 || r0 > 0;
+    last = row == 0 || r0 + GP::ROWS < N;
+    const int hr = threadIdx.x >> 2, ha = (threadIdx.x >> 1) & 1, side = threadIdx.x & 1;
+    halo = threadIdx.x < 4 * (GP::ROWS + 2);
+    hok = r0 - 1 + hr >= 0 && r0 - 1 + hr < N && (side ? c0 + GP::BC < N : c0 > 0);
+    hsrc = (ha ? xp : x) + (ptrdiff_t)(r0 - 1 + hr) * N + (side ? c0 + GP::BC : c0 - 4);
+    hdst = stg + ha * GP::STG + hr * GP::LDR + side * (GP::BC + 4);
+  }
+  __device__ __forceinline__ void issue(size_t off_slice) const {
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+      const bool ok = i == 0 ? first : (i == ITEMS - 1 ? last : true);
+      tc05::cp_async16(dst + 2 * i * GP::LDR, ok ? src + off_slice + 2 * i * N : src + off_slice + 2 * N, ok);
     }
-    reinterpret_cast<float4*>(slot + rowi * GP::LDR)[q] = yv;
+    if (halo) tc05::cp_async16(hdst, hok ? hsrc + off_slice : src + off_slice + 2 * N, hok);
   }
+};
+template <int N>
+__device__ __forceinline__ void stage_to_ring(float2* slot, const float* stg, float beta) {
+  using GP = GeoP<N>;
+  fill_ring<N>(slot, beta, [&](int i, int q, int which) {
+    return reinterpret_cast<const float4*>(stg + which * GP::STG + i * GP::LDR)[q];
+  });
 }
 
-// x and x_prev of one slice (the ring's rows and columns) into the staging area by
-// asynchronous 16-byte copies, zero-filled outside the image
-template <int N>
-__device__ __forceinline__ void stage_issue(float* stg, const float* x, const float* xp, size_t off_slice, int r0,
-                                            int c0) {
-  using GP = GeoP<N>;
-  constexpr int Q = GP::LDR / 4;
-  for (int e = threadIdx.x; e < (GP::R + 2) * Q; e += GP::THREADS) {
-    const int q = e % Q, rowi = e / Q;
-    const int rr = r0 - 1 + rowi, cc = c0 - 4 + 4 * q;
-    const bool ok = rr >= 0 && rr < N && cc >= 0 && cc < N;
-    const size_t off = ok ? off_slice + (size_t)rr * N + cc : off_slice;
-    tc05::cp_async16(stg + 4 * e, x + off, ok);
-    tc05::cp_async16(stg + GP::RING + 4 * e, xp + off, ok);
-  }
+// Keeps a loop constant in its registers: the compiler otherwise rebuilds the two halves of every
+// packed constant with moves at each use (six of the 22 instructions of a pair).
+__device__ __forceinline__ float2 pin(float2 v) {
+  asm volatile("" : "+f"(v.x), "+f"(v.y));
+  return v;
 }
-// y = x + beta (x - x_prev) from the staging area into a ring slot, and the copy shifted by
-// one column (shifted[i] = y[i + 1]) after it
-template <int N>
-__device__ __forceinline__ void stage_to_ring(float* slot, const float* stg, float beta) {
-  using GP = GeoP<N>;
-  for (int e = threadIdx.x; e < GP::RING / 4; e += GP::THREADS) {
-    const float4 xv = reinterpret_cast<const float4*>(stg)[e];
-    const float4 pv = reinterpret_cast<const float4*>(stg + GP::RING)[e];
-    const float4 y =
-        make_float4(fmaf(beta, xv.x - pv.x, xv.x), fmaf(beta, xv.y - pv.y, xv.y), fmaf(beta, xv.z - pv.z, xv.z),
-                    fmaf(beta, xv.w - pv.w, xv.w));
-    float nx = 0.f;
-    if (4 * e + 4 < GP::RING) {
-      const float x4 = stg[4 * e + 4], p4 = stg[GP::RING + 4 * e + 4];
-      nx = fmaf(beta, x4 - p4, x4);
-    }
-    reinterpret_cast<float4*>(slot)[e] = y;
-    reinterpret_cast<float4*>(slot + GP::RING)[e] = make_float4(y.y, y.z, y.w, nx);
+// Constants of the packed pair term.
+struct PairK {
+  float2 half_qp, qp_l2, p, qmp, one;
+  float2 half_q2, q2_l2;  // q != 2 only
+};
+template <bool Q2>
+__device__ __forceinline__ PairK pair_k(const PriorC& c) {
+  PairK k;
+  // q = p: any positive exponent this small gives 1 for every difference but 0, whose term vanishes
+  k.half_qp = pin(f2(fmaxf(0.5f * c.qp, 1.5e-38f)));
+  k.qp_l2 = pin(f2(c.qp_l2_inv_csig));
+  k.p = pin(f2(c.p));
+  k.qmp = pin(f2(c.qp));
+  k.one = pin(f2(1.f));
+  if constexpr (!Q2) {
+    k.half_q2 = f2(0.5f * (c.q - 2.0f));
+    k.q2_l2 = f2((c.q - 2.0f) * c.l2_inv_sig);
   }
+  return k;
 }
-// the shifted copy of a ring slot whose y part is in place
-template <int N>
-__device__ __forceinline__ void ring_shift(float* slot) {
-  using GP = GeoP<N>;
-  for (int e = threadIdx.x; e < GP::RING / 4; e += GP::THREADS) {
-    const float4 v = reinterpret_cast<const float4*>(slot)[e];
-    const float nx = 4 * e + 4 < GP::RING ? slot[4 * e + 4] : 0.f;
-    reinterpret_cast<float4*>(slot + GP::RING)[e] = make_float4(v.y, v.z, v.w, nx);
-  }
-}
-
-// The lane's neighbour pair at column offset DX in a ring row (y part; the shifted copy sits
-// RING floats further): DX = -1: (y[a - 1], y[a]), 0: (y[a], y[b]), +1: (y[b], y[b + 1]).
-// A neighbour outside the image reads the voxel itself: with ROWE for a missing row (row_ok
-// false), with COLE for a missing column a - 1 or b + 1.
-template <int N, int DX, bool ROWE, bool COLE>
-__device__ __forceinline__ float2 nb_pair(const float* row, int ia, float2 y, bool row_ok, bool okL, bool okR) {
-  constexpr int RING = GeoP<N>::RING;
-  float2 n;
-  if constexpr (DX < 0)
-    n = *reinterpret_cast<const float2*>(row + RING + ia - 2);
-  else if constexpr (DX == 0)
-    n = *reinterpret_cast<const float2*>(row + ia);
-  else
-    n = *reinterpret_cast<const float2*>(row + RING + ia);
-  if constexpr (COLE) {
-    if constexpr (DX < 0) n.x = okL ? n.x : y.x;
-    if constexpr (DX > 0) n.y = okR ? n.y : y.y;
-  }
-  if constexpr (ROWE) n = row_ok ? n : y;
-  return n;
-}
-
-// Weighted pair value f = w sigma^2 rho'(y - nb) / sigma^2 of two pairs at once (the weight
-// arrives as wq = w (q - p) / sigma^2, wp = w p / sigma^2), with the identity of nbr2:
-// sigma^2 rho'(d) = d |d/sigma|^(q-2) r (p + (q - p) r), r = 1 / (1 + |d/(c sigma)|^(q-p)).
-// With PH, ph += sigma^2 rho(d) = d^2 |d/sigma|^(q-2) r (unweighted).
-template <bool Q2, bool PH>
-__device__ __forceinline__ float2 pairv(float2 y, float2 nb, const PriorK& k, float2 wq, float2 wp, float2& ph) {
-  const float2 d = f2fma(nb, f2(-1.f), y);
-  const float2 sq = f2fma(d, d, f2(1e-30f));
+// Unweighted pair value v = sigma^2 rho'(nb - y) of two pairs at once from n = -y, with the identity
+//   sigma^2 rho'(d) = d |d/sigma|^(q-2) r (p + (q - p) r), r = 1 / (1 + |d/(c sigma)|^(q-p)).
+// With PH, ph += sigma^2 rho(d) = d^2 |d/sigma|^(q-2) r (unweighted).  MX, MY: the first / second
+// half counts only when okx / oky.  For q = 2 the exponent is at most 1 and s is limited to 63 (a
+// difference of 10^19 times c sigma), so that the product of the two e stays finite; log2 0 = -inf
+// gives r = 1 there, and d = 0 ends both terms.  For q != 2 the logarithm is kept finite, since the
+// second exponential would meet it with a negative factor.
+template <bool Q2, bool PH, bool MX, bool MY>
+__device__ __forceinline__ float2 pairv(float2 n, float2 nb, const PairK& k, bool okx, bool oky, float2& ph) {
+  float2 d = f2add(nb, n);
+  if constexpr (MX) d.x = okx ? d.x : 0.f;
+  if constexpr (MY) d.y = oky ? d.y : 0.f;
+  const float2 sq = Q2 ? f2mul(d, d) : f2fma(d, d, f2(1e-30f));
   const float2 la = make_float2(lg2a(sq.x), lg2a(sq.y));
-  const float2 s = f2fma(k.half_qp, la, k.qp_l2);
-  const float2 e = f2add(make_float2(ex2a(s.x), ex2a(s.y)), f2(1.f));
-  const float2 r = make_float2(rcpa(e.x), rcpa(e.y));
+  float2 s = f2fma(k.half_qp, la, k.qp_l2);
+  float2 r;
+  if constexpr (Q2) {
+    s = make_float2(fminf(s.x, 63.f), fminf(s.y, 63.f));
+    const float2 e = f2add(make_float2(ex2a(s.x), ex2a(s.y)), k.one);
+    const float ri = rcpa(e.x * e.y);
+    r = make_float2(ri * e.y, ri * e.x);
+  } else {
+    const float2 e = f2add(make_float2(ex2a(s.x), ex2a(s.y)), k.one);
+    r = make_float2(rcpa(e.x), rcpa(e.y));
+  }
   float2 dr = f2mul(d, r);
   if constexpr (!Q2) {
     const float2 s2 = f2fma(k.half_q2, la, k.q2_l2);
     dr = f2mul(dr, make_float2(ex2a(s2.x), ex2a(s2.y)));
   }
   if constexpr (PH) ph = f2fma(d, dr, ph);
-  return f2mul(dr, f2fma(wq, r, wp));
+  return f2mul(dr, f2fma(k.qmp, r, k.p));
 }
 
 // hi + lo += v with the rounding error of the addition kept in lo (Knuth's TwoSum): the
@@ -1005,186 +1005,220 @@ __device__ __forceinline__ void block_partials_f(float (&hi)[kParts], float (&lo
   }
 }
 
-// class weights of the pair values: wq = w (q - p) / sigma^2, wp = w p / sigma^2 for the face,
-// edge and corner neighbours
-struct PairW {
-  float2 wq[3], wp[3];
+// What the boundary tests know about the block and the lane.
+struct BandB {
+  bool okT, okB;  // image row r0 - 1 (above the first band) and r0 + 2R (below the second) exist
+  bool okL, okR;  // this lane's columns c - 1 and c + 1 exist
 };
-
-// the three pairs (+1, DY, -1 / 0 / +1) from source voxels (a, b) into ring row T of the next
-// slice: +f to the source, -f to the target (own lanes) or sent to the lane that owns it
-template <int N, bool Q2, bool PH, bool ROWE, bool COLE, int DY>
-__device__ __forceinline__ void cross3(float2 y, const float* T, int ia, bool rok, bool okL, bool okR,
-                                       const PriorK& k, const PairW& pw, float2& gsrc, float2& C, float& sR,
-                                       float& sL, float2 (&phr)[3]) {
-  constexpr int CS = DY == 0 ? 1 : 2;  // class of the dx = -1, +1 pairs
-  constexpr int C0 = DY == 0 ? 0 : 1;  // class of the dx = 0 pair
-  float2 f = pairv<Q2, PH>(y, nb_pair<N, -1, ROWE, COLE>(T, ia, y, rok, okL, okR), k, pw.wq[CS], pw.wp[CS], phr[CS]);
-  gsrc = f2add(gsrc, f);
-  sL += f.x;
-  C.x -= f.y;
-  f = pairv<Q2, PH>(y, nb_pair<N, 0, ROWE, COLE>(T, ia, y, rok, okL, okR), k, pw.wq[C0], pw.wp[C0], phr[C0]);
-  gsrc = f2add(gsrc, f);
-  C = f2fma(f, f2(-1.f), C);
-  f = pairv<Q2, PH>(y, nb_pair<N, 1, ROWE, COLE>(T, ia, y, rok, okL, okR), k, pw.wq[CS], pw.wp[CS], phr[CS]);
-  gsrc = f2add(gsrc, f);
-  C.y -= f.x;
-  sR += f.y;
+// The pairs across the warp's outer columns that a lane evaluates, into target row u = lane % R:
+//   zs: the warp's first column from the column before it, rows u (lanes 0 .. R - 1) and u - 1
+//       (R .. 2R - 1), and its last column from the column after it, row u - 1 (2R .. 3R - 1);
+//   zs + 1, the block's first and last warp only, whose neighbours belong to other blocks: that
+//       side's column from rows u - 1, u, u + 1 of zs.
+// The other pairs into slice zs + 1 across a warp's columns are handed over by the neighbouring
+// warp, which has a barrier's time for it.
+struct OuterItem {
+  int src, tgt;  // ring places of the source and the target
+  float w;       // class weight
+  bool on, okx, oky;
+};
+template <int N>
+__device__ __forceinline__ OuterItem outer_item(bool cross, const float2 (&w)[3], const BandB& bb, int warp, int c0w) {
+  using GP = GeoP<N>;
+  constexpr int R = GP::R;
+  const int lane = threadIdx.x & 31, kd = lane / R, u = lane - kd * R;
+  OuterItem it;
+  const bool left = cross ? warp == 0 : kd < 2;
+  const int sr = cross ? kd - 1 : (kd == 0 ? 0 : -1);
+  it.on = kd < 3 && (!cross || warp == 0 || warp == GP::WPB - 1) && (left ? c0w > 0 : c0w + 32 < N);
+  const int tc = 32 * warp + 4 + (left ? 0 : 31);
+  it.tgt = it.on ? (u + 1) * GP::LDR + tc : 0;
+  it.src = it.on ? (u + sr + 1) * GP::LDR + (left ? tc - 1 : tc + 1) : 0;
+  it.w = cross ? (sr != 0 ? w[2].x : w[1].x) : (kd == 0 ? w[0].x : w[1].x);
+  it.okx = u + sr >= 0 || bb.okT;
+  it.oky = u + sr < R || bb.okB;
+  return it;
+}
+// the weighted value of the lane's outer pair, and its sums over the lanes of the same row
+template <int N, bool Q2, bool ROWE>
+__device__ __forceinline__ void outer_sums(const float2* S0, const float2* T, const OuterItem& it, const PairK& k,
+                                           float2& v, float2& v2, float2& v3) {
+  constexpr int R = GeoP<N>::R;
+  float2 unused = f2(0.f);
+  const float2 sv = S0[it.src];
+  v = pairv<Q2, false, true, true>(make_float2(-sv.x, -sv.y), T[it.tgt], k, it.on && (!ROWE || it.okx),
+                                   it.on && (!ROWE || it.oky), unused);
+  v = f2mul(f2(it.w), v);
+  float2 a, b;
+  a.x = __shfl_down_sync(0xffffffffu, v.x, R);
+  a.y = __shfl_down_sync(0xffffffffu, v.y, R);
+  b.x = __shfl_down_sync(0xffffffffu, v.x, 2 * R);
+  b.y = __shfl_down_sync(0xffffffffu, v.y, 2 * R);
+  v2 = f2add(v, a);
+  v3 = f2add(v, f2add(a, b));
 }
 
-// One slice step of a band: every pair whose source voxel lies in slice zs (ring slot S0) and
-// whose other end lies in zs or zs + 1 (slot S1, when have1).  The carried contributions of
-// slice zs (cr, this thread's entries, row stride BC / 2) start the gradient rows and are
-// replaced by those of slice zs + 1.  PRE: only the pairs into slice zs + 1 (a chunk start);
-// otherwise each owned row t is handed to fin(t, gradient sum, y) once complete, with ph the
-// unweighted sigma^2 rho sums by class of the pairs the band owns.  ROWE: the band is the
-// image's first or last; COLE: the warp holds its first or last 64 columns.  Elsewhere every
-// neighbour lies inside the image and the boundary tests drop out.
-template <int N, bool Q2, bool PHI, bool PRE, bool ROWE, bool COLE, class Fin>
-__device__ __forceinline__ void band_step(const float* S0, const float* S1, bool have1, int r0, int c0w, int ia,
-                                          bool okL_, bool okR_, float2* cr, float* edge, const PriorK& k,
-                                          const PairW& pw, float2 (&ph)[3], Fin&& fin) {
+// One slice step of a block's two bands: every pair with an end in the owned rows whose source
+// voxel lies in slice zs (ring slot S0) and whose other end lies in zs or zs + 1 (slot S1, when
+// have1).  The carried contributions of slice zs (cr, this thread's entries, one per row, and the
+// neighbouring warps' shares xin) start the sums of the rows and are replaced by those of slice
+// zs + 1 (cr and the shares xout for the neighbouring warps).  PRE: only the pairs into slice
+// zs + 1 (a chunk start); otherwise pre(u) is called a row ahead and fin(u, h, -y) once row u is
+// complete, with h = -(the prior gradient) and ph the unweighted sigma^2 rho sums by class of the
+// pairs whose target row the band owns.  w: class weights w / sigma^2 (face, edge, corner).  ROWE:
+// the block holds the image's first or last rows; COLE: the warp holds its first or last columns.
+// Elsewhere every neighbour lies inside the image and the boundary tests drop out.
+template <int N, bool Q2, bool PHI, bool PRE, bool ROWE, bool COLE, class Pre, class Fin>
+__device__ __forceinline__ void band_step(const float2* S0, const float2* S1, bool have1, const BandB& bb,
+                                          const OuterItem& it, const OuterItem& itx, int ic, float2* cr, float2* edge,
+                                          const float2* xin, float2* xout, const PairK& k, const float2 (&w)[3],
+                                          float2 (&ph)[3], Pre&& pre, Fin&& fin) {
   using GP = GeoP<N>;
-  constexpr int R = GP::R, LDR = GP::LDR, HALF = GP::NEDGE / 2, CRS = GP::BC / 2;
+  constexpr int R = GP::R, LDR = GP::LDR, CRS = GP::THREADS;
   constexpr bool PH = PHI && !PRE;
-  const int lane = threadIdx.x & 31;
-  const int cw = ia - 4 - 2 * lane;  // ring column of the warp's first column, minus 4
-  const bool top = !ROWE || r0 > 0, bot = !ROWE || r0 + R < N;
-  const bool okL = !COLE || okL_, okR = !COLE || okR_;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const float2 zero = f2(0.f);
+  auto neg = [](float2 v) { return make_float2(-v.x, -v.y); };
+  auto sub = [](float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); };
 
-  // ---- pairs across the warp's outer columns, evaluated by the receiving warp.  Item
-  // kd * R + t is one pair into column c0w (kd < 5) or c0w + 63 (kd >= 5) of row t:
-  //   kd 0: (0, 0, +1) from row t       kd 5: (0, +1, -1) from row t - 1
-  //   kd 1: (0, +1, +1) from row t - 1  kd 6..8: (+1, -1 / 0 / +1, -1) from rows t + 1, t, t - 1
-  //   kd 2..4: (+1, -1 / 0 / +1, +1) from rows t + 1, t, t - 1
-  // (kd 2..4 and 6..8 land in slice zs + 1).  Two items per lane; slot = -f for the target.
-  if (lane < HALF) {
-    float ys[2], yt[2], wq[2], wp[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = lane + h * HALF;
-      const int kd = i / R, t = i - kd * R;
-      const bool left = kd < 5;
-      const int sr = (kd == 0 || kd == 3 || kd == 7) ? 0 : ((kd == 2 || kd == 6) ? 1 : -1);
-      const bool cross = kd >= 2 && kd != 5;
-      const int cls = kd == 0 ? 0 : ((kd & 1) ? 1 : 2);
-      const int tr = t + sr;
-      const bool ok = (!ROWE || (r0 + tr >= 0 && r0 + tr < N)) && (!COLE || (left ? c0w > 0 : c0w + 64 < N)) &&
-                      (cross ? have1 : !PRE);
-      const float tv = (cross ? S1 : S0)[(t + 1) * LDR + cw + (left ? 4 : 67)];
-      const float sv = S0[(tr + 1) * LDR + cw + (left ? 3 : 68)];
-      ys[h] = ok ? sv : tv;
-      yt[h] = tv;
-      wq[h] = cls == 0 ? pw.wq[0].x : (cls == 1 ? pw.wq[1].x : pw.wq[2].x);
-      wp[h] = cls == 0 ? pw.wp[0].x : (cls == 1 ? pw.wp[1].x : pw.wp[2].x);
+  // ---- the pairs across the warp's outer columns (OuterItem), summed per target row
+  {
+    float2 v, v2, v3;
+    if constexpr (!PRE) {
+      outer_sums<N, Q2, ROWE>(S0, S0, it, k, v, v2, v3);
+      if (lane < R) edge[lane] = v2;
+      if (lane >= 2 * R && lane < 3 * R) edge[lane - R] = v;
     }
-    float2 unused;
-    const float2 f = pairv<Q2, false>(make_float2(ys[0], ys[1]), make_float2(yt[0], yt[1]), k,
-                                      make_float2(wq[0], wq[1]), make_float2(wp[0], wp[1]), unused);
-    edge[lane] = -f.x;
-    edge[lane + HALF] = -f.y;
+    if (have1 && (warp == 0 || warp == GP::WPB - 1)) {
+      outer_sums<N, Q2, ROWE>(S0, S1, itx, k, v, v2, v3);
+      if (lane < R) edge[2 * R + lane] = v3;
+    }
   }
   __syncwarp();
+  // lane 0 starts its rows from the left sums, lane 31 from the right ones, the others from zero; into
+  // slice zs + 1 only the block's outer lanes
+  const float2* es = edge + (lane == 0 ? 0 : (lane == 31 ? R : 3 * R));
+  const float2* ex =
+      edge + ((lane == 0 && warp == 0) || (lane == 31 && warp == GP::WPB - 1) ? 2 * R : 3 * R);
+  // the share of lane 31's pairs belongs to the next warp's first column, lane 0's to the last of the one before
+  float2* xo = xout + (lane == 31 ? (warp + 2) * R : (GP::WPB + 2) * R + warp * R);
+  const float2* xi = xin + (lane == 31 ? (GP::WPB + 2) * R : 0) + (lane == 0 || lane == 31 ? (warp + 1) * R : 0);
 
-  // ---- the row walk: source rows -1 .. R of slice zs (ring row t + 1 holds image row r0 + t),
-  // unrolled at compile time so that the row tests and the window slides cost nothing
-  const float2 zero = f2(0.f);
-  float2 gc = zero, gn = PRE ? zero : cr[0];                                // gradient rows t, t + 1
-  float2 cm = zero, cc = zero, cp = zero;                                   // carry rows t - 1, t, t + 1
-  float sRc = 0.f, sRn = 0.f, sLc = 0.f, sLn = 0.f;                         // sends into rows t, t + 1
-  float sR1m = 0.f, sR1c = 0.f, sR1p = 0.f, sL1m = 0.f, sL1c = 0.f, sL1p = 0.f;
-  SFor<-1, R + 1>::run([&](auto t_) {
-    constexpr int t = decltype(t_)::value;
-    constexpr bool own = t >= 0 && t < R;
-    const float* rowt = S0 + (t + 1) * LDR;  // slice zs, row t
-    const float2 y = *reinterpret_cast<const float2*>(rowt + ia);
-    float2 phr[3] = {zero, zero, zero};
-    if constexpr (!PRE && own) {  // (0, 0, +1), face
-      const float2 f = pairv<Q2, PH>(y, nb_pair<N, 1, ROWE, COLE>(rowt, ia, y, true, okL, okR), k, pw.wq[0], pw.wp[0],
-                                     phr[0]);
-      gc = f2add(gc, f);
-      gc.y -= f.x;
-      sRc += f.y;
+  // the neighbouring lanes' shares (dx = +-1) added to a target row's sum
+  const bool inL = lane > 0, inR = lane < 31;
+  auto receive = [&](float2 c, float2 sR, float2 sL) {
+    float2 a, b;
+    a.x = __shfl_up_sync(0xffffffffu, sR.x, 1);
+    a.y = __shfl_up_sync(0xffffffffu, sR.y, 1);
+    b.x = __shfl_down_sync(0xffffffffu, sL.x, 1);
+    b.y = __shfl_down_sync(0xffffffffu, sL.y, 1);
+    a = make_float2(inL ? a.x : 0.f, inL ? a.y : 0.f);
+    b = make_float2(inR ? b.x : 0.f, inR ? b.y : 0.f);
+    return f2add(c, f2add(a, b));
+  };
+  // carried sums of a row: the thread's own and, at the warp's ends, the neighbouring warp's
+  auto carried = [&](int u) { return sub(neg(cr[u * CRS]), xi[u]); };
+  // a pair at column offset DX; mx, my: the first / second half's row exists (ROWE only)
+  auto pair = [&](auto DX_, auto PH_, float2 n, float2 nb, bool mx, bool my, float2& p) {
+    constexpr int DX = decltype(DX_)::value;
+    constexpr bool C = COLE && DX != 0;
+    const bool okc = DX < 0 ? bb.okL : bb.okR;
+    return pairv<Q2, decltype(PH_)::value, ROWE || C, ROWE || C>(n, nb, k, (!ROWE || mx) && (!C || okc),
+                                                                 (!ROWE || my) && (!C || okc), p);
+  };
+  using Lf = std::integral_constant<int, -1>;
+  using Ce = std::integral_constant<int, 0>;
+  using Ri = std::integral_constant<int, 1>;
+  using No = std::false_type;
+  using Ph = std::integral_constant<bool, PH>;
+  float2 unused = zero;
+
+  // ---- the row walk
+  const float2* p0 = S0 + ic;       // row u - 1 of slice zs while row u is the target
+  const float2* p1 = S1 + LDR + ic; // row u of slice zs + 1
+  float2 nm = neg(p0[0]), n0 = neg(p0[LDR]);  // -y of rows u - 1, u
+  float2 hm = zero, h0 = PRE ? zero : carried(0);  // their sums
+  if (!PRE && have1) {  // u = -1: source row 0
+    h0 = f2fma(w[2], pair(Lf{}, No{}, n0, p1[-LDR - 1], bb.okT, true, unused), h0);
+    h0 = f2fma(w[1], pair(Ce{}, No{}, n0, p1[-LDR], bb.okT, true, unused), h0);
+    h0 = f2fma(w[2], pair(Ri{}, No{}, n0, p1[-LDR + 1], bb.okT, true, unused), h0);
+  }
+#pragma unroll 1
+  for (int u = 0; u < R; ++u) {
+    const bool mT = u > 0 || bb.okT, mB = u + 1 < R || bb.okB;  // rows u - 1 / u + 1 exist in both halves
+    const float2 np = neg(p0[2 * LDR]);
+    float2 hp = PRE || u + 1 >= R ? zero : carried(u + 1);
+    if constexpr (!PRE) {
+      pre(u);
+      const float2 L = p0[LDR - 1], C = p0[LDR], Rr = p0[LDR + 1];
+      float2 c = es[u], sR, sL;
+      // from row u - 1: (0, +1, -1 / 0 / +1)
+      float2 v = pair(Lf{}, Ph{}, nm, L, mT, true, ph[1]);
+      hm = f2fma(w[1], v, hm);
+      sL = f2mul(w[1], v);
+      v = pair(Ce{}, Ph{}, nm, C, mT, true, ph[0]);
+      hm = f2fma(w[0], v, hm);
+      c = f2fma(w[0], v, c);
+      v = pair(Ri{}, Ph{}, nm, Rr, mT, true, ph[1]);
+      hm = f2fma(w[1], v, hm);
+      sR = f2mul(w[1], v);
+      // (0, 0, +1), then the row's total
+      v = pair(Ri{}, Ph{}, n0, Rr, true, true, ph[0]);
+      h0 = f2fma(w[0], v, h0);
+      sR = f2fma(w[0], v, sR);
+      h0 = sub(h0, receive(c, sR, sL));
     }
-    if constexpr (!PRE && t < R) {
-      if (own || top) {  // (0, +1, -1 / 0 / +1) into row t + 1
-        const bool rok = !ROWE || r0 + t + 1 < N;
-        const float* rown = rowt + LDR;
-        float2 f = pairv<Q2, PH>(y, nb_pair<N, -1, ROWE, COLE>(rown, ia, y, rok, okL, okR), k, pw.wq[1], pw.wp[1], phr[1]);
-        gc = f2add(gc, f);
-        sLn += f.x;
-        gn.x -= f.y;
-        f = pairv<Q2, PH>(y, nb_pair<N, 0, ROWE, COLE>(rown, ia, y, rok, okL, okR), k, pw.wq[0], pw.wp[0], phr[0]);
-        gc = f2add(gc, f);
-        gn = f2fma(f, f2(-1.f), gn);
-        f = pairv<Q2, PH>(y, nb_pair<N, 1, ROWE, COLE>(rown, ia, y, rok, okL, okR), k, pw.wq[1], pw.wp[1], phr[1]);
-        gc = f2add(gc, f);
-        gn.y -= f.x;
-        sRn += f.y;
-      }
+    if (have1) {
+      const float2 L = p1[-1], C = p1[0], Rr = p1[1];
+      float2 c = ex[u], sR = zero, sL = zero;
+      // the three pairs from one source row
+      auto three = [&](auto CS_, float2 n, float2& h, bool mx, bool my) {
+        constexpr int CS = decltype(CS_)::value, C0 = CS - 1;
+        float2 v = pair(Lf{}, Ph{}, n, L, mx, my, ph[CS]);
+        h = f2fma(w[CS], v, h);
+        sL = f2fma(w[CS], v, sL);
+        v = pair(Ce{}, Ph{}, n, C, mx, my, ph[C0]);
+        h = f2fma(w[C0], v, h);
+        c = f2fma(w[C0], v, c);
+        v = pair(Ri{}, Ph{}, n, Rr, mx, my, ph[CS]);
+        h = f2fma(w[CS], v, h);
+        sR = f2fma(w[CS], v, sR);
+      };
+      using Diag = std::integral_constant<int, 2>;
+      three(Diag{}, nm, hm, mT, true);
+      three(std::integral_constant<int, 1>{}, n0, h0, true, true);
+      three(Diag{}, np, hp, true, mB);
+      cr[u * CRS] = receive(c, sR, sL);
+      if (!inL) xo[u] = sL;
+      if (!inR) xo[u] = sR;
     }
-    if (have1) {  // (+1, dy, dx) into rows t - 1, t, t + 1 of slice zs + 1
-      if constexpr (t >= 0) {
-        if (own || bot)
-          cross3<N, Q2, PH, ROWE, COLE, -1>(y, S1 + t * LDR, ia, !ROWE || r0 + t - 1 >= 0, okL, okR, k, pw, gc, cm, sR1m,
-                                      sL1m, phr);
-      }
-      if constexpr (own)
-        cross3<N, Q2, PH, ROWE, COLE, 0>(y, S1 + (t + 1) * LDR, ia, true, okL, okR, k, pw, gc, cc, sR1c, sL1c, phr);
-      if constexpr (t < R) {
-        if (own || top)
-          cross3<N, Q2, PH, ROWE, COLE, 1>(y, S1 + (t + 2) * LDR, ia, !ROWE || r0 + t + 1 < N, okL, okR, k, pw, gc, cp,
-                                     sR1p, sL1p, phr);
-      }
-    }
-    if constexpr (PH && own) {
-#pragma unroll
-      for (int j = 0; j < 3; ++j) ph[j] = f2add(ph[j], phr[j]);
-    }
-    // gradient row t (in-plane sources t - 1, t) and carry row t - 1 (sources t - 2 .. t) are
-    // complete: take the neighbouring lanes' shares
-    if constexpr (!PRE && own) {
-      const float rx = __shfl_up_sync(0xffffffffu, sRc, 1), lx = __shfl_down_sync(0xffffffffu, sLc, 1);
-      gc.x -= lane > 0 ? rx : 0.f;
-      gc.y -= lane < 31 ? lx : 0.f;
-      if (lane == 0) gc.x += edge[t] + edge[R + t];
-      if (lane == 31) gc.y += edge[5 * R + t];
-      fin(t, gc, y);
-    }
-    if constexpr (t >= 1) {
-      const float rx1 = __shfl_up_sync(0xffffffffu, sR1m, 1), lx1 = __shfl_down_sync(0xffffffffu, sL1m, 1);
-      cm.x -= lane > 0 ? rx1 : 0.f;
-      cm.y -= lane < 31 ? lx1 : 0.f;
-      if (lane == 0) cm.x += edge[2 * R + t - 1] + edge[3 * R + t - 1] + edge[4 * R + t - 1];
-      if (lane == 31) cm.y += edge[6 * R + t - 1] + edge[7 * R + t - 1] + edge[8 * R + t - 1];
-      cr[(t - 1) * CRS] = cm;
-    }
+    if constexpr (!PRE)
+      if (u >= 1) fin(u - 1, hm, nm);
     // slide the windows down one row
-    gc = gn;
-    if constexpr (!PRE && t + 2 < R)
-      gn = cr[(t + 2) * CRS];
-    else
-      gn = zero;
-    sRc = sRn;
-    sRn = 0.f;
-    sLc = sLn;
-    sLn = 0.f;
-    cm = cc;
-    cc = cp;
-    cp = zero;
-    sR1m = sR1c;
-    sR1c = sR1p;
-    sR1p = 0.f;
-    sL1m = sL1c;
-    sL1c = sL1p;
-    sL1p = 0.f;
-  });
+    nm = n0;
+    n0 = np;
+    hm = h0;
+    h0 = hp;
+    p0 += LDR;
+    p1 += LDR;
+  }
+  if constexpr (!PRE) {  // u = R: source row R - 1
+    hm = f2fma(w[1], pair(Lf{}, No{}, nm, p0[LDR - 1], true, bb.okB, unused), hm);
+    hm = f2fma(w[0], pair(Ce{}, No{}, nm, p0[LDR], true, bb.okB, unused), hm);
+    hm = f2fma(w[1], pair(Ri{}, No{}, nm, p0[LDR + 1], true, bb.okB, unused), hm);
+    if (have1) {
+      hm = f2fma(w[2], pair(Lf{}, No{}, nm, p1[-1], true, bb.okB, unused), hm);
+      hm = f2fma(w[1], pair(Ce{}, No{}, nm, p1[0], true, bb.okB, unused), hm);
+      hm = f2fma(w[2], pair(Ri{}, No{}, nm, p1[1], true, bb.okB, unused), hm);
+    }
+    fin(R - 1, hm, nm);
+  }
 }
 
 // kz: K (*) y of the group from pass 3a ([slice][row][col]); phase: in Iterate mode, the storage
 // phase this launch belongs to (0 FP32, 1 BF16), checked like the other passes.
 template <int N, int MODE, bool Q2, bool MULTI>
-__global__ void __launch_bounds__(GeoP<N>::THREADS, 2)
+__global__ void __launch_bounds__(GeoP<N>::THREADS, 512 / GeoP<N>::THREADS)
     k_pass3(const __grid_constant__ GroupSet gs, StepArgs a, PriorC pc, const float* apply_out, int phase,
             double* partials, int block_offset) {
   using GP = GeoP<N>;
@@ -1229,11 +1263,10 @@ __global__ void __launch_bounds__(GeoP<N>::THREADS, 2)
   const int cb = (bid_ / GP::NB) % GP::CB;
   const int chunk = bid_ / (GP::NB * GP::CB);
   const int z0 = g.zlo + chunk * zc, z1 = min(g.zlo + (g.zn > 0 ? g.zn : S), z0 + zc);
-  const int r0 = band * R, c0 = cb * GP::BC;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int c0w = c0 + 64 * warp;
-  const int acol = c0w + 2 * lane;  // this lane's voxels: columns acol, acol + 1
-  const int ia = 64 * warp + 2 * lane + 4;
+  const int r0 = band * GP::ROWS, c0 = cb * GP::BC;
+  const int warp = threadIdx.x >> 5;
+  const int col = c0 + threadIdx.x;  // this lane's column
+  const int ic = threadIdx.x + 4;    // and its place in a ring row
   const size_t N2 = (size_t)N * N;
 
   float hi[kParts], lo[kParts];  // compensated FP32 sums of the block's slices
@@ -1243,122 +1276,127 @@ __global__ void __launch_bounds__(GeoP<N>::THREADS, 2)
   if constexpr (!PRIOR) {
     // Apply: pass 3a wrote K (*) x to the output itself; only the partial sums remain
     for (int z = z0; z < z1; ++z) {
-      float2 acc0 = f2(0.f), acc5 = f2(0.f);
+      float acc0 = 0.f, acc5 = 0.f;
 #pragma unroll
-      for (int t = 0; t < R; ++t) {
-        const size_t o = (size_t)z * N2 + (size_t)(r0 + t) * N + acol;
-        const float2 zd = __ldg(reinterpret_cast<const float2*>(kz + o));
-        const float2 xv = __ldg(reinterpret_cast<const float2*>(x + o));
-        acc0 = f2fma(xv, zd, acc0);
-        acc5 = f2fma(zd, zd, acc5);
+      for (int t = 0; t < GP::ROWS; ++t) {
+        const size_t o = (size_t)z * N2 + (size_t)(r0 + t) * N + col;
+        const float zd = __ldg(kz + o), xv = __ldg(x + o);
+        acc0 = fmaf(xv, zd, acc0);
+        acc5 = fmaf(zd, zd, acc5);
       }
-      two_sum_add(hi[0], lo[0], acc0.x + acc0.y);
-      two_sum_add(hi[5], lo[5], acc5.x + acc5.y);
+      two_sum_add(hi[0], lo[0], acc0);
+      two_sum_add(hi[5], lo[5], acc5);
     }
   } else {
-    const PriorK pk = prior_k(pc);
-    PairW pw;
-    const float wcls[3] = {pc.wf * pc.inv_sig2, pc.we * pc.inv_sig2, pc.wc * pc.inv_sig2};
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      pw.wq[j] = f2(wcls[j] * pc.qp);
-      pw.wp[j] = f2(wcls[j] * pc.p);
-    }
-    const float2 lam = f2(pc.lam);
-    const bool okL = acol > 0, okR = acol + 2 < N;
-    float* ring = reinterpret_cast<float*>(sm);
-    constexpr int SLOT = 2 * GP::RING;  // y and its shifted copy
-    float* stg = ring + 2 * SLOT;
-    float2* cr = reinterpret_cast<float2*>(stg + 2 * GP::RING) + 32 * warp + lane;
-    float* edge = stg + 2 * GP::RING + R * GP::BC + warp * GP::NEDGE;
-    float2* fin_in = reinterpret_cast<float2*>(stg + 2 * GP::RING + R * GP::BC + GP::WPB * GP::NEDGE) + threadIdx.x;
-    // K (*) y, R*g and x_k of row t of slice zz at this thread's voxels, into fin_in
-    auto fetch = [&](int zz, int t) {
-      const size_t o = (size_t)zz * N2 + (size_t)(r0 + t) * N + acol;
-      float2* d = fin_in + 3 * t * GP::THREADS;
-      tc05::cp_async8(d, kz + o);
-      tc05::cp_async8(d + GP::THREADS, atg + o);
-      if constexpr (UPDATE) tc05::cp_async8(d + 2 * GP::THREADS, x + o);
-    };
+    const PairK pk = pair_k<Q2>(pc);
+    const float2 w[3] = {pin(f2(pc.wf * pc.inv_sig2)), pin(f2(pc.we * pc.inv_sig2)), pin(f2(pc.wc * pc.inv_sig2))};
+    const float2 mlam = f2(-pc.lam);
+    BandB bb;
+    bb.okT = r0 > 0;
+    bb.okB = r0 + GP::ROWS < N;
+    const int c0w = c0 + 32 * warp;
+    bb.okL = col > 0;
+    bb.okR = col + 1 < N;
+    const OuterItem it = outer_item<N>(false, w, bb, warp, c0w), itx = outer_item<N>(true, w, bb, warp, c0w);
+    float2* ring = sm;
+    float2* cr = ring + 2 * GP::RING + threadIdx.x;
+    float2* edge = ring + 2 * GP::RING + R * GP::THREADS + warp * GP::EDGE;
+    float2* xch = ring + 2 * GP::RING + R * GP::THREADS + GP::WPB * GP::EDGE;
+    float* stg = reinterpret_cast<float*>(xch + 2 * GP::XCH);
+    if ((threadIdx.x & 31) < R) edge[3 * R + (threadIdx.x & 31)] = f2(0.f);
+    // shares[parity]: [side][warp + 1][row]; the places beyond the block's warps stay zero
+    for (int i = threadIdx.x; i < 2 * GP::XCH; i += GP::THREADS) xch[i] = f2(0.f);
     float2 ph[3] = {f2(0.f), f2(0.f), f2(0.f)};
-    load_ring_p<N>(ring + (z0 & 1) * SLOT, x, xp, beta, (size_t)z0 * N2, r0, c0);
+    load_ring_p<N>(ring + (z0 & 1) * GP::RING, x, xp, beta, (size_t)z0 * N2, r0, c0);
     if (z0 > 0) {
-      load_ring_p<N>(ring + ((z0 - 1) & 1) * SLOT, x, xp, beta, (size_t)(z0 - 1) * N2, r0, c0);
+      load_ring_p<N>(ring + ((z0 - 1) & 1) * GP::RING, x, xp, beta, (size_t)(z0 - 1) * N2, r0, c0);
     } else {
 #pragma unroll
-      for (int t = 0; t < R; ++t) cr[t * (GP::BC / 2)] = f2(0.f);
+      for (int t = 0; t < R; ++t) cr[t * GP::THREADS] = f2(0.f);
     }
-    __syncthreads();
-    ring_shift<N>(ring + (z0 & 1) * SLOT);
-    if (z0 > 0) ring_shift<N>(ring + ((z0 - 1) & 1) * SLOT);
-    if (z0 + 1 < S) stage_issue<N>(stg, x, xp, (size_t)(z0 + 1) * N2, r0, c0);
-#pragma unroll
-    for (int t = 0; t < R; ++t) fetch(z0, t);
+    const Stager<N> stager(stg, x, xp, r0, c0);
+    if (z0 + 1 < S) stager.issue((size_t)(z0 + 1) * N2);
     __syncthreads();
     // boundary tests only where the warp's neighbourhoods leave the image
-    const bool rowe = !(r0 > 0 && r0 + R < N), cole = !(c0w > 0 && c0w + 64 < N);
+    const bool rowe = !(bb.okT && bb.okB), cole = !(c0w > 0 && c0w + 32 < N);
+    auto none = [](int) {};
     if (z0 > 0) {
       auto fin0 = [](int, float2, float2) {};
-      const float* s0 = ring + ((z0 - 1) & 1) * SLOT;
-      const float* s1 = ring + (z0 & 1) * SLOT;
-      if (rowe)
-        band_step<N, Q2, PHI, true, true, true>(s0, s1, true, r0, c0w, ia, okL, okR, cr, edge, pk, pw, ph, fin0);
-      else if (cole)
-        band_step<N, Q2, PHI, true, false, true>(s0, s1, true, r0, c0w, ia, okL, okR, cr, edge, pk, pw, ph, fin0);
+      const float2* s0 = ring + ((z0 - 1) & 1) * GP::RING;
+      const float2* s1 = ring + (z0 & 1) * GP::RING;
+      float2* xo0 = xch + (z0 & 1) * GP::XCH;
+      const float2* xi0 = xo0;  // not read
+      if (rowe || cole)
+        band_step<N, Q2, PHI, true, true, true>(s0, s1, true, bb, it, itx, ic, cr, edge, xi0, xo0, pk, w, ph, none, fin0);
       else
-        band_step<N, Q2, PHI, true, false, false>(s0, s1, true, r0, c0w, ia, okL, okR, cr, edge, pk, pw, ph, fin0);
+        band_step<N, Q2, PHI, true, false, false>(s0, s1, true, bb, it, itx, ic, cr, edge, xi0, xo0, pk, w, ph, none, fin0);
     }
     for (int z = z0; z < z1; ++z) {
       // every thread has finished slice z - 1, so its ring slot takes slice z + 1 from the
       // staging area; then the staging area takes slice z + 2 while slice z is worked on
       tc05::cp_async_wait_all();
       __syncthreads();
-      if (z + 1 < S) stage_to_ring<N>(ring + ((z + 1) & 1) * SLOT, stg, beta);
+      if (z + 1 < S) stage_to_ring<N>(ring + ((z + 1) & 1) * GP::RING, stg, beta);
       __syncthreads();
-      if (z + 1 < z1 && z + 2 < S) stage_issue<N>(stg, x, xp, (size_t)(z + 2) * N2, r0, c0);
+      if (z + 1 < z1 && z + 2 < S) stager.issue((size_t)(z + 2) * N2);
       float2 acc[kParts];
 #pragma unroll
       for (int j = 0; j < kParts; ++j) acc[j] = f2(0.f);
-      const size_t img = (size_t)z * N2 + acol;
-      const bool more = z + 1 < z1;
-      auto fin = [&](int t, float2 gsum, float2 yv) {
-        const size_t ro = (size_t)(r0 + t) * N;
-        const float2* v = fin_in + 3 * t * GP::THREADS;
-        const float2 zd = v[0], at = v[GP::THREADS];
-        const float2 Gv = f2fma(lam, gsum, f2fma(at, f2(-1.f), zd));
+      const size_t img = (size_t)z * N2 + (size_t)r0 * N + col;
+      const float *kzp = kz + img, *atp = atg + img, *xkp = x + img;
+      float* op = out + img;
+      // K (*) y, R*g and x_k of row u, loaded while the rows u - 1 and u are worked on
+      float2 zd, at, xv, zdn, atn, xvn;
+      zd = at = xv = zdn = atn = xvn = f2(0.f);
+      auto pre = [&](int u) {
+        zd = zdn;
+        at = atn;
+        zdn = make_float2(__ldg(kzp + u * N), __ldg(kzp + (u + R) * N));
+        atn = make_float2(__ldg(atp + u * N), __ldg(atp + (u + R) * N));
+        if constexpr (UPDATE) {
+          xv = xvn;
+          xvn = make_float2(__ldg(xkp + u * N), __ldg(xkp + (u + R) * N));
+        }
+      };
+      auto fin = [&](int u, float2 h, float2 n) {
+        if (u == R - 1) {  // the last row was not followed by another
+          zd = zdn;
+          at = atn;
+          xv = xvn;
+        }
+        const float2 yv = make_float2(-n.x, -n.y);
+        const float2 Gv = f2fma(mlam, h, make_float2(zd.x - at.x, zd.y - at.y));
         acc[0] = f2fma(yv, zd, acc[0]);
         acc[1] = f2fma(yv, at, acc[1]);
         acc[4] = f2fma(Gv, Gv, acc[4]);
         if constexpr (MODE == (int)Pass3Mode::Gradient) {
-          *reinterpret_cast<float2*>(out + img + ro) = Gv;
+          op[u * N] = Gv.x;
+          op[(u + R) * N] = Gv.y;
         } else if constexpr (UPDATE) {
-          const float2 xv = v[2 * GP::THREADS];
           float2 xn = f2fma(f2(-invL), Gv, yv);
           if (pc.nonneg) xn = make_float2(fmaxf(xn.x, 0.f), fmaxf(xn.y, 0.f));
-          *reinterpret_cast<float2*>(out + img + ro) = xn;
-          acc[3] = f2fma(Gv, f2fma(xv, f2(-1.f), xn), acc[3]);
+          op[u * N] = xn.x;
+          op[(u + R) * N] = xn.y;
+          acc[3] = f2fma(Gv, make_float2(xn.x - xv.x, xn.y - xv.y), acc[3]);
         }
-        if (more) fetch(z + 1, t);  // this row's slots are free again
       };
-      const float* s0 = ring + (z & 1) * SLOT;
-      const float* s1 = ring + ((z + 1) & 1) * SLOT;
-      if (rowe)
-        band_step<N, Q2, PHI, false, true, true>(s0, s1, z + 1 < S, r0, c0w, ia, okL, okR, cr, edge, pk, pw, ph, fin);
-      else if (cole)
-        band_step<N, Q2, PHI, false, false, true>(s0, s1, z + 1 < S, r0, c0w, ia, okL, okR, cr, edge, pk, pw, ph,
-                                                  fin);
+      const float2* s0 = ring + (z & 1) * GP::RING;
+      const float2* s1 = ring + ((z + 1) & 1) * GP::RING;
+      const float2* xi = xch + (z & 1) * GP::XCH;        // what slice z - 1 handed over
+      float2* xo = xch + ((z + 1) & 1) * GP::XCH;
+      if (rowe || cole)
+        band_step<N, Q2, PHI, false, true, true>(s0, s1, z + 1 < S, bb, it, itx, ic, cr, edge, xi, xo, pk, w, ph, pre, fin);
       else
-        band_step<N, Q2, PHI, false, false, false>(s0, s1, z + 1 < S, r0, c0w, ia, okL, okR, cr, edge, pk, pw, ph,
-                                                   fin);
+        band_step<N, Q2, PHI, false, false, false>(s0, s1, z + 1 < S, bb, it, itx, ic, cr, edge, xi, xo, pk, w, ph, pre, fin);
       if constexpr (PHI) {
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-          acc[2] = f2fma(f2(wcls[j]), ph[j], acc[2]);
+          acc[2] = f2fma(w[j], ph[j], acc[2]);
           ph[j] = f2(0.f);
         }
       }
 #pragma unroll
-      for (int j = 0; j < kParts; ++j) two_sum_add(hi[j], lo[j], acc[j].x + acc[j].y);
+      for (int j = 0; j < 5; ++j) two_sum_add(hi[j], lo[j], acc[j].x + acc[j].y);
     }
   }
   block_partials_f<GP::WPB>(hi, lo, red, partials + (size_t)(block_offset + blockIdx.x) * kParts);
