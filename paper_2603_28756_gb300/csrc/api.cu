@@ -50,9 +50,6 @@ static std::mutex g_tune_mu;
 static std::map<std::pair<int, int>, int> g_tuned_zc;
 // slices per spectrum chunk chosen by tmbir_autotune, keyed the same way
 static std::map<std::pair<int, int>, int> g_tuned_sc;
-// rows per block of passes 1 and 3a (sides with variants), keyed the same way
-static std::map<std::pair<int, int>, std::pair<int, int>> g_tuned_rb;
-
 static int tuned_zc(int N, int S) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   auto it = g_tuned_zc.find({N, S});
@@ -62,11 +59,6 @@ static int tuned_sc(int N, int S) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   auto it = g_tuned_sc.find({N, S});
   return it == g_tuned_sc.end() ? 0 : it->second;
-}
-static std::pair<int, int> tuned_rb(int N, int S) {
-  std::lock_guard<std::mutex> lk(g_tune_mu);
-  auto it = g_tuned_rb.find({N, S});
-  return it == g_tuned_rb.end() ? std::make_pair(0, 0) : it->second;
 }
 
 // ---------------------------------------------------------------- small device kernels
@@ -403,8 +395,6 @@ int tmbir_set_workspace(tmbir_ctx* ctx, void* d_ws, size_t bytes) {
     d.span = (float)g.span;
     d.zc = tuned_zc(d.N, d.S);
     d.sc = tuned_sc(d.N, d.S);
-    d.rb1 = tuned_rb(d.N, d.S).first;
-    d.rb3 = tuned_rb(d.N, d.S).second;
     d.chat = reinterpret_cast<float*>(ws + c.off_chat[i]);
     d.twN = reinterpret_cast<float2*>(ws + c.off_twN[i]);
     d.twM = reinterpret_cast<float2*>(ws + c.off_twM[i]);
@@ -429,16 +419,21 @@ int tmbir_set_workspace(tmbir_ctx* ctx, void* d_ws, size_t bytes) {
                                  c.stream));
       d.wts = w;
     }
-    // twiddle tables: twN[k][t] = exp(-2 pi i t k / N) in the group-FFT layout (the plain
-    // table exp(-2 pi i j / N) for the block-FFT sides), twM[n] = exp(-2 pi i n / 2N)
+    // twiddle tables: twN[k][t] = exp(-2 pi i t k / TP) of the side's group FFT, for the sides split into
+    // 512-point transforms followed by exp(-2 pi i 2^l m / 2N), m < 512, l = 1, 2, 3 as far as the side
+    // uses them; twM[n] = exp(-2 pi i n / 2N)
     int T, P;
     fft_shape(g.N, &T, &P);
     std::vector<float2> twN((size_t)T * P), twM(g.N);
     for (int k = 0; k < P; ++k)
       for (int t = 0; t < T; ++t) {
-        const long long q = block_fft_N(g.N) ? (long long)k * T + t : (long long)t * k % g.N;
-        const double a = -2.0 * M_PI * (double)q / g.N;
+        const double a = -2.0 * M_PI * (double)((long long)t * k % (T * P)) / (T * P);
         twN[(size_t)k * T + t] = make_float2((float)std::cos(a), (float)std::sin(a));
+      }
+    for (int l = 1; chat_split(g.N) > 2 && 1 << l < chat_split(g.N); ++l)
+      for (int m = 0; m < 512; ++m) {
+        const double a = -M_PI * (double)((m << l) % (2 * g.N)) / g.N;
+        twN.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
       }
     for (int n = 0; n < g.N; ++n) {
       const double a = -M_PI * (double)n / g.N;
@@ -1211,35 +1206,6 @@ int tmbir_autotune(tmbir_ctx* ctx, const float* d_x, const float* d_atg, const t
       if (h_sc) h_sc[i] = best_sc;
       std::lock_guard<std::mutex> lk(g_tune_mu);
       g_tuned_sc[{g.N, g.S}] = best_sc;
-    }
-    // rows per block of passes 1 and 3a, where the side has variants (4 or 8 rows)
-    if (g.N == 2048) {
-      auto time_ms = [&](auto&& launch, float* out) {
-        for (int rep = 0; rep < 3 && rc == TMBIR_OK; ++rep) {
-          if (rep == 1) cudaEventRecord(e0, s);
-          rc = launch();
-        }
-        if (rc) return;
-        cudaEventRecord(e1, s);
-        if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(out, e0, e1) != cudaSuccess)
-          rc = set_error(TMBIR_ERR_CUDA, "autotune: event timing failed");
-      };
-      float best1 = 1e30f, best3 = 1e30f;
-      int rb1 = 4, rb3 = 8;
-      for (int rb : {4, 8}) {
-        float t1 = 0.f, t3 = 0.f;
-        g.rb1 = g.rb3 = rb;
-        time_ms([&] { return launch_pass1(g, a, s, false); }, &t1);
-        time_ms([&] { return launch_pass3(g, a, Pass3Mode::Iterate, pc, nullptr, 0, s, false, 1); }, &t3);
-        if (rc) break;
-        if (t1 < best1) best1 = t1, rb1 = rb;
-        if (t3 < best3) best3 = t3, rb3 = rb;
-      }
-      if (rc) break;
-      g.rb1 = rb1;
-      g.rb3 = rb3;
-      std::lock_guard<std::mutex> lk(g_tune_mu);
-      g_tuned_rb[{g.N, g.S}] = {rb1, rb3};
     }
     if ((rc = launch_convolution(g, a, Pass3Mode::Iterate, pc, s))) break;
     std::vector<int> cands;

@@ -230,9 +230,7 @@ __device__ __forceinline__ void reg_dft(C (&a)[P]) {
 
 // ---------------------------------------------------------------- group FFT of length n = T * P
 // Thread layout in and out: thread t of the group holds x[t + T*i], i < P.
-// tw: table of exp(-2*pi*i*t*k1/n) at tw[k1 * TWS * T + t] (conjugated on the fly for the
-// inverse); TWS = 1 is the table [P][T] of this length, TWS = 2 reads every other row of the
-// table of a transform twice as long (exp(-2 pi i t (2 k1) / 2n) = exp(-2 pi i t k1 / n)).
+// tw: table of exp(-2*pi*i*t*k1/n) at tw[k1 * T + t] (conjugated on the fly for the inverse).
 // sm: T*(P+1) complex values of shared memory owned by this group.
 template <int T_, int P_>
 struct GroupFFT {
@@ -243,12 +241,12 @@ struct GroupFFT {
   static_assert(P % T == 0, "P must be a multiple of T");
   static_assert(T <= 32 && (32 % T) == 0, "group must divide a warp");
 
-  template <int DIR, class C, int TWS = 1>
+  template <int DIR, class C>
   __device__ __forceinline__ static void run(C (&v)[P], C* sm, const C* __restrict__ tw, int t) {
     reg_dft<P, DIR, C>(v);
     SFor<1, P>::run([&](auto k_) {
       constexpr int k1 = decltype(k_)::value;
-      C w = __ldg(&tw[k1 * TWS * T + t]);
+      C w = __ldg(&tw[k1 * T + t]);
       v[k1] = DIR < 0 ? cmul(v[k1], w) : cmulc(v[k1], w);
     });
     __syncwarp();
@@ -274,7 +272,7 @@ struct GroupFFT {
   }
 };
 
-// group shape for a transform of length n (a power of two from 64 to 2048, or 1536, 2560)
+// group shape for an image side n
 template <int n>
 struct FFTShape;
 template <> struct FFTShape<64> { using type = GroupFFT<8, 8>; };
@@ -282,14 +280,14 @@ template <> struct FFTShape<128> { using type = GroupFFT<8, 16>; };
 template <> struct FFTShape<256> { using type = GroupFFT<16, 16>; };
 template <> struct FFTShape<512> { using type = GroupFFT<16, 32>; };
 template <> struct FFTShape<1024> { using type = GroupFFT<32, 32>; };
-template <> struct FFTShape<2048> { using type = GroupFFT<32, 64>; };
-// Sides with a factor 3 or 5 use the block FFT (block_fft.cuh); the shape only fixes the rows
-// per block of the row passes and of the stencil (32 threads per row).
-template <int T_, int P_>
-struct RowShape {
-  static constexpr int T = T_, P = P_, SMEM = T * (P + 1);
-};
-template <> struct FFTShape<1536> { using type = RowShape<32, 48>; };
-template <> struct FFTShape<2560> { using type = RowShape<32, 80>; };
+// The sides above 1024 are split into 512-point transforms: as one transform a thread would hold 64
+// values and spill, or the length has a factor 3 or 5 (the shape is that of their twiddle table).
+template <> struct FFTShape<1536> { using type = GroupFFT<16, 32>; };
+template <> struct FFTShape<2048> { using type = GroupFFT<16, 32>; };
+template <> struct FFTShape<2560> { using type = GroupFFT<16, 32>; };
+template <int n>
+constexpr bool is_split_side() {
+  return n > 1024;
+}
 
 }  // namespace tmbir

@@ -89,8 +89,8 @@ struct GroupDev {
   size_t sino_off;     // first element of the group in the stacked sinogram
   float span;
   // Toeplitz operator
-  float* chat;         // [N+1][2][N] real spectrum, even/odd rows of the 2N grid, scaled by 1/(2N)^2
-  float2* twN;         // [P][T] exp(-2 pi i t k / N) for the row/column group FFT
+  float* chat;         // [N+1][C][2N/C] real spectrum, rows u = C k + j of the 2N grid as [j][k], C = chat_split(N), / (2N)^2
+  float2* twN;         // [P][T] exp(-2 pi i t k / TP) of the group FFT; sides above 1024: then exp(-2 pi i 2^l m / 2N), m < 512, at 512 l
   float2* twM;         // [N] exp(-2 pi i n / 2N)
   float2* spec;        // [S][N+1][N] intermediate spectra
   // setup
@@ -115,7 +115,6 @@ struct GroupDev {
   // neighbours only (the halo of a slab of a larger volume)
   int zlo, zn;
   int sc;              // slices per spectrum chunk of passes 1, 2, 3a (0: the default rule)
-  int rb1, rb3;        // rows per block of passes 1 and 3a where a side has variants (0: default)
 };
 
 // Up to kMergeMax consecutive groups of one image side that one launch of a pass covers: block
@@ -265,9 +264,9 @@ int launch_pass2(const GroupDev& g, const IterState* st, cudaStream_t s, bool bf
 int launch_pass3(const GroupDev& g, const StepArgs& a, Pass3Mode mode, const PriorC& pc, double* partials,
                  int block_offset, cudaStream_t s, bool bf16 = false, int part = 3);
 // The passes of n consecutive groups (n <= kMergeMax) of one image side in one launch each, in
-// Iterate mode (a.gm is the first group's momentum state).  The groups must share the rows per
-// block of passes 1 and 3a and hold their spectra in one chunk (launch_set_ok); pass 3b's blocks
-// write the partial-sum rows the groups' separate launches would.
+// Iterate mode (a.gm is the first group's momentum state).  The groups must hold their spectra in
+// one chunk (launch_set_ok); pass 3b's blocks write the partial-sum rows the groups' separate
+// launches would.
 bool launch_set_ok(const GroupDev& first, const GroupDev& g);
 int launch_passes_set(const GroupDev* gs, int n, const StepArgs& a, const PriorC& pc, double* partials,
                       int block_offset, cudaStream_t s, bool bf16);
@@ -319,8 +318,9 @@ int launch_finalize(IterState* st, GroupMom* gm, const double* partials, const G
                     cudaStream_t s, cudaGraphConditionalHandle cond = 0, int use_cond = 0, int trip_launches = 0);
 int launch_sum_partials(const double* partials, int nblocks, double* out, cudaStream_t s);
 bool supported_N(int N);
-bool block_fft_N(int N);  // sides with a factor 3 or 5 (block-FFT passes, plain twiddle table)
-void fft_shape(int N, int* T, int* P);
+// transforms per column of pass 2: the even and odd halves, or the 512-point transforms of the sides above 1024
+inline int chat_split(int N) { return N > 1024 ? 2 * N / 512 : 2; }
+void fft_shape(int N, int* T, int* P);  // shape of the group FFT whose twiddle table a side keeps
 
 // setup.cu ------------------------------------------------------------------
 int setup_tables(Ctx& c);  // enqueue uploads of twiddles / psi tables into the workspace

@@ -585,14 +585,13 @@ __global__ void k_circulant(const double* __restrict__ K, int N, double2* Cg) {
   }
 }
 
-// chat[v][h][k] = Re C_hat[u = 2k + h][v] / M^2, spectrum transposed ([kx = v][ky = u])
-__global__ void k_chat_layout(const double2* __restrict__ B, int N, float* chat) {
-  const int M = 2 * N;
-  const size_t total = (size_t)(N + 1) * 2 * N;
+// chat[v][j][k] = Re C_hat[u = C k + j][v] / M^2, j < C, spectrum transposed ([kx = v][ky = u])
+__global__ void k_chat_layout(const double2* __restrict__ B, int N, int C, float* chat) {
+  const int M = 2 * N, K = M / C;
+  const size_t total = (size_t)(N + 1) * M;
   for (size_t id = blockIdx.x * (size_t)blockDim.x + threadIdx.x; id < total; id += (size_t)gridDim.x * blockDim.x) {
-    const int k = (int)(id % N), h = (int)((id / N) % 2), v = (int)(id / (2 * (size_t)N));
-    const int u = 2 * k + h;
-    chat[id] = (float)(B[(size_t)v * M + u].x / ((double)M * (double)M));
+    const int k = (int)(id % K), j = (int)((id / K) % C), v = (int)(id / M);
+    chat[id] = (float)(B[(size_t)v * M + C * k + j].x / ((double)M * (double)M));
   }
 }
 
@@ -865,7 +864,7 @@ static int circulant_spectrum(Ctx& c, int gi) {
   k_circulant<<<1024, 256, 0, s>>>(g.K, N, cg);
   TMBIR_CHECK_LAUNCH();
   if (int e = fft2_transposed(cg, ct, M, 1, -1, tw, s)) return e;
-  k_chat_layout<<<1024, 256, 0, s>>>(ct, N, g.chat);
+  k_chat_layout<<<1024, 256, 0, s>>>(ct, N, chat_split(N), g.chat);
   TMBIR_CHECK_LAUNCH();
   return TMBIR_OK;
 }

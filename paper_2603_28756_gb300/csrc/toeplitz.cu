@@ -9,7 +9,6 @@ namespace tmbir {
 bool supported_N(int N) {
   return N == 64 || N == 128 || N == 256 || N == 512 || N == 1024 || N == 2048 || N == 1536 || N == 2560;
 }
-bool block_fft_N(int N) { return N == 1536 || N == 2560; }
 
 void fft_shape(int N, int* T, int* P) {
   switch (N) {
@@ -18,8 +17,7 @@ void fft_shape(int N, int* T, int* P) {
     case 256: *T = 16; *P = 16; break;
     case 512: *T = 16; *P = 32; break;
     case 1024: *T = 32; *P = 32; break;
-    case 2048: *T = 32; *P = 64; break;
-    default: *T = 32; *P = N / 32; break;  // 1536, 2560: rows of the block-FFT passes
+    default: *T = 16; *P = 32; break;  // 1536, 2048, 2560: their 512-point transforms
   }
 }
 
@@ -191,8 +189,7 @@ int launch_pass3(const GroupDev& g, const StepArgs& a, Pass3Mode m, const PriorC
   TMBIR_DISPATCH_N(g.N, pass3_, &g, 1, a, m, pc, partials, off, bf16, part, s);
 }
 bool launch_set_ok(const GroupDev& first, const GroupDev& g) {
-  return g.N == first.N && g.rb1 == first.rb1 && g.rb3 == first.rb3 && spec_chunk(g) == g.S &&
-         spec_chunk(first) == first.S;
+  return g.N == first.N && spec_chunk(g) == g.S && spec_chunk(first) == first.S;
 }
 static int pass1_set(const GroupDev* gs, int n, const StepArgs& a, cudaStream_t s, bool bf16) {
   TMBIR_DISPATCH_N(gs[0].N, pass1_, gs, n, a, bf16, s);

@@ -23,7 +23,6 @@
 #pragma once
 #include <cuda_bf16.h>
 
-#include "block_fft.cuh"
 #include "fft.cuh"
 #include "internal.h"
 #include "tc05.cuh"
@@ -373,23 +372,76 @@ __global__ void TMBIR_P3A_BOUNDS(Geo3a<N>::THREADS) k_pass3a(const __grid_consta
   });
 }
 
-// ---------------------------------------------------------------- passes 1, 2, 3a for 1536 and 2560
-// The same three passes with block-wide FFTs (block_fft.cuh) instead of group FFTs: a block of
-// 256 threads transforms one row or column at a time.  Layouts, scaling and the packed-real
-// split are those of the group-FFT passes.
-template <int N>
-struct BGeo {
-  static constexpr int THREADS = 256;
-  static constexpr int RB = Geo<N>::RB;             // rows per block, as the stencil expects
+// ---------------------------------------------------------------- passes 1, 2, 3a for 1536, 2048 and 2560
+// N = 512 J (J = 3, 4, 5): every transform is split into transforms of 512 points, one register group
+// FFT (16 threads x 32 values) each, by a J-point DFT and a twiddle in registers before (forward) or
+// after (inverse) it, which is also where the zero padding and the crop are pruned.  Layouts, scaling
+// and the packed-real split are those of the other passes (w = exp(-2 pi i / N), W = exp(-2 pi i / 2N)):
+//   pass 1: the packed row z has N/2 nonzero values,
+//           Z[J k + j] = DFT_512(w^(jm) sum_q z[m + 512 q] exp(-2 pi i j q / J))[k];
+//   pass 2: the column c has N nonzero values of 2N,
+//           X[2J k + j] = DFT_512(W^(jm) sum_q c[m + 512 q] exp(-2 pi i j q / 2J))[k], the even and odd j
+//           as two J-point DFTs; after the kernel multiply the kept rows m + 512 q are
+//           sum_j W^(-jm) exp(2 pi i j q / 2J) u_j[m], u_j the inverse 512-point transforms;
+//   pass 3a: z[m + 512 q] = sum_j w^(-jm) exp(2 pi i j q / J) u_j[m], u_j of Z[J k + j].
+// A shared-memory round trip carries the values between the J-point DFTs (threads along m) and the
+// group FFTs (one per j), and one more is inside each group FFT.
+//
+// Bound by the shared-memory / L1 data pipe (75 % busy in all three), so its wavefronts are what the
+// layouts save: twiddles come from tables that are contiguous in m (W^m, W^2m, W^4m, W^8m; the others
+// are one product of two of these), the kernel spectrum is stored per j, and for J = 4 a staged row
+// keeps the four residues of v apart (stride-4 accesses would meet in four banks).  Measured per
+// launch, pass 1 / 2 / 3a: 6 x 2560^2 177 / 369 / 179 us, 8 x 1536^2 92 / 144 / 96 us (632 / 1215 /
+// 570 and 188 / 448 / 212 us with the four-stage block-wide Stockham transform, five round trips with a
+// block barrier each, that this replaced); 32 x 2048^2 540 / 932 / 582 us (707 / 1026 / 690 us with
+// 1024-point transforms of one warp).
+template <int N, int RBp = 4>
+struct GeoH {
+  static constexpr int H = 512, J = N / H, J2 = 2 * J;
+  using F = GroupFFT<16, 32>;
+  static constexpr int RB = RBp;                          // rows per block of passes 1 and 3a
   static constexpr int NB = N / RB;
-  static constexpr int LD = N + 4;
-  static constexpr size_t SM_ROWS = (size_t)(2 * N + RB * LD) * sizeof(float2);  // X, Y, RB staged rows
-  static constexpr size_t SM_COL = (size_t)4 * N * sizeof(float2);              // X, Y, column, sum
+  static constexpr int UNITS = RB * J;                    // group FFTs per block in passes 1 and 3a
+  static constexpr int THREADS = 16 * UNITS;
+  // staged rows (complex): place of v = J k + j in a row, row stride.  The half-warps of the split
+  // take four rows x four consecutive v, those of the group FFTs 16 consecutive k.
+  static constexpr bool PLANES = J == 4;
+  static constexpr int HP = H + 4;
+  static constexpr int LDZ = PLANES ? J * HP + 1 : N + 4;
+  __device__ __forceinline__ static int place(int v) { return PLANES ? (v % J) * HP + v / J : v; }
+  __device__ __forceinline__ static int place(int k, int j) { return PLANES ? j * HP + k : J * k + j; }
+  static constexpr int THREADS2 = 16 * J2;                // pass 2: one column per block
+  static constexpr size_t SM_ROWS = (size_t)(RB * LDZ > UNITS * F::SMEM ? RB * LDZ : UNITS * F::SMEM) * sizeof(float2);
+  static constexpr size_t SM_COL = (size_t)J2 * F::SMEM * sizeof(float2);
+  static_assert(N % H == 0 && THREADS % 32 == 0 && THREADS2 % 32 == 0, "split");
 };
 
+// Pass 3a gathers eight rows (64-byte segments of the column-major spectrum, half the load
+// wavefronts of four): 582 against 647 us at 32 x 2048^2, 96 against 112 us at 8 x 1536^2, except at
+// 2560, where eight rows leave one block per SM (190 against 179 us); pass 1, whose stores need no
+// registers while they are in flight, keeps four and more blocks per SM (540 against 636 us at 2048).
+template <int N>
+using GeoH3 = GeoH<N, N == 2560 ? 4 : 8>;
+
+// w[j] = W^(2^L j m) for j < J: the powers of two from the side's tables (twM[m] = W^m,
+// twN[512 l + m] = W^(2^l m)), the others as one product of two of them (7 = 4 + 3: two products)
+template <int L, int J>
+__device__ __forceinline__ void tw_powers(const GroupDev& g, int m, float2 (&w)[J]) {
+  SFor<1, J>::run([&](auto j_) {
+    constexpr int j = decltype(j_)::value;
+    constexpr int l = j >= 8 ? 3 : (j >= 4 ? 2 : (j >= 2 ? 1 : 0));
+    if constexpr (j == 1 << l)
+      w[j] = __ldg(L + l == 0 ? &g.twM[m] : &g.twN[512 * (L + l) + m]);
+    else
+      w[j] = cmul(w[1 << l], w[j - (1 << l)]);
+  });
+}
+
 template <int N, bool BF>
-__global__ void __launch_bounds__(256) k_pass1_b(const __grid_constant__ GroupSet gs, StepArgs a) {
-  using BG = BGeo<N>;
+__global__ void __launch_bounds__(GeoH<N>::THREADS) k_pass1_h(const __grid_constant__ GroupSet gs, StepArgs a) {
+  using Q = GeoH<N>;
+  using F = typename Q::F;
+  constexpr int J = Q::J, H = Q::H, RB = Q::RB, LDZ = Q::LDZ, T = F::T, P = F::P;
   extern __shared__ float2 sm[];
   int bid_;
   const int gi_ = gs.pick(bid_);
@@ -408,197 +460,47 @@ __global__ void __launch_bounds__(256) k_pass1_b(const __grid_constant__ GroupSe
     xp = a.xprev;
     beta = a.beta;
   }
-  const int s = bid_ / BG::NB, rb = bid_ % BG::NB;
-  float2* X = sm;
-  float2* Y = sm + N;
-  float2* tb = sm + 2 * N;
-  for (int rr = 0; rr < BG::RB; ++rr) {
-    __syncthreads();  // the previous row's transform has been read
-    const size_t base = g.img_off + ((size_t)s * N + rb * BG::RB + rr) * N;
-    // packed real row z[n] = y[2n] + i y[2n+1] for n < N/2, zero padding above
-    batched_copy<BG::THREADS, 4>(
-        N / 2,
-        [&](int n) {
-          const float2 xv = __ldg(reinterpret_cast<const float2*>(x + base) + n);
-          const float2 pv = __ldg(reinterpret_cast<const float2*>(xp + base) + n);
-          return make_float2(fmaf(beta, xv.x - pv.x, xv.x), fmaf(beta, xv.y - pv.y, xv.y));
-        },
-        [&](int n, float2 v) { X[n] = v; });
-    for (int n = N / 2 + threadIdx.x; n < N; n += BG::THREADS) X[n] = make_float2(0.f, 0.f);
-    const float2* Z = block_fft<N, -1>(X, Y, g.twN);
-    // Y[v] = E[v] + w^v O[v] from Z[v] and Z[N - v]; the Nyquist term Y[N] = Re Z0 - Im Z0
-    for (int v = threadIdx.x; v < N; v += BG::THREADS) {
-      const float2 z = Z[v], zs = Z[(N - v) % N];
-      const float2 e = make_float2(0.5f * (z.x + zs.x), 0.5f * (z.y - zs.y));
-      const float2 o = make_float2(0.5f * (z.y + zs.y), -0.5f * (z.x - zs.x));
-      tb[rr * BG::LD + v] = cadd(e, cmul(__ldg(&g.twM[v]), o));
-    }
-    if (threadIdx.x == 0) tb[rr * BG::LD + N] = make_float2(Z[0].x - Z[0].y, 0.f);
+  const int s = bid_ / Q::NB, rb = bid_ % Q::NB;
+  const size_t base = g.img_off + ((size_t)s * N + rb * RB) * N;
+  // packed rows z[m] = y[2m] + i y[2m+1], m < N/2, through the J-point DFTs into the units' buffers
+#pragma unroll 2
+  for (int e = threadIdx.x; e < RB * H; e += Q::THREADS) {
+    const int rr = e / H, m = e % H;
+    const float2* xr = reinterpret_cast<const float2*>(x + base + (size_t)rr * N);
+    const float2* pr = reinterpret_cast<const float2*>(xp + base + (size_t)rr * N);
+    float2 c[J], w[J];
+    SFor<0, J>::run([&](auto q_) {
+      constexpr int q = decltype(q_)::value;
+      c[q] = make_float2(0.f, 0.f);
+      if constexpr (q * H < N / 2) {
+        if ((q + 1) * H <= N / 2 || m < N / 2 - q * H) {
+          const float2 xv = __ldg(xr + m + q * H), pv = __ldg(pr + m + q * H);
+          c[q] = make_float2(fmaf(beta, xv.x - pv.x, xv.x), fmaf(beta, xv.y - pv.y, xv.y));
+        }
+      }
+    });
+    tw_powers<1>(g, m, w);
+    reg_dft<J, -1, float2>(c);
+    float2* b = sm + rr * J * F::SMEM + m;
+    SFor<0, J>::run([&](auto j_) {
+      constexpr int j = decltype(j_)::value;
+      b[j * F::SMEM] = j ? cmul(c[j], w[j]) : c[j];
+    });
   }
   __syncthreads();
-  using IO = SpecIO<BF>;
-  typename IO::T* out = reinterpret_cast<typename IO::T*>(g.spec) + (size_t)s * (N + 1) * N + rb * BG::RB;
-  for (int e = threadIdx.x; e < (N + 1) * BG::RB; e += BG::THREADS) {
-    const int vv = e / BG::RB, rr = e - vv * BG::RB;
-    IO::st(out, (size_t)vv * N + rr, tb[rr * BG::LD + vv]);
-  }
-}
-
-template <int N, bool BF>
-__global__ void __launch_bounds__(256) k_pass2_b(const __grid_constant__ GroupSet gs, const IterState* st) {
-  using BG = BGeo<N>;
-  extern __shared__ float2 sm[];
-  int bid_;
-  const int gi_ = gs.pick(bid_);
-  const GroupDev& g = gs.g[gi_];
-  if (st && skip_iter<BF>(st)) return;
-  int vcol, s;
-  column_of(bid_, g.S, N + 1, vcol, s);
-  using IO = SpecIO<BF>;
-  typename IO::T* p = reinterpret_cast<typename IO::T*>(g.spec) + ((size_t)s * (N + 1) + vcol) * N;
-  float2* X = sm;
-  float2* Y = sm + N;
-  float2* col = sm + 2 * N;
-  float2* sum = sm + 3 * N;
-  batched_copy<BG::THREADS, 8>(N, [&](int r) { return IO::ld(p, r); }, [&](int r, float2 v) { col[r] = v; });
-  for (int h = 0; h < 2; ++h) {
-    __syncthreads();
-    // even half: the column; odd half: the column times exp(-2 pi i r / 2N)
-    for (int r = threadIdx.x; r < N; r += BG::THREADS) X[r] = h ? cmul(col[r], __ldg(&g.twM[r])) : col[r];
-    float2* F = block_fft<N, -1>(X, Y, g.twN);
-    const float* cc = g.chat + ((size_t)vcol * 2 + h) * N;
-    for (int k = threadIdx.x; k < N; k += BG::THREADS) {
-      const float c = __ldg(&cc[k]);
-      F[k] = make_float2(F[k].x * c, F[k].y * c);
-    }
-    float2* G = block_fft<N, 1>(F, F == X ? Y : X, g.twN);
-    for (int r = threadIdx.x; r < N; r += BG::THREADS) {
-      const float2 v = h ? cmulc(G[r], __ldg(&g.twM[r])) : G[r];
-      sum[r] = h ? cadd(sum[r], v) : v;
-    }
-  }
-  __syncthreads();
-  for (int r = threadIdx.x; r < N; r += BG::THREADS) IO::st(p, r, sum[r]);
-}
-
-template <int N, bool BF>
-__global__ void __launch_bounds__(256) k_pass3a_b(const __grid_constant__ GroupSet gs, const IterState* st, float* apply_out) {
-  using BG = BGeo<N>;
-  extern __shared__ float2 sm[];
-  int bid_;
-  const int gi_ = gs.pick(bid_);
-  const GroupDev& g = gs.g[gi_];
-  float* kz = apply_out ? apply_out + g.img_off : g.kz;
-  if (st && skip_iter<BF>(st)) return;
-  const int s = bid_ / BG::NB, rb = bid_ % BG::NB;
-  const int r0 = rb * BG::RB;
-  float2* X = sm;
-  float2* Y = sm + N;
-  float2* tb = sm + 2 * N;
-  {
-    using IO = SpecIO<BF>;
-    const typename IO::T* sp = reinterpret_cast<const typename IO::T*>(g.spec) + (size_t)s * (N + 1) * N + r0;
-    batched_copy<BG::THREADS, 8>(
-        (N + 1) * BG::RB, [&](int e) { return IO::ld(sp, (size_t)(e / BG::RB) * N + e % BG::RB); },
-        [&](int e, float2 v) { tb[(e % BG::RB) * BG::LD + e / BG::RB] = v; });
-  }
-  for (int rr = 0; rr < BG::RB; ++rr) {
-    __syncthreads();
-    // the length-2N real inverse as a length-N complex inverse of Z[v] = E[v] + i O[v]
-    for (int vp = threadIdx.x; vp < N; vp += BG::THREADS) {
-      const float2 zv = tb[rr * BG::LD + vp];
-      const float2 zr = tb[rr * BG::LD + N - vp];
-      const float2 e = make_float2(zv.x + zr.x, zv.y - zr.y);
-      const float2 d = make_float2(zv.x - zr.x, zv.y + zr.y);
-      const float2 o = cmulc(d, __ldg(&g.twM[vp]));
-      X[vp] = make_float2(e.x - o.y, e.y + o.x);
-    }
-    const float2* Z = block_fft<N, 1>(X, Y, g.twN);
-    float2* out = reinterpret_cast<float2*>(kz + ((size_t)s * N + r0 + rr) * N);
-    for (int n = threadIdx.x; n < N / 2; n += BG::THREADS) out[n] = Z[n];
-  }
-}
-
-// ---------------------------------------------------------------- passes 1, 2, 3a for N = 2048
-// At N = 2048 a thread of the register group FFT would hold 64 complex values (254 registers,
-// spills in pass 2).  The zero padding lets each transform split into transforms of half the
-// length, so these passes run the 1024-point group FFT of N = 1024 (32 threads x 32 values),
-// one warp per part, with the same layouts and scaling as the group-FFT passes
-// (w = exp(-2 pi i / 2048), W = exp(-2 pi i / 4096)):
-//   pass 1: the packed row z has 1024 nonzero values of 2048, so
-//           Z[2k + j] = DFT_1024(z[m] w^(jm))[k], j = 0, 1 (two warps per row);
-//   pass 2: the column c has 2048 nonzero values of 4096, so
-//           X[4k + j] = DFT_1024(W^(jm) (c[m] + (-i)^j c[m + 1024]))[k], j = 0..3 (four warps
-//           per column); after the kernel multiply the kept rows n = m + 1024 q are
-//           sum_j W^(-jm) i^(jq) u_j[m], u_j the inverse 1024-point transforms;
-//   pass 3a: only the first 1024 packed outputs are kept, z[n] = sum_j w^(-jn) u_j[n], u_j the
-//           inverse 1024-point transforms of Z[2k + j], j = 0, 1 (two warps per row).
-// Each has the flops of the unsplit transforms (the split is the first radix-2 or radix-4
-// stage, pruned by the padding and the crop).
-struct Q2048 {
-  static constexpr int N = 2048, H = 1024;
-  using F = GroupFFT<32, 32>;
-  static constexpr int LDZ = N + 4;  // row stride (complex) of staged rows
-  // rows per block of passes 1 and 3a (two warps per row): 4 or 8, chosen per group by the
-  // autotuner (GroupDev::rb1, rb3); eight rows write and gather 64-byte segments of the
-  // column-major spectrum but hold one 135 KB block per SM, four rows 32-byte segments with two
-  // or three blocks per SM whose phases overlap
-  static constexpr int RB1 = 4;      // default of pass 1
-  static constexpr int RB3 = 8;      // default of pass 3a
-  template <int RB>
-  static constexpr size_t sm_rows() {  // staged rows and the warps' exchange buffers, aliased
-    return (size_t)(RB * LDZ > 2 * RB * F::SMEM ? RB * LDZ : 2 * RB * F::SMEM) * sizeof(float2);
-  }
-  static constexpr size_t SM2 = (size_t)(N + 4 * F::SMEM) * sizeof(float2);  // column + 4 exchange buffers
-};
-
-// W^n = exp(-2 pi i n / 4096) for 0 <= n < 4096 from the table of n < 2048 (W^(n + 2048) = -W^n)
-__device__ __forceinline__ float2 tw4096(const float2* __restrict__ twM, int n) {
-  const float2 w = __ldg(&twM[n & 2047]);
-  return n < 2048 ? w : make_float2(-w.x, -w.y);
-}
-
-template <bool BF, int RB>
-__global__ void __launch_bounds__(64 * RB) k_pass1_q(const __grid_constant__ GroupSet gs, StepArgs a) {
-  using Q = Q2048;
-  constexpr int N = Q::N, T = 32, P = 32, LDZ = Q::LDZ, THREADS = 64 * RB, NB = N / RB;
-  extern __shared__ float2 sm[];
-  int bid_;
-  const int gi_ = gs.pick(bid_);
-  const GroupDev& g = gs.g[gi_];
-  const float *x, *xp;
-  float beta;
-  if (a.st) {
-    if (skip_iter<BF>(a.st)) return;
-    const int cur = a.st->cur;
-    x = cur == 0 ? a.xb[0] : (cur == 1 ? a.xb[1] : a.xb[2]);
-    xp = cur == 0 ? a.xb[2] : (cur == 1 ? a.xb[0] : a.xb[1]);
-    beta = (float)(a.gm + gi_)->beta;
-  } else {
-    x = a.x;
-    xp = a.xprev;
-    beta = a.beta;
-  }
-  const int s = bid_ / NB, rb = bid_ % NB;
-  const int warp = threadIdx.x >> 5, t = threadIdx.x & 31, rl = warp >> 1, j = warp & 1;
-  const size_t base = g.img_off + ((size_t)s * N + rb * RB + rl) * N;
-  // packed row z[m] = y[2m] + i y[2m+1], m < 1024 (the padding above is zero), times w^(jm)
+  const int unit = threadIdx.x / T, t = threadIdx.x % T, rl = unit / J, j = unit - rl * J;
+  float2* xs = sm + unit * F::SMEM;
   float2 v[P];
   SFor<0, P>::run([&](auto i_) {
     constexpr int i = decltype(i_)::value;
-    const int m = t + T * i;
-    const float2 xv = __ldg(reinterpret_cast<const float2*>(x + base) + m);
-    const float2 pv = __ldg(reinterpret_cast<const float2*>(xp + base) + m);
-    float2 z = make_float2(fmaf(beta, xv.x - pv.x, xv.x), fmaf(beta, xv.y - pv.y, xv.y));
-    if (j) z = cmul(z, __ldg(&g.twM[2 * m]));  // w^m = W^(2m)
-    v[i] = z;
+    v[i] = xs[t + T * i];
   });
-  Q::F::template run<-1, float2, 2>(v, sm + warp * Q::F::SMEM, g.twN, t);
+  F::template run<-1>(v, xs, g.twN, t);
   __syncthreads();  // every exchange buffer is free: the staged rows alias them
   float2* zrow = sm + rl * LDZ;
   SFor<0, P>::run([&](auto i_) {
     constexpr int i = decltype(i_)::value;
-    zrow[2 * (t + T * i) + j] = v[i];
+    zrow[Q::place(t + T * i, j)] = v[i];
   });
   __syncthreads();
   // split Y[v] = E[v] + W^v O[v] with E = (Z[v] + conj Z[N - v]) / 2, O = (Z[v] - conj Z[N - v]) / 2i,
@@ -607,10 +509,11 @@ __global__ void __launch_bounds__(64 * RB) k_pass1_q(const __grid_constant__ Gro
   // written column-major (RB-row segments)
   using IO = SpecIO<BF>;
   typename IO::T* out = reinterpret_cast<typename IO::T*>(g.spec) + (size_t)s * (N + 1) * N + rb * RB;
-  for (int e = threadIdx.x; e < (N / 2 + 1) * RB; e += THREADS) {
+#pragma unroll 2
+  for (int e = threadIdx.x; e < (N / 2 + 1) * RB; e += Q::THREADS) {
     const int vv = e / RB, rr = e - vv * RB;
     const float2* zr = sm + rr * LDZ;
-    const float2 z = zr[vv], zs = zr[(N - vv) & (N - 1)];
+    const float2 z = zr[Q::place(vv)], zs = zr[Q::place(vv ? N - vv : 0)];
     const float2 ev = make_float2(0.5f * (z.x + zs.x), 0.5f * (z.y - zs.y));
     const float2 od = make_float2(0.5f * (z.y + zs.y), -0.5f * (z.x - zs.x));
     const float2 wo = cmul(__ldg(&g.twM[vv]), od);
@@ -619,158 +522,171 @@ __global__ void __launch_bounds__(64 * RB) k_pass1_q(const __grid_constant__ Gro
   }
 }
 
-template <bool BF>
-__global__ void __launch_bounds__(128, 3) k_pass2_q(const __grid_constant__ GroupSet gs, const IterState* st) {
-  using Q = Q2048;
-  constexpr int N = Q::N, H = Q::H, T = 32, P = 32;
+template <int N, bool BF>
+__global__ void __launch_bounds__(GeoH<N>::THREADS2) k_pass2_h(const __grid_constant__ GroupSet gs, const IterState* st) {
+  using Q = GeoH<N>;
+  using F = typename Q::F;
+  constexpr int J = Q::J, J2 = Q::J2, H = Q::H, T = F::T, P = F::P, NT = Q::THREADS2;
   extern __shared__ float2 sm[];
   int bid_;
   const int gi_ = gs.pick(bid_);
   const GroupDev& g = gs.g[gi_];
   if (st && skip_iter<BF>(st)) return;
-  const int j = threadIdx.x >> 5, t = threadIdx.x & 31;
   int vcol, s;
   column_of(bid_, g.S, N + 1, vcol, s);
   using IO = SpecIO<BF>;
   typename IO::T* p = reinterpret_cast<typename IO::T*>(g.spec) + ((size_t)s * (N + 1) + vcol) * N;
-  float2* col = sm;
-  if constexpr (!BF) {
-    // all of the column's copies in flight at once
-    SFor<0, N / 128>::run([&](auto i_) {
-      constexpr int i = decltype(i_)::value;
-      tc05::cp_async8(&col[threadIdx.x + 128 * i], p + threadIdx.x + 128 * i);
+  // the J values of each m through the two J-point DFTs into the units' buffers
+  constexpr int IT = (H + NT - 1) / NT;
+  float2 c[IT][J];
+  SFor<0, IT>::run([&](auto k_) {
+    constexpr int k = decltype(k_)::value;
+    const int m = threadIdx.x + k * NT;
+    SFor<0, J>::run([&](auto q_) {
+      constexpr int q = decltype(q_)::value;
+      c[k][q] = m < H ? IO::ld(p, m + q * H) : make_float2(0.f, 0.f);
     });
-    tc05::cp_async_wait_all();
-  } else {
-    batched_copy<128, 16>(N, [&](int r) { return IO::ld(p, r); }, [&](int r, float2 v) { col[r] = v; });
-  }
+  });
+  SFor<0, IT>::run([&](auto k_) {
+    constexpr int k = decltype(k_)::value;
+    const int m = threadIdx.x + k * NT;
+    if (m < H) {
+      float2 w[J2], o[J];
+      tw_powers<0>(g, m, w);
+      SFor<0, J>::run([&](auto q_) {
+        constexpr int q = decltype(q_)::value;
+        o[q] = twmul<q, J2, -1>(c[k][q]);
+      });
+      reg_dft<J, -1, float2>(c[k]);
+      reg_dft<J, -1, float2>(o);
+      SFor<0, J>::run([&](auto i_) {
+        constexpr int i = decltype(i_)::value;
+        sm[2 * i * F::SMEM + m] = i ? cmul(c[k][i], w[2 * i]) : c[k][i];
+        sm[(2 * i + 1) * F::SMEM + m] = cmul(o[i], w[2 * i + 1]);
+      });
+    }
+  });
   __syncthreads();
+  const int j = threadIdx.x / T, t = threadIdx.x % T;
+  float2* xs = sm + j * F::SMEM;
   float2 v[P];
-  // y_j[m] = W^(jm) (c[m] + (-i)^j c[m + 1024]) with m = t + 32 i; W^(jm) = W^(jt) W^(32 j i), the
-  // first factor one table read per thread, the second a compile-time constant per element
-  auto prologue = [&](auto J_) {
-    constexpr int J = decltype(J_)::value;
-    const float2 base = tw4096(g.twM, J * t);
-    SFor<0, P>::run([&](auto i_) {
-      constexpr int i = decltype(i_)::value;
-      const int m = t + T * i;
-      const float2 a0 = col[m], b = col[m + H];
-      float2 c;
-      if constexpr (J == 0)
-        c = cadd(a0, b);
-      else if constexpr (J == 1)
-        c = make_float2(a0.x + b.y, a0.y - b.x);  // a + (-i) b
-      else if constexpr (J == 2)
-        c = csub(a0, b);
-      else
-        c = make_float2(a0.x - b.y, a0.y + b.x);  // a + i b
-      if constexpr (J != 0) c = cmul(c, twmul<32 * J * i, 4096, -1>(base));
-      v[i] = c;
-    });
-  };
-  switch (j) {
-    case 0: prologue(std::integral_constant<int, 0>{}); break;
-    case 1: prologue(std::integral_constant<int, 1>{}); break;
-    case 2: prologue(std::integral_constant<int, 2>{}); break;
-    default: prologue(std::integral_constant<int, 3>{}); break;
-  }
-  float2* xs = sm + N + j * Q::F::SMEM;
-  Q::F::template run<-1, float2, 2>(v, xs, g.twN, t);
-  // v[i] = X[4k + j], k = t + 32 i: row 4k + j of the 2N grid is row 2k + (j >> 1) of the
-  // (j & 1) half of the kernel spectrum
-  const float* cc = g.chat + ((size_t)vcol * 2 + (j & 1)) * N + (j >> 1);
   SFor<0, P>::run([&](auto i_) {
     constexpr int i = decltype(i_)::value;
-    const float c = __ldg(&cc[2 * (t + T * i)]);
-    v[i] = make_float2(v[i].x * c, v[i].y * c);
+    v[i] = xs[t + T * i];
   });
-  Q::F::template run<1, float2, 2>(v, xs, g.twN, t);
-  __syncwarp();  // the transform's last exchange reads are done: the buffer takes W^(-jm) u_j
-  auto epilogue = [&](auto J_) {
-    constexpr int J = decltype(J_)::value;
-    const float2 base = tw4096(g.twM, J * t);
-    SFor<0, P>::run([&](auto i_) {
-      constexpr int i = decltype(i_)::value;
-      if constexpr (J == 0)
-        xs[t + T * i] = v[i];
-      else
-        xs[t + T * i] = cmulc(v[i], twmul<32 * J * i, 4096, -1>(base));
-    });
-  };
-  switch (j) {
-    case 0: epilogue(std::integral_constant<int, 0>{}); break;
-    case 1: epilogue(std::integral_constant<int, 1>{}); break;
-    case 2: epilogue(std::integral_constant<int, 2>{}); break;
-    default: epilogue(std::integral_constant<int, 3>{}); break;
-  }
+  F::template run<-1>(v, xs, g.twN, t);
+  // v[i] = X[2J k + j], k = t + 16 i
+  const float* cc = g.chat + (size_t)vcol * 2 * N + j * H;
+  SFor<0, P>::run([&](auto i_) {
+    constexpr int i = decltype(i_)::value;
+    const float f = __ldg(&cc[t + T * i]);
+    v[i] = make_float2(v[i].x * f, v[i].y * f);
+  });
+  F::template run<1>(v, xs, g.twN, t);
+  __syncwarp();  // the transform's last exchange reads are done
+  SFor<0, P>::run([&](auto i_) {
+    constexpr int i = decltype(i_)::value;
+    xs[t + T * i] = v[i];
+  });
   __syncthreads();
-  // kept rows: z[m] = v_0 + v_1 + v_2 + v_3, z[m + 1024] = (v_0 - v_2) + i (v_1 - v_3)
-  const float2* b0 = sm + N;
-  for (int m = threadIdx.x; m < H; m += 128) {
-    const float2 a0 = b0[m], a1 = b0[Q::F::SMEM + m], a2 = b0[2 * Q::F::SMEM + m], a3 = b0[3 * Q::F::SMEM + m];
-    const float2 s02 = cadd(a0, a2), d02 = csub(a0, a2), s13 = cadd(a1, a3), d13 = csub(a1, a3);
-    IO::st(p, m, cadd(s02, s13));
-    IO::st(p, m + H, make_float2(d02.x - d13.y, d02.y + d13.x));
+  for (int m = threadIdx.x; m < H; m += NT) {
+    float2 w[J2], e[J], o[J];
+    tw_powers<0>(g, m, w);
+    SFor<0, J>::run([&](auto i_) {
+      constexpr int i = decltype(i_)::value;
+      e[i] = sm[2 * i * F::SMEM + m];
+      if constexpr (i > 0) e[i] = cmulc(e[i], w[2 * i]);
+      o[i] = cmulc(sm[(2 * i + 1) * F::SMEM + m], w[2 * i + 1]);
+    });
+    reg_dft<J, 1, float2>(e);
+    reg_dft<J, 1, float2>(o);
+    SFor<0, J>::run([&](auto q_) {
+      constexpr int q = decltype(q_)::value;
+      IO::st(p, m + q * H, cadd(e[q], twmul<q, J2, 1>(o[q])));
+    });
   }
 }
 
-template <bool BF, int RB>
-__global__ void __launch_bounds__(64 * RB, 8 / RB) k_pass3a_q(const __grid_constant__ GroupSet gs, const IterState* st, float* apply_out) {
-  using Q = Q2048;
-  constexpr int N = Q::N, T = 32, P = 32, LDZ = Q::LDZ, THREADS = 64 * RB, NB = N / RB;
+template <int N, bool BF>
+__global__ void __launch_bounds__(GeoH3<N>::THREADS) k_pass3a_h(const __grid_constant__ GroupSet gs, const IterState* st, float* apply_out) {
+  using Q = GeoH3<N>;
+  using F = typename Q::F;
+  constexpr int J = Q::J, H = Q::H, RB = Q::RB, LDZ = Q::LDZ, T = F::T, P = F::P;
   extern __shared__ float2 sm[];
   int bid_;
   const int gi_ = gs.pick(bid_);
   const GroupDev& g = gs.g[gi_];
   float* kz = apply_out ? apply_out + g.img_off : g.kz;
   if (st && skip_iter<BF>(st)) return;
-  const int s = bid_ / NB, rb = bid_ % NB;
-  const int warp = threadIdx.x >> 5, t = threadIdx.x & 31, rl = warp >> 1, j = warp & 1;
+  const int s = bid_ / Q::NB, rb = bid_ % Q::NB;
   const int r0 = rb * RB;
   {
+    // the length-2N real inverse as a length-N complex inverse of Z[v] = E[v] + i O[v], two mirrored
+    // values at a time: with e, o of v, Z[N - v] = conj(e) + i conj(o)
     using IO = SpecIO<BF>;
     const typename IO::T* sp = reinterpret_cast<const typename IO::T*>(g.spec) + (size_t)s * (N + 1) * N + r0;
-    if constexpr (!BF) {
-      // RB-row segments of the column-major spectrum, all copies in flight at once
-      for (int e = threadIdx.x; e < (N + 1) * RB; e += THREADS) {
-        const int vv = e / RB, rr = e - vv * RB;
-        tc05::cp_async8(&sm[rr * LDZ + vv], sp + (size_t)vv * N + rr);
+    constexpr int B = 4, COUNT = (N / 2 + 1) * RB;
+    for (int e0 = threadIdx.x; e0 < COUNT; e0 += B * Q::THREADS) {
+      float2 zv[B], zr[B], w[B];
+#pragma unroll
+      for (int b = 0; b < B; ++b) {
+        const int e = e0 + b * Q::THREADS, vv = e / RB, rr = e - vv * RB;
+        if (e < COUNT) {
+          zv[b] = IO::ld(sp, (size_t)vv * N + rr);
+          zr[b] = IO::ld(sp, (size_t)(N - vv) * N + rr);
+          w[b] = __ldg(&g.twM[vv]);
+        }
       }
-      tc05::cp_async_wait_all();
-    } else {
-      batched_copy<THREADS, 8>(
-          (N + 1) * RB, [&](int e) { return IO::ld(sp, (size_t)(e / RB) * N + e % RB); },
-          [&](int e, float2 v) { sm[(e % RB) * LDZ + e / RB] = v; });
+#pragma unroll
+      for (int b = 0; b < B; ++b) {
+        const int e = e0 + b * Q::THREADS, vv = e / RB, rr = e - vv * RB;
+        if (e < COUNT) {
+          const float2 ev = make_float2(zv[b].x + zr[b].x, zv[b].y - zr[b].y);
+          const float2 d = make_float2(zv[b].x - zr[b].x, zv[b].y + zr[b].y);
+          const float2 o = cmulc(d, w[b]);
+          sm[rr * LDZ + Q::place(vv)] = make_float2(ev.x - o.y, ev.y + o.x);
+          sm[rr * LDZ + Q::place(N - vv)] = make_float2(ev.x + o.y, o.x - ev.y);  // (Z[N] is not used)
+        }
+      }
     }
   }
   __syncthreads();
-  // the length-2N real inverse as the length-N complex inverse of Z[v] = E[v] + i O[v], at the
-  // v = 2k + j of this warp
-  float2 q[P];
-  const float2* row = sm + rl * LDZ;
+  const int unit = threadIdx.x / T, t = threadIdx.x % T, rl = unit / J, j = unit - rl * J;
+  const float2* zrow = sm + rl * LDZ;
+  float2 v[P];
   SFor<0, P>::run([&](auto i_) {
     constexpr int i = decltype(i_)::value;
-    const int vp = 2 * (t + T * i) + j;
-    const float2 zv = row[vp], zr = row[N - vp];
-    const float2 e = make_float2(zv.x + zr.x, zv.y - zr.y);
-    const float2 d = make_float2(zv.x - zr.x, zv.y + zr.y);
-    const float2 o = cmulc(d, __ldg(&g.twM[vp]));
-    q[i] = make_float2(e.x - o.y, e.y + o.x);
+    v[i] = zrow[Q::place(t + T * i, j)];
   });
   __syncthreads();  // the staged rows are read: the exchange buffers alias them
-  float2* xs = sm + warp * Q::F::SMEM;
-  Q::F::template run<1, float2, 2>(q, xs, g.twN, t);
+  float2* xs = sm + unit * F::SMEM;
+  F::template run<1>(v, xs, g.twN, t);
   __syncwarp();
   SFor<0, P>::run([&](auto i_) {
     constexpr int i = decltype(i_)::value;
-    const int n = t + T * i;
-    xs[n] = j ? cmulc(q[i], __ldg(&g.twM[2 * n])) : q[i];  // w^(-jn) u_j[n]
+    xs[t + T * i] = v[i];
   });
   __syncthreads();
-  // z[n] = sum_j w^(-jn) u_j[n]: each warp of the row sums one half of it
-  const float2* o0 = sm + (2 * rl) * Q::F::SMEM;
-  float2* out = reinterpret_cast<float2*>(kz + ((size_t)s * N + r0 + rl) * N);
-  for (int n = j * (Q::H / 2) + t; n < (j + 1) * (Q::H / 2); n += 32) out[n] = cadd(o0[n], o0[Q::F::SMEM + n]);
+  // the kept N/2 packed outputs
+#pragma unroll 2
+  for (int e = threadIdx.x; e < RB * H; e += Q::THREADS) {
+    const int rr = e / H, m = e % H;
+    float2 c[J], w[J];
+    tw_powers<1>(g, m, w);
+    const float2* b = sm + rr * J * F::SMEM + m;
+    SFor<0, J>::run([&](auto j_) {
+      constexpr int jj = decltype(j_)::value;
+      c[jj] = b[jj * F::SMEM];
+      if constexpr (jj > 0) c[jj] = cmulc(c[jj], w[jj]);
+    });
+    reg_dft<J, 1, float2>(c);
+    float2* out = reinterpret_cast<float2*>(kz + ((size_t)s * N + r0 + rr) * N);
+    SFor<0, J>::run([&](auto q_) {
+      constexpr int q = decltype(q_)::value;
+      if constexpr (q * H < N / 2)
+        if ((q + 1) * H <= N / 2 || m < N / 2 - q * H) out[m + q * H] = c[q];
+    });
+  }
 }
 
 // ---------------------------------------------------------------- pass 3b: gradient and update
@@ -1409,27 +1325,14 @@ static int set_smem_limits() {
   using Gr = Geo3a<N>;
   static bool done = false;
   if (done) return TMBIR_OK;
-  if constexpr (N == 2048) {
-    using Q = Q2048;
-    const int s4 = (int)Q::sm_rows<4>(), s8 = (int)Q::sm_rows<8>();
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass1_q<false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass1_q<true, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass1_q<false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, s8));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass1_q<true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, s8));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass2_q<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Q::SM2));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass2_q<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Q::SM2));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass3a_q<false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass3a_q<true, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, s4));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass3a_q<false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, s8));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass3a_q<true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, s8));
-  } else if constexpr (is_block_fft_size<N>()) {
-    using BG = BGeo<N>;
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass1_b<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BG::SM_ROWS));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass1_b<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BG::SM_ROWS));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass2_b<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BG::SM_COL));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass2_b<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BG::SM_COL));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass3a_b<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BG::SM_ROWS));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_pass3a_b<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BG::SM_ROWS));
+  if constexpr (is_split_side<N>()) {
+    using Q = GeoH<N>;
+    TMBIR_CUDA(cudaFuncSetAttribute(k_pass1_h<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Q::SM_ROWS));
+    TMBIR_CUDA(cudaFuncSetAttribute(k_pass1_h<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Q::SM_ROWS));
+    TMBIR_CUDA(cudaFuncSetAttribute(k_pass2_h<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Q::SM_COL));
+    TMBIR_CUDA(cudaFuncSetAttribute(k_pass2_h<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Q::SM_COL));
+    TMBIR_CUDA(cudaFuncSetAttribute(k_pass3a_h<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GeoH3<N>::SM_ROWS));
+    TMBIR_CUDA(cudaFuncSetAttribute(k_pass3a_h<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GeoH3<N>::SM_ROWS));
   } else {
     TMBIR_CUDA(cudaFuncSetAttribute(k_pass1<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Gm::SM1));
     TMBIR_CUDA(cudaFuncSetAttribute(k_pass1<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Gm::SM1));
@@ -1469,28 +1372,13 @@ template <int N>
 static int pass1_n(const GroupDev* gs, int n, const StepArgs& a, bool bf16, cudaStream_t s) {
   using Gm = Geo<N>;
   if (int e = set_smem_limits<N>()) return e;
-  if constexpr (N == 2048) {
-    using Q = Q2048;
-    if ((gs[0].rb1 ? gs[0].rb1 : Q::RB1) == 8) {
-      const GroupSet set = make_set(gs, n, [](const GroupDev& g) { return g.S * (N / 8); });
-      if (bf16)
-        k_pass1_q<true, 8><<<set.boff[n], 512, Q::sm_rows<8>(), s>>>(set, a);
-      else
-        k_pass1_q<false, 8><<<set.boff[n], 512, Q::sm_rows<8>(), s>>>(set, a);
-    } else {
-      const GroupSet set = make_set(gs, n, [](const GroupDev& g) { return g.S * (N / 4); });
-      if (bf16)
-        k_pass1_q<true, 4><<<set.boff[n], 256, Q::sm_rows<4>(), s>>>(set, a);
-      else
-        k_pass1_q<false, 4><<<set.boff[n], 256, Q::sm_rows<4>(), s>>>(set, a);
-    }
-  } else if constexpr (is_block_fft_size<N>()) {
-    using BG = BGeo<N>;
-    const GroupSet set = make_set(gs, n, [](const GroupDev& g) { return g.S * BG::NB; });
+  if constexpr (is_split_side<N>()) {
+    using Q = GeoH<N>;
+    const GroupSet set = make_set(gs, n, [](const GroupDev& g) { return g.S * Q::NB; });
     if (bf16)
-      k_pass1_b<N, true><<<set.boff[n], BG::THREADS, BG::SM_ROWS, s>>>(set, a);
+      k_pass1_h<N, true><<<set.boff[n], Q::THREADS, Q::SM_ROWS, s>>>(set, a);
     else
-      k_pass1_b<N, false><<<set.boff[n], BG::THREADS, BG::SM_ROWS, s>>>(set, a);
+      k_pass1_h<N, false><<<set.boff[n], Q::THREADS, Q::SM_ROWS, s>>>(set, a);
   } else {
     const GroupSet set = make_set(gs, n, [](const GroupDev& g) { return g.S * Gm::NB; });
     if (bf16)
@@ -1505,19 +1393,13 @@ template <int N>
 static int pass2_n(const GroupDev* gs, int n, const IterState* st, bool bf16, cudaStream_t s) {
   using Gm = Geo<N>;
   if (int e = set_smem_limits<N>()) return e;
-  if constexpr (N == 2048) {
+  if constexpr (is_split_side<N>()) {
+    using Q = GeoH<N>;
     const GroupSet set = make_set(gs, n, [](const GroupDev& g) { return g.S * (N + 1); });
     if (bf16)
-      k_pass2_q<true><<<set.boff[n], 128, Q2048::SM2, s>>>(set, st);
+      k_pass2_h<N, true><<<set.boff[n], Q::THREADS2, Q::SM_COL, s>>>(set, st);
     else
-      k_pass2_q<false><<<set.boff[n], 128, Q2048::SM2, s>>>(set, st);
-  } else if constexpr (is_block_fft_size<N>()) {
-    using BG = BGeo<N>;
-    const GroupSet set = make_set(gs, n, [](const GroupDev& g) { return g.S * (N + 1); });
-    if (bf16)
-      k_pass2_b<N, true><<<set.boff[n], BG::THREADS, BG::SM_COL, s>>>(set, st);
-    else
-      k_pass2_b<N, false><<<set.boff[n], BG::THREADS, BG::SM_COL, s>>>(set, st);
+      k_pass2_h<N, false><<<set.boff[n], Q::THREADS2, Q::SM_COL, s>>>(set, st);
   } else {
     const GroupSet set =
         make_set(gs, n, [](const GroupDev& g) { return (g.S * (N + 1) + Gm::CPB - 1) / Gm::CPB; });
@@ -1575,28 +1457,13 @@ static int pass3_n(const GroupDev* gs, int n, const StepArgs& a, Pass3Mode m, co
   float* apply_out = m == Pass3Mode::Apply ? a.out : nullptr;
   const IterState* st = m == Pass3Mode::Iterate ? a.st : nullptr;
   if (part & 1) {
-    if constexpr (N == 2048) {
-      using Q = Q2048;
-      if ((gs[0].rb3 ? gs[0].rb3 : Q::RB3) == 8) {
-        const GroupSet set = make_set(gs, n, [](const GroupDev& g) { return g.S * (N / 8); });
-        if (bf16)
-          k_pass3a_q<true, 8><<<set.boff[n], 512, Q::sm_rows<8>(), s>>>(set, st, apply_out);
-        else
-          k_pass3a_q<false, 8><<<set.boff[n], 512, Q::sm_rows<8>(), s>>>(set, st, apply_out);
-      } else {
-        const GroupSet set = make_set(gs, n, [](const GroupDev& g) { return g.S * (N / 4); });
-        if (bf16)
-          k_pass3a_q<true, 4><<<set.boff[n], 256, Q::sm_rows<4>(), s>>>(set, st, apply_out);
-        else
-          k_pass3a_q<false, 4><<<set.boff[n], 256, Q::sm_rows<4>(), s>>>(set, st, apply_out);
-      }
-    } else if constexpr (is_block_fft_size<N>()) {
-      using BG = BGeo<N>;
-      const GroupSet set = make_set(gs, n, [](const GroupDev& g) { return g.S * BG::NB; });
+    if constexpr (is_split_side<N>()) {
+      using Q = GeoH3<N>;
+      const GroupSet set = make_set(gs, n, [](const GroupDev& g) { return g.S * Q::NB; });
       if (bf16)
-        k_pass3a_b<N, true><<<set.boff[n], BG::THREADS, BG::SM_ROWS, s>>>(set, st, apply_out);
+        k_pass3a_h<N, true><<<set.boff[n], Q::THREADS, Q::SM_ROWS, s>>>(set, st, apply_out);
       else
-        k_pass3a_b<N, false><<<set.boff[n], BG::THREADS, BG::SM_ROWS, s>>>(set, st, apply_out);
+        k_pass3a_h<N, false><<<set.boff[n], Q::THREADS, Q::SM_ROWS, s>>>(set, st, apply_out);
     } else {
       const GroupSet set = make_set(gs, n, [](const GroupDev& g) { return g.S * Gm::NB; });
       if (bf16)

@@ -82,3 +82,23 @@ def test_many_groups_reduce_like_one(orc):
         torch.cuda.synchronize()
         assert torch.equal(x[off:off + n], x1), k
         off += n
+
+
+# pass 3b: bands of four and of eight rows, one and several column blocks, one slice and several,
+# small and very large differences (the shared reciprocal), p = q (no threshold term)
+@pytest.mark.parametrize("N,S,p,scale", [(64, 3, 1.2, 1.0), (256, 2, 1.0, 1e6), (512, 3, 1.2, 1.0), (512, 1, 2.0, 1.0),
+                                         (1024, 2, 1.0, 1e-3)])
+def test_prior_bands(orc, N, S, p, scale):
+    th = synth.angles(4)
+    ctx = tm.Context([tm.Group(N=N, angles=list(th), n_slices=S)])
+    ctx.build_operator(torch.zeros(S * 4 * N, device="cuda"))
+    x = synth.random_image(np.random.default_rng(N + S), (S, N, N), scale)
+    zero = torch.zeros(S * N * N, device="cuda")
+    prm = dict(p=p, q=2.0, c=0.01, sigma=0.1)
+    # the prior alone: the gradient with it minus the gradient without, lambda so large that the
+    # data term's rounding does not count
+    lam = 1e12
+    G = host(ctx.gradient(dev(x), zero, tm.Params(**prm, lam=lam)), x.shape)
+    G0 = host(ctx.gradient(dev(x), zero, tm.Params(**prm, lam=0.0)), x.shape)
+    ref = orc.prior(x.astype(np.float64), orc.Prior(**prm, lam=lam))[0]
+    assert rel(G - G0, ref) < 1e-5
