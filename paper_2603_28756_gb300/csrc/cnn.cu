@@ -96,7 +96,7 @@ __global__ void k_cnn_pack(const float* __restrict__ master, __nv_bfloat16* wg1,
 // bytes) later.  Each warp moves its 32 pixels of every row out with tcgen05.ld.
 // MASK (data gradient): the result is multiplied by (mask[p][n] > 0).
 template <bool BIAS_RELU, bool MASK>
-__global__ void __launch_bounds__(128) k_conv32(const __nv_bfloat16* __restrict__ in, int B, int H, int W,
+__global__ void __launch_bounds__(128, 3) k_conv32(const __nv_bfloat16* __restrict__ in, int B, int H, int W,
                                                 const __nv_bfloat16* __restrict__ wpk, const float* __restrict__ bias,
                                                 const __nv_bfloat16* __restrict__ mask, __nv_bfloat16* __restrict__ out,
                                                 int* err) {
@@ -131,18 +131,15 @@ __global__ void __launch_bounds__(128) k_conv32(const __nv_bfloat16* __restrict_
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int tx = tile % tiles_x, ty = (tile / tiles_x) % tiles_y, b = tile / (tiles_x * tiles_y);
     const int y0 = ty * kRows, x0 = tx * kTM;
-    // thread t copies staged pixel t (threads 0, 1 also pixels 128, 129) of every staged row
-    for (int px = threadIdx.x; px < kTX; px += blockDim.x) {
-      const int gx = x0 - 1 + px;
+    // four neighbouring threads copy the four chunks of a staged pixel (whole sectors of 64 bytes)
+    for (int i = threadIdx.x; i < kTX * 4; i += blockDim.x) {
+      const int px = i >> 2, j = i & 3, gx = x0 - 1 + px;
       const bool vx = gx >= 0 && gx < W;
 #pragma unroll
       for (int sr = 0; sr < kRows + 2; ++sr) {
         const int gy = y0 + sr - 1;
         const bool v = vx && gy >= 0 && gy < H;
-        const __nv_bfloat16* src = v ? in + (((size_t)b * H + gy) * W + gx) * kC : in;
-        unsigned char* dst = sa + sr * 4 * kChunkB + px * 16;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) tc::cp_async16(dst + j * kChunkB, v ? src + 8 * j : in, v);
+        tc::cp_async16(sa + (sr * 4 + j) * kChunkB + px * 16, v ? in + (((size_t)b * H + gy) * W + gx) * kC + 8 * j : in, v);
       }
     }
     tc::cp_async_wait_all();  // this tile's rows (and, the first time, the weights)
@@ -175,6 +172,9 @@ __global__ void __launch_bounds__(128) k_conv32(const __nv_bfloat16* __restrict_
     }
     tc::fence_after_sync();
     const int gx = x0 + warp * 32 + lane;
+    // the warp's 32 pixels of every row, gathered over the staged rows (the MMAs have read them) and
+    // written out as one bulk copy per row: a thread's 64 bytes of one pixel are half sectors otherwise
+    unsigned char* so = sa + warp * kRows * 2048;
 #pragma unroll 1
     for (int r = 0; r < kRows; ++r) {
       float v[32];
@@ -200,7 +200,7 @@ __global__ void __launch_bounds__(128) k_conv32(const __nv_bfloat16* __restrict_
           }
         }
       }
-      uint4* dst = reinterpret_cast<uint4*>(out + pbase);
+      uint4* dst = reinterpret_cast<uint4*>(so + r * 2048 + lane * 64);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         uint4 o;
@@ -210,10 +210,19 @@ __global__ void __launch_bounds__(128) k_conv32(const __nv_bfloat16* __restrict_
         dst[q] = o;
       }
     }
+    tc::fence_async_shared();
+    __syncwarp();
+    const int npx = min(32, W - (x0 + warp * 32));
+    if (lane < kRows && npx > 0 && y0 + lane < H) {
+      tc::bulk_store(out + (((size_t)b * H + y0 + lane) * W + x0 + warp * 32) * kC, so + lane * 2048, npx * 64);
+      tc::bulk_commit();
+      tc::bulk_wait_read();
+    }
     // TMEM and the staged rows are reused by the next tile
     tc::fence_before_sync();
     __syncthreads();
   }
+  tc::bulk_wait_all();
   if (failed) {
     // give the outstanding MMAs a second bounded chance to finish before freeing their TMEM
     tc::mbar_wait(&bar, parity ^ 1u, kMmaPolls);
@@ -233,12 +242,13 @@ __global__ void __launch_bounds__(256) k_conv_first(const float* __restrict__ x,
                                                     const float* __restrict__ master, __nv_bfloat16* __restrict__ a0) {
   __shared__ float xt[kFH + 2][kFW + 2];
   const int cg = threadIdx.x & 7, ps = threadIdx.x >> 3;
-  float wr[4][9], br[4];
+  float2 wr[2][9], br[2];  // channel pairs
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
+  for (int c = 0; c < 2; ++c) {
+    const float* w = master + kOff0 + (4 * cg + 2 * c) * 9;
 #pragma unroll
-    for (int t = 0; t < 9; ++t) wr[c][t] = master[kOff0 + (4 * cg + c) * 9 + t];
-    br[c] = master[kOff0 + kW0 + 4 * cg + c];
+    for (int t = 0; t < 9; ++t) wr[c][t] = make_float2(w[t], w[9 + t]);
+    br[c] = make_float2(master[kOff0 + kW0 + 4 * cg + 2 * c], master[kOff0 + kW0 + 4 * cg + 2 * c + 1]);
   }
   const int tiles_x = (W + kFW - 1) / kFW, tiles_y = (H + kFH - 1) / kFH;
   const int tpi = tiles_x * tiles_y;
@@ -252,122 +262,172 @@ __global__ void __launch_bounds__(256) k_conv_first(const float* __restrict__ x,
           (gy >= 0 && gy < H && gx >= 0 && gx < W) ? x[((size_t)b * H + gy) * W + gx] : 0.f;
     }
     __syncthreads();
-#pragma unroll 2
+    // the 3 x 3 window slides down the rows: three shared loads per pixel
+    float2 nb[9];
+#pragma unroll
+    for (int t = 0; t < 6; ++t) nb[t + 3] = make_float2(xt[t / 3][ps + t % 3], xt[t / 3][ps + t % 3]);
+#pragma unroll
     for (int ly = 0; ly < kFH; ++ly) {
+#pragma unroll
+      for (int t = 0; t < 6; ++t) nb[t] = nb[t + 3];
+#pragma unroll
+      for (int t = 0; t < 3; ++t) nb[6 + t] = make_float2(xt[ly + 2][ps + t], xt[ly + 2][ps + t]);
       const int gy = y0 + ly, gx = x0 + ps;
       if (gy >= H || gx >= W) continue;
-      float nb[9];
+      float2 v[2];
 #pragma unroll
-      for (int t = 0; t < 9; ++t) nb[t] = xt[ly + t / 3][ps + t % 3];
-      float v[4];
+      for (int c = 0; c < 2; ++c) {
+        float2 acc = br[c];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        float acc = br[c];
-#pragma unroll
-        for (int t = 0; t < 9; ++t) acc = fmaf(wr[c][t], nb[t], acc);
-        v[c] = fmaxf(acc, 0.f);
+        for (int t = 0; t < 9; ++t) acc = __ffma2_rn(wr[c][t], nb[t], acc);
+        v[c] = make_float2(fmaxf(acc.x, 0.f), fmaxf(acc.y, 0.f));
       }
       uint2 o;
-      reinterpret_cast<__nv_bfloat162*>(&o)[0] = __floats2bfloat162_rn(v[0], v[1]);
-      reinterpret_cast<__nv_bfloat162*>(&o)[1] = __floats2bfloat162_rn(v[2], v[3]);
+      reinterpret_cast<__nv_bfloat162*>(&o)[0] = __floats2bfloat162_rn(v[0].x, v[0].y);
+      reinterpret_cast<__nv_bfloat162*>(&o)[1] = __floats2bfloat162_rn(v[1].x, v[1].y);
       *reinterpret_cast<uint2*>(a0 + (((size_t)b * H + gy) * W + gx) * kC + 4 * cg) = o;
     }
   }
 }
 
 // out[p] = b3 + sum_{tap, ci} w3[ci][tap] a2[p + tap][ci], as out[p] = b3 + sum_tap T[p + tap][tap]
-// with T[q][tap] = sum_ci w3[ci][tap] a2[q][ci]: a block computes T once per pixel of its 8 x 32
+// with T[q][tap] = sum_ci w3[ci][tap] a2[q][ci]: a block computes T once per pixel of its 16 x 32
 // tile plus a one-pixel halo (each activation vector read once) and sums the nine shifted
-// entries from shared memory.
+// entries from shared memory.  Four lanes share a pixel, eight channels each (one 16-byte load, whole
+// lines per warp) with their 72 weights in registers as channel pairs; their nine partial sums are
+// added by exchanging halves, so that a lane ends with two or three of the nine.  Bound by FP32 issue
+// and by the activation stream (64 B per pixel).
 // DGRAD: the data gradient of layer 0, gin[p] = sum_{tap, co} w0[co][tap] g0[p - tap][co]: the same
 // sums with layer 0's weights, the taps flipped and no bias.
-constexpr int kLH = 8, kLW = 32;
+constexpr int kLH = 16, kLW = 32;
 template <bool DGRAD>
 __global__ void __launch_bounds__(256, 2) k_conv_last(const __nv_bfloat16* __restrict__ a2, int B, int H, int W,
                                                       const float* __restrict__ master, float* __restrict__ out) {
-  __shared__ __align__(16) float w[kC][12];  // w3[ci][tap], rows padded to 12 for 16-byte vector reads
-  __shared__ float T[(kLH + 2) * (kLW + 2)][9];
-  for (int i = threadIdx.x; i < kC * 9; i += blockDim.x)
-    w[i / 9][DGRAD ? 8 - i % 9 : i % 9] = master[(DGRAD ? kOff0 : kOff3) + i];
+  constexpr int PX = (kLH + 2) * (kLW + 2);
+  __shared__ float T[PX][9];
+  const int q = threadIdx.x & 3;  // channels 8 q .. 8 q + 7
+  const bool b0 = q & 1, b1 = q & 2;
+  float2 w[4][9];
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+      const float* m = master + (DGRAD ? kOff0 : kOff3) + (8 * q + 2 * c) * 9 + (DGRAD ? 8 - t : t);
+      w[c][t] = make_float2(m[0], m[9]);
+    }
   const float b3 = DGRAD ? 0.f : master[kOff3 + kW3];
   const int tiles_x = (W + kLW - 1) / kLW, tiles_y = (H + kLH - 1) / kLH;
   const int tpi = tiles_x * tiles_y;
   for (int tile = blockIdx.x; tile < B * tpi; tile += gridDim.x) {
     const int b = tile / tpi, ty = (tile % tpi) / tiles_x, tx = tile % tiles_x;
     const int y0 = ty * kLH, x0 = tx * kLW;
-    __syncthreads();  // weights loaded; T of the previous tile consumed
-    for (int q = threadIdx.x; q < (kLH + 2) * (kLW + 2); q += blockDim.x) {
-      const int gy = y0 - 1 + q / (kLW + 2), gx = x0 - 1 + q % (kLW + 2);
+    __syncthreads();  // T of the previous tile consumed
+#pragma unroll 2
+    for (int i = threadIdx.x >> 2; i < (PX + 7) / 8 * 8; i += 64) {
+      const int gy = y0 - 1 + i / (kLW + 2), gx = x0 - 1 + i % (kLW + 2);
+      uint4 u = make_uint4(0, 0, 0, 0);
+      if (i < PX && gy >= 0 && gy < H && gx >= 0 && gx < W)
+        u = __ldg(reinterpret_cast<const uint4*>(a2 + (((size_t)b * H + gy) * W + gx) * kC) + q);
+      const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
+      float2 s[9];
+#pragma unroll
+      for (int t = 0; t < 9; ++t) s[t] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float2 a = __bfloat1622float2(h[c]);
+#pragma unroll
+        for (int t = 0; t < 9; ++t) s[t] = __ffma2_rn(w[c][t], a, s[t]);
+      }
       float t[9];
 #pragma unroll
-      for (int k = 0; k < 9; ++k) t[k] = 0.f;
-      if (gy >= 0 && gy < H && gx >= 0 && gx < W) {
-        const uint4* src = reinterpret_cast<const uint4*>(a2 + (((size_t)b * H + gy) * W + gx) * kC);
-#pragma unroll 1
-        for (int v4 = 0; v4 < 4; ++v4) {
-          const uint4 u = src[v4];
-          const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&u);
+      for (int k = 0; k < 9; ++k) t[k] = s[k].x + s[k].y;
+      // lanes differing in bit 0 share taps 0-3 / 4-7, then in bit 1 the pairs; tap 8 by all
 #pragma unroll
-          for (int h = 0; h < 8; ++h) {
-            const float a = h & 1 ? __high2float(h2[h / 2]) : __low2float(h2[h / 2]);
-            const float* wr = w[8 * v4 + h];
-            const float4 w0 = *reinterpret_cast<const float4*>(wr);
-            const float4 w1 = *reinterpret_cast<const float4*>(wr + 4);
-            t[0] = fmaf(w0.x, a, t[0]);
-            t[1] = fmaf(w0.y, a, t[1]);
-            t[2] = fmaf(w0.z, a, t[2]);
-            t[3] = fmaf(w0.w, a, t[3]);
-            t[4] = fmaf(w1.x, a, t[4]);
-            t[5] = fmaf(w1.y, a, t[5]);
-            t[6] = fmaf(w1.z, a, t[6]);
-            t[7] = fmaf(w1.w, a, t[7]);
-            t[8] = fmaf(wr[8], a, t[8]);
-          }
-        }
+      for (int k = 0; k < 4; ++k) {
+        const float give = b0 ? t[k] : t[k + 4];
+        t[k] = (b0 ? t[k + 4] : t[k]) + __shfl_xor_sync(0xffffffffu, give, 1);
       }
 #pragma unroll
-      for (int k = 0; k < 9; ++k) T[q][k] = t[k];
+      for (int k = 0; k < 2; ++k) {
+        const float give = b1 ? t[k] : t[k + 2];
+        t[k] = (b1 ? t[k + 2] : t[k]) + __shfl_xor_sync(0xffffffffu, give, 2);
+      }
+      t[8] += __shfl_xor_sync(0xffffffffu, t[8], 1);
+      t[8] += __shfl_xor_sync(0xffffffffu, t[8], 2);
+      if (i < PX) {
+        float* d = T[i] + (b0 ? 4 : 0) + (b1 ? 2 : 0);
+        d[0] = t[0];
+        d[1] = t[1];
+        if (q == 0) T[i][8] = t[8];
+      }
     }
     __syncthreads();
-    const int ly = threadIdx.x / kLW, lx = threadIdx.x % kLW;
-    const int gy = y0 + ly, gx = x0 + lx;
-    if (gy < H && gx < W) {
-      float s = b3;
 #pragma unroll
-      for (int k = 0; k < 9; ++k) s += T[(ly + k / 3) * (kLW + 2) + lx + k % 3][k];
-      out[((size_t)b * H + gy) * W + gx] = s;
+    for (int r = 0; r < kLH / 8; ++r) {
+      const int ly = threadIdx.x / kLW + 8 * r, lx = threadIdx.x % kLW;
+      const int gy = y0 + ly, gx = x0 + lx;
+      if (gy < H && gx < W) {
+        float s = b3;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) s += T[(ly + k / 3) * (kLW + 2) + lx + k % 3][k];
+        out[((size_t)b * H + gy) * W + gx] = s;
+      }
     }
   }
 }
 
-// g2[p][ci] = (a2[p][ci] > 0) * sum_tap w3[ci][tap] gout[p - tap]
-__global__ void k_last_dgrad(const float* __restrict__ gout, const __nv_bfloat16* __restrict__ a2, int B, int H, int W,
-                             const float* __restrict__ master, __nv_bfloat16* __restrict__ g2) {
-  __shared__ float w[kW3];
-  for (int i = threadIdx.x; i < kW3; i += blockDim.x) w[i] = master[kOff3 + i];
-  __syncthreads();
-  const size_t total = (size_t)B * H * W;
-  for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < total; p += (size_t)gridDim.x * blockDim.x) {
-    const int xx = (int)(p % W), yy = (int)((p / W) % H);
-    const size_t b = p / ((size_t)H * W);
-    float gg[9];
+// g2[p][ci] = (a2[p][ci] > 0) * sum_tap w3[ci][tap] gout[p - tap].  A block stages a 16 x 32 tile of
+// gout with a one-pixel halo; four lanes share a pixel, eight channels each with their weights in
+// registers, so the mask is read and the result written in whole lines.
+__global__ void __launch_bounds__(256, 2) k_last_dgrad(const float* __restrict__ gout, const __nv_bfloat16* __restrict__ a2,
+                                                       int B, int H, int W, const float* __restrict__ master,
+                                                       __nv_bfloat16* __restrict__ g2) {
+  __shared__ float gt[kLH + 2][kLW + 2];
+  const int q = threadIdx.x & 3;
+  float2 w[4][9];
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
 #pragma unroll
     for (int t = 0; t < 9; ++t) {
-      const int gy = yy - (t / 3 - 1), gx = xx - (t % 3 - 1);
-      gg[t] = (gy >= 0 && gy < H && gx >= 0 && gx < W) ? gout[(b * H + gy) * W + gx] : 0.f;
+      const float* m = master + kOff3 + (8 * q + 2 * c) * 9 + t;
+      w[c][t] = make_float2(m[0], m[9]);
     }
-    const __nv_bfloat162* a = reinterpret_cast<const __nv_bfloat162*>(a2 + p * kC);
-    __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(g2 + p * kC);
-#pragma unroll 4
-    for (int c = 0; c < kC; c += 2) {
-      float s0 = 0.f, s1 = 0.f;
+  const int tiles_x = (W + kLW - 1) / kLW, tiles_y = (H + kLH - 1) / kLH;
+  const int tpi = tiles_x * tiles_y;
+  for (int tile = blockIdx.x; tile < B * tpi; tile += gridDim.x) {
+    const int b = tile / tpi, ty = (tile % tpi) / tiles_x, tx = tile % tiles_x;
+    const int y0 = ty * kLH, x0 = tx * kLW;
+    __syncthreads();
+    for (int i = threadIdx.x; i < (kLH + 2) * (kLW + 2); i += blockDim.x) {
+      const int gy = y0 - 1 + i / (kLW + 2), gx = x0 - 1 + i % (kLW + 2);
+      gt[i / (kLW + 2)][i % (kLW + 2)] =
+          (gy >= 0 && gy < H && gx >= 0 && gx < W) ? __ldg(gout + ((size_t)b * H + gy) * W + gx) : 0.f;
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int i = threadIdx.x >> 2; i < kLH * kLW; i += 64) {
+      const int ly = i / kLW, lx = i % kLW, gy = y0 + ly, gx = x0 + lx;
+      if (gy >= H || gx >= W) continue;
+      const size_t at = (((size_t)b * H + gy) * W + gx) * kC + 8 * q;
+      const uint4 mk = __ldg(reinterpret_cast<const uint4*>(a2 + at));
+      const __nv_bfloat162* mh = reinterpret_cast<const __nv_bfloat162*>(&mk);
+      float2 s[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) s[c] = make_float2(0.f, 0.f);
 #pragma unroll
       for (int t = 0; t < 9; ++t) {
-        s0 = fmaf(w[c * 9 + t], gg[t], s0);
-        s1 = fmaf(w[(c + 1) * 9 + t], gg[t], s1);
+        const float gv = gt[ly + 2 - t / 3][lx + 2 - t % 3];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) s[c] = __ffma2_rn(w[c][t], make_float2(gv, gv), s[c]);
       }
-      const float2 av = __bfloat1622float2(a[c / 2]);
-      o[c / 2] = __floats2bfloat162_rn(av.x > 0.f ? s0 : 0.f, av.y > 0.f ? s1 : 0.f);
+      uint4 o;
+      __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&o);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float2 a = __bfloat1622float2(mh[c]);
+        oh[c] = __floats2bfloat162_rn(a.x > 0.f ? s[c].x : 0.f, a.y > 0.f ? s[c].y : 0.f);
+      }
+      *reinterpret_cast<uint4*>(g2 + at) = o;
     }
   }
 }
@@ -393,9 +453,9 @@ constexpr int kGRowB = 4 * kTM * 16;               // bytes of one staged row of
 constexpr int kGInB = 6 * kChunkB;                 // one staged input row: four chunks, ones, zeros
 constexpr int kGSmemG = (kGRows + 3) * kGRowB;     // rows y0 - 1 .. y0 + kGRows + 1 (the last stays zero)
 constexpr int kGradSmem = kGSmemG + kGRows * kGInB;
-constexpr int kGCols = 112;                        // D columns: dx 0 | dx 1, ones | dx 2
 
-__global__ void __launch_bounds__(128) k_wgrad32(const __nv_bfloat16* __restrict__ g, const __nv_bfloat16* __restrict__ in,
+
+__global__ void __launch_bounds__(128, 2) k_wgrad32(const __nv_bfloat16* __restrict__ g, const __nv_bfloat16* __restrict__ in,
                                                  int B, int H, int W, float* __restrict__ part, int* err) {
   namespace tc = tc05;
   extern __shared__ __align__(128) unsigned char smraw[];
@@ -436,27 +496,24 @@ __global__ void __launch_bounds__(128) k_wgrad32(const __nv_bfloat16* __restrict
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int tx = tile % tiles_x, ty = (tile / tiles_x) % tiles_y, b = tile / (tiles_x * tiles_y);
     const int y0 = ty * kGRows, x0 = tx * kTM;
-    {
-      const int gx = x0 + threadIdx.x;
+    // four neighbouring threads copy the four chunks of a staged pixel
+    for (int i = threadIdx.x; i < kTX * 4; i += blockDim.x) {
+      const int px = i >> 2, j = i & 3;
+      if (px < kTM) {
+        const int gx = x0 + px;
 #pragma unroll
-      for (int r = 0; r < kGRows + 2; ++r) {
-        const int gy = y0 - 1 + r;
-        const bool v = gx < W && gy >= 0 && gy < H;
-        const __nv_bfloat16* src = v ? g + (((size_t)b * H + gy) * W + gx) * kC : g;
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          tc::cp_async16(sg + r * kGRowB + j * (kTM * 16) + threadIdx.x * 16, v ? src + 8 * j : g, v);
+        for (int r = 0; r < kGRows + 2; ++r) {
+          const int gy = y0 - 1 + r;
+          const bool v = gx < W && gy >= 0 && gy < H;
+          tc::cp_async16(sg + r * kGRowB + j * (kTM * 16) + px * 16, v ? g + (((size_t)b * H + gy) * W + gx) * kC + 8 * j : g, v);
+        }
       }
-    }
-    for (int px = threadIdx.x; px < kTX; px += blockDim.x) {
       const int gx = x0 - 1 + px;
 #pragma unroll
       for (int r = 0; r < kGRows; ++r) {
         const int gy = y0 + r;
         const bool v = gx >= 0 && gx < W && gy < H;
-        const __nv_bfloat16* src = v ? in + (((size_t)b * H + gy) * W + gx) * kC : in;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) tc::cp_async16(si + r * kGInB + j * kChunkB + px * 16, v ? src + 8 * j : in, v);
+        tc::cp_async16(si + r * kGInB + j * kChunkB + px * 16, v ? in + (((size_t)b * H + gy) * W + gx) * kC + 8 * j : in, v);
       }
     }
     tc::cp_async_wait_all();
