@@ -468,50 +468,65 @@ __global__ void k_wt_to_df(double* wt, size_t n) {
   }
 }
 
-// grid[b][cell] = sum_j wt[j] strengths[idx[j]][b], B slices per launch (sample-major strengths)
+// acc += w v in the gather's arithmetic
+__device__ __forceinline__ void gather_add(float w, float v, float& acc) { acc = fmaf(w, v, acc); }
+// Double-word: the compensated dot product of Ogita, Rump and Oishi (2005): the exact rounding errors
+// of the product and of the sum, and the low parts' products, are collected in acc.lo; the pair is
+// renormalised once at the end of a row (gather_end) instead of twice per entry: 12 operations, not 19.
+__device__ __forceinline__ void gather_add(df w, df v, df& acc) {
+  const float p = __fmul_rn(w.hi, v.hi), e = __fmaf_rn(w.hi, v.hi, -p);
+  const df s = two_sum(acc.hi, p);
+  const float l = __fmaf_rn(w.lo, v.hi, __fmaf_rn(w.hi, v.lo, acc.lo));
+  acc = df(s.hi, __fadd_rn(l, __fadd_rn(s.lo, e)));
+}
+__device__ __forceinline__ float gather_end(float acc) { return acc; }
+__device__ __forceinline__ df gather_end(df acc) { return two_sum(acc.hi, acc.lo); }
+
+// grid[b][cell] = sum_j wt[j] strengths[idx[j]][b], B slice pairs per launch (sample-major
+// strengths).  U entries per step with all their loads issued first (the index load and the
+// dependent strength loads are a latency chain); the accumulation order is that of one at a time.
 template <int B, class C>
 __global__ void k_csr_gather(const int* __restrict__ ptr, const int* __restrict__ idx, const double* __restrict__ wt,
                              int ncells, const C* __restrict__ strengths, C* __restrict__ grid, int nb) {
   using S = real_t<C>;
+  constexpr int U = B >= 4 ? 2 : (B == 2 ? 4 : 8);
   for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < ncells; cell += gridDim.x * blockDim.x) {
     C acc[B];
 #pragma unroll
     for (int b = 0; b < B; ++b) acc[b] = mkc((S)0, (S)0);
     const int e = ptr[cell + 1];
     int j = ptr[cell];
-    // two entries per step with all their loads issued first (the index load and the dependent
-    // strength loads are a latency chain); the accumulation order is that of one at a time
-    for (; j + 1 < e; j += 2) {
-      const C* sv0 = strengths + (size_t)idx[j] * B;
-      const C* sv1 = strengths + (size_t)idx[j + 1] * B;
-      const S w0 = load_wt<S>(wt, j), w1 = load_wt<S>(wt, j + 1);
-      C v0[B], v1[B];
+    for (; j + U <= e; j += U) {
+      S w[U];
+      C v[U][B];
 #pragma unroll
-      for (int b = 0; b < B; ++b) {
-        v0[b] = sv0[b];
-        v1[b] = sv1[b];
+      for (int u = 0; u < U; ++u) {
+        const C* sv = strengths + (size_t)idx[j + u] * B;
+        w[u] = load_wt<S>(wt, j + u);
+#pragma unroll
+        for (int b = 0; b < B; ++b) v[u][b] = sv[b];
       }
 #pragma unroll
-      for (int b = 0; b < B; ++b) {
-        acc[b].x = fmar(w0, v0[b].x, acc[b].x);
-        acc[b].y = fmar(w0, v0[b].y, acc[b].y);
-        acc[b].x = fmar(w1, v1[b].x, acc[b].x);
-        acc[b].y = fmar(w1, v1[b].y, acc[b].y);
-      }
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+          gather_add(w[u], v[u][b].x, acc[b].x);
+          gather_add(w[u], v[u][b].y, acc[b].y);
+        }
     }
-    if (j < e) {
+    for (; j < e; ++j) {
       const C* sv = strengths + (size_t)idx[j] * B;
       const S w = load_wt<S>(wt, j);
 #pragma unroll
       for (int b = 0; b < B; ++b) {
         const C v = sv[b];
-        acc[b].x = fmar(w, v.x, acc[b].x);
-        acc[b].y = fmar(w, v.y, acc[b].y);
+        gather_add(w, v.x, acc[b].x);
+        gather_add(w, v.y, acc[b].y);
       }
     }
 #pragma unroll
     for (int b = 0; b < B; ++b)
-      if (b < nb) grid[(size_t)b * ncells + cell] = acc[b];
+      if (b < nb) grid[(size_t)b * ncells + cell] = mkc(gather_end(acc[b].x), gather_end(acc[b].y));
   }
 }
 // tmp[b][j][r] = grid[b][r][(j - N/2) mod nf] for the N kept x-modes j (column pruning)
@@ -534,12 +549,15 @@ __global__ void k_transpose_prune(const C* __restrict__ in, C* __restrict__ out,
 // slice 2p from the real part, slice 2p + 1 (when there is one) from the imaginary part of pair p.
 // tmp is column-major ([c][r']) and out row-major, so 32 x 32 tiles pass through shared memory
 // and both sides are read and written along their contiguous index.  Grid: (N/32, N/32, pairs).
+// The factors 1 / psi are double-words (FP64 divisions, one per row and column of the tile), so that a
+// pixel takes two double-word products on the FP32 pipe instead of conversions and products on the
+// FP64 one, whose rate bound this kernel.
 template <class C>
 __global__ void __launch_bounds__(256) k_deconv_pruned(const C* __restrict__ B, int nf, int N, int nb,
                                                        const double* __restrict__ psi, float scale,
                                                        float* __restrict__ out) {
   __shared__ C tile[32][33];
-  __shared__ double inv_r[32], inv_c[32];  // 1 / psi of the tile's rows and columns
+  __shared__ df inv_r[32], inv_c[32];  // scale / psi of the tile's rows, 1 / psi of its columns
   const int p = blockIdx.z, c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   const C* Bp = B + (size_t)p * N * nf;
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {  // column c0 + i, rows r0 .. r0 + 31
@@ -548,17 +566,17 @@ __global__ void __launch_bounds__(256) k_deconv_pruned(const C* __restrict__ B, 
   }
   if (threadIdx.y == 0) {  // one division per row and column of the tile instead of one per pixel
     const int r = r0 + threadIdx.x, c = c0 + threadIdx.x;
-    inv_r[threadIdx.x] = r < N ? 1.0 / psi[r] : 0.0;
-    inv_c[threadIdx.x] = c < N ? 1.0 / psi[c] : 0.0;
+    inv_r[threadIdx.x] = df(r < N ? scale / psi[r] : 0.0);
+    inv_c[threadIdx.x] = df(c < N ? 1.0 / psi[c] : 0.0);
   }
   __syncthreads();
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {  // row r0 + i, columns c0 .. c0 + 31
     const int r = r0 + i, c = c0 + threadIdx.x;
     if (c >= N || r >= N) continue;
     const C v = tile[threadIdx.x][i];
-    const double f = scale * inv_c[threadIdx.x] * inv_r[i];
-    out[((size_t)(2 * p) * N + r) * N + c] = (float)((double)v.x * f);
-    if (2 * p + 1 < nb) out[((size_t)(2 * p + 1) * N + r) * N + c] = (float)((double)v.y * f);
+    const df f = inv_c[threadIdx.x] * inv_r[i];
+    out[((size_t)(2 * p) * N + r) * N + c] = (df(v.x) * f).hi;
+    if (2 * p + 1 < nb) out[((size_t)(2 * p + 1) * N + r) * N + c] = (df(v.y) * f).hi;
   }
 }
 
@@ -595,31 +613,57 @@ __global__ void k_chat_layout(const double2* __restrict__ B, int N, int C, float
   }
 }
 
-// real sinogram rows -> complex rows for the radial FFT, optional ramp filter (Eq. 12 with the
-// unit-pitch Ram-Lak kernel h[0] = 1/4, h[odd n] = -1/(pi^2 n^2), h[even n != 0] = 0; linear
-// convolution over the detector, FP32 -- only the FBP start uses it)
+// real sinogram rows -> complex rows for the radial FFT
 template <class C>
-__global__ void k_prepare_rows(const float* __restrict__ sino, int nd, size_t rows, int ramp, C* out) {
-  extern __shared__ float srow[];
-  float* htab = srow + nd;
+__global__ void k_prepare_rows(const float* __restrict__ sino, size_t n, C* out) {
   using S = real_t<C>;
-  if (ramp) {
-    for (int n = threadIdx.x; n < nd; n += blockDim.x)
-      htab[n] = (n & 1) ? (float)(-1.0 / (M_PI * M_PI * (double)n * (double)n)) : 0.f;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+    out[i] = mkc((S)sino[i], (S)0);
+}
+// The same through the ramp filter (Eq. 12 with the unit-pitch Ram-Lak kernel h[0] = 1/4, h[odd n] =
+// -1/(pi^2 n^2), h[even n != 0] = 0; linear convolution over the detector, FP32 -- only the FBP start
+// uses it).  An output couples to the inputs of the other parity alone: with m = 2 i + a,
+//   out_1[i] = s_1[i] / 4 + sum_k s_0[k] G[i - k],  out_0[i] = s_0[i] / 4 + sum_k s_1[k] G[i - k - 1],
+// G[d] = h(2 d + 1).  A thread owns eight consecutive i of one parity, so that one input and one
+// new value of G serve eight products (two shared loads per product bound the direct form: 0.8 ms for
+// 1024 rows of 2048 bins).  G is stored with a gap every eight values: threads read it eight apart.
+__global__ void __launch_bounds__(256) k_ramp_rows(const float* __restrict__ sino, int nd, size_t rows, float2* out) {
+  extern __shared__ float rs[];
+  const int half = nd / 2;
+  float* srow = rs;            // [2][half]: the row by parity
+  float* G = rs + nd;          // G[d] at place(d + half)
+  auto place = [](int i) { return i + (i >> 3); };
+  for (int i = threadIdx.x; i < nd; i += blockDim.x) {
+    const double n = 2.0 * (i - half) + 1.0;
+    G[place(i)] = (float)(-1.0 / (M_PI * M_PI * n * n));
   }
   for (size_t row = blockIdx.x; row < rows; row += gridDim.x) {
-    const float* g = sino + row * nd;
     __syncthreads();
-    for (int m = threadIdx.x; m < nd; m += blockDim.x) srow[m] = g[m];
+    for (int m = threadIdx.x; m < nd; m += blockDim.x) srow[(m & 1) * half + (m >> 1)] = sino[row * nd + m];
     __syncthreads();
-    for (int m = threadIdx.x; m < nd; m += blockDim.x) {
-      float v = srow[m];
-      if (ramp) {
-        float acc = 0.25f * srow[m];
-        for (int m2 = (m & 1) ? 0 : 1; m2 < nd; m2 += 2) acc = fmaf(srow[m2], htab[m > m2 ? m - m2 : m2 - m], acc);
-        v = acc;
+    for (int u = threadIdx.x; u < nd / 8; u += blockDim.x) {
+      const int a = u >= nd / 16 ? 1 : 0, i0 = 8 * (u - a * (nd / 16));
+      const float* own = srow + a * half + i0;
+      const float* in = srow + (1 - a) * half;
+      float acc[8], w[8];
+      const int c = i0 + half + a - 1;  // G index of (t = 0, k = 0)
+#pragma unroll
+      for (int t = 0; t < 8; ++t) acc[t] = 0.25f * own[t];
+      // w[(t - k) mod 8] = G[i0 + t - k + a - 1]
+#pragma unroll
+      for (int t = 1; t < 8; ++t) w[t] = G[place(c + t)];
+      for (int k0 = 0; k0 < half; k0 += 8) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const float s = in[k0 + k];
+          const int q = c - k0 - k;
+          w[(8 - k) & 7] = G[place(q)];
+#pragma unroll
+          for (int t = 0; t < 8; ++t) acc[t] = fmaf(s, w[(t - k) & 7], acc[t]);
+        }
       }
-      out[row * nd + m] = mkc((S)v, (S)0);
+#pragma unroll
+      for (int t = 0; t < 8; ++t) out[row * nd + 2 * (i0 + t) + a] = make_float2(acc[t], 0.f);
     }
   }
 }
@@ -683,12 +727,36 @@ __global__ void k_sum_half(const double* __restrict__ part, int n, double* out) 
 __global__ void k_fill(float* x, size_t n, float v) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) x[i] = v;
 }
-// v = w / ||w||, ||w||^2 = sums[5];  lam = sums[0] (v.w)
-__global__ void k_normalize(const float* __restrict__ w, float* __restrict__ v, size_t n, const double* sums, double* lam) {
-  const double nrm = sqrt(sums[5]);
-  const float inv = (float)(1.0 / nrm);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) v[i] = w[i] * inv;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *lam = sums[0];
+// v = w / ||w|| and lam = v.w from pass 3b's partial sums (columns 5 and 0), which every block adds
+// up for itself in the same fixed order: one launch per power step instead of two
+__global__ void __launch_bounds__(256) k_normalize(const float* __restrict__ w, float* __restrict__ v, size_t n,
+                                                   const double* __restrict__ partials, int nblocks, double* lam) {
+  __shared__ double sh[8][2];
+  double s0 = 0.0, s5 = 0.0;
+  for (int b = threadIdx.x; b < nblocks; b += 256) {
+    s0 += partials[(size_t)b * kParts];
+    s5 += partials[(size_t)b * kParts + 5];
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    s0 += __shfl_down_sync(0xffffffffu, s0, o);
+    s5 += __shfl_down_sync(0xffffffffu, s5, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    sh[threadIdx.x >> 5][0] = s0;
+    sh[threadIdx.x >> 5][1] = s5;
+  }
+  __syncthreads();
+  s0 = s5 = 0.0;
+  for (int k = 0; k < 8; ++k) {
+    s0 += sh[k][0];
+    s5 += sh[k][1];
+  }
+  const float inv = (float)(1.0 / sqrt(s5));
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n / 4; i += (size_t)gridDim.x * blockDim.x) {
+    const float4 x = reinterpret_cast<const float4*>(w)[i];
+    reinterpret_cast<float4*>(v)[i] = make_float4(x.x * inv, x.y * inv, x.z * inv, x.w * inv);
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *lam = s0;
 }
 
 // ---------------------------------------------------------------- host side
@@ -729,18 +797,26 @@ void nufft_psi_table(int nmodes, int nfine, int w, double beta, std::vector<doub
   std::vector<double> x, wt;
   gauss_legendre(4 * w + 40, x, wt);
   const int off = (nmodes % 2 == 1) ? (nmodes - 1) / 2 : nmodes / 2;
-  out.resize(nmodes);
-  for (int i = 0; i < nmodes; ++i) {
-    const int d = i - off;
-    double s = 0.0;
-    for (size_t q = 0; q < x.size(); ++q) {
-      const double u = 0.5 * w * x[q];
-      const double z = x[q];
-      const double t = 1.0 - z * z;
-      const double psi = t > 0 ? exp(beta * (sqrt(t) - 1.0)) : 0.0;
-      s += wt[q] * psi * cos(2.0 * M_PI * d * u / nfine);
+  out.assign(nmodes, 0.0);
+  // per node, cos(d theta) by rotation, restarted from the library's sine and cosine every 32 modes (the
+  // rotations add about 32 units of roundoff), for d >= 0: the table is even in d
+  for (size_t q = 0; q < x.size(); ++q) {
+    const double t = 1.0 - x[q] * x[q];
+    const double f = 0.5 * w * wt[q] * (t > 0 ? exp(beta * (sqrt(t) - 1.0)) : 0.0);
+    const double theta = 2.0 * M_PI * (0.5 * w * x[q]) / nfine;
+    const double cr = cos(theta), sr = sin(theta);
+    double c = 1.0, s = 0.0;
+    for (int d = 0; d <= off; ++d) {
+      if (d % 32 == 0) {
+        c = cos(d * theta);
+        s = sin(d * theta);
+      }
+      out[off - d] += f * c;
+      if (d > 0 && off + d < nmodes) out[off + d] += f * c;
+      const double cn = c * cr - s * sr;
+      s = s * cr + c * sr;
+      c = cn;
     }
-    out[i] = 0.5 * w * s;
   }
 }
 
@@ -913,6 +989,8 @@ int build_spread_matrix(Ctx& c, int gi) {
   return TMBIR_OK;
 }
 
+static int place_len(int nd) { return nd + nd / 8; }  // the gapped table of k_ramp_rows
+
 template <class C>
 static int backproject_t(Ctx& c, int gi, const float* d_sino, float* d_out, bool ramp, float scale, char* scratch,
                          cudaStream_t s, bool local_out, const double* wts) {
@@ -931,19 +1009,34 @@ static int backproject_t(Ctx& c, int gi, const float* d_sino, float* d_out, bool
     const int nb = std::min(B, g.S - b0);
     const float* sino_b = d_sino + g.sino_off + (size_t)b0 * rows;
     // radial 1D transform of every projection: G(a, k)
-    k_prepare_rows<C><<<(int)std::min<size_t>((size_t)nb * na, 4096), 256, 2 * nd * sizeof(float), s>>>(
-        sino_b, nd, (size_t)nb * na, ramp ? 1 : 0, strengths);
+    if constexpr (sizeof(real_t<C>) == 4) {
+      if (ramp)
+        k_ramp_rows<<<(int)std::min<size_t>((size_t)nb * na, 152 * 8), 256, (nd + place_len(nd)) * sizeof(float), s>>>(
+            sino_b, nd, (size_t)nb * na, strengths);
+    }
+    if (!ramp)
+      k_prepare_rows<C><<<(int)std::min<size_t>(((size_t)nb * rows + 255) / 256, 152 * 16), 256, 0, s>>>(
+          sino_b, (size_t)nb * rows, strengths);
     TMBIR_CHECK_LAUNCH();
     k_twiddle<C><<<(nd + 255) / 256, 256, 0, s>>>(tw, nd);
     TMBIR_CHECK_LAUNCH();
     if (int e = fft_rows(strengths, nd, nb * na, +1, tw, s)) return e;
-    constexpr int PB = kBackprojBatch / 2;  // slice pairs per batch
+    // slice pairs of the batch; the gather is instantiated for one, two and four (a sample's strengths
+    // and the sums of the absent pairs cost the same as those of the others)
     const int np = (nb + 1) / 2;
-    k_strength_pack<PB, C><<<1024, 256, 0, s>>>(strengths, nd, rows, nb, strengths_t, wts);
-    TMBIR_CHECK_LAUNCH();
-    k_csr_gather<PB, C><<<(ncells + 255) / 256, 256, 0, s>>>(sp.ptr, sp.idx, sp.wt, ncells, strengths_t,
-                                                              grid, np);
-    TMBIR_CHECK_LAUNCH();
+    auto gather = [&](auto PB_) -> int {
+      constexpr int PB = decltype(PB_)::value;
+      k_strength_pack<PB, C><<<1024, 256, 0, s>>>(strengths, nd, rows, nb, strengths_t, wts);
+      TMBIR_CHECK_LAUNCH();
+      k_csr_gather<PB, C><<<(ncells + 255) / 256, 256, 0, s>>>(sp.ptr, sp.idx, sp.wt, ncells, strengths_t, grid, np);
+      TMBIR_CHECK_LAUNCH();
+      return TMBIR_OK;
+    };
+    static_assert(kBackprojBatch == 8, "pairs per batch");
+    if (int e = np == 1   ? gather(std::integral_constant<int, 1>{})
+                : np == 2 ? gather(std::integral_constant<int, 2>{})
+                          : gather(std::integral_constant<int, 4>{}))
+      return e;
     k_twiddle<C><<<(nf + 255) / 256, 256, 0, s>>>(tw, nf);
     TMBIR_CHECK_LAUNCH();
     // 2D transform of the pair grids with the output pruned to the N x N image modes
@@ -1168,8 +1261,7 @@ int power_iteration(Ctx& c, int gi, int steps) {
     a.st = nullptr;
     if (int e = launch_convolution(g, a, Pass3Mode::Apply, pc, s)) return e;
     if (int e = launch_pass3(g, a, Pass3Mode::Apply, pc, c.partials, 0, s, false, 2)) return e;
-    if (int e = launch_sum_partials(c.partials, blocks_pass3(g), c.dscal, s)) return e;
-    k_normalize<<<256, 256, 0, s>>>(w, v, n, c.dscal, g.lam_max);
+    k_normalize<<<152, 256, 0, s>>>(w, v, n, c.partials, blocks_pass3(g), g.lam_max);
     TMBIR_CHECK_LAUNCH();
   }
   return TMBIR_OK;
