@@ -6,9 +6,10 @@
 // The two 32 -> 32 layers are implicit GEMMs on the 5th-generation tensor cores (tcgen05.mma,
 // BF16 operands in shared memory, FP32 accumulators in TMEM): M = 128 pixels of an image row,
 // N = 32 output channels, K = 9 taps x 32 channels.
-// Their data gradient is the same kernel run on the flipped, transposed weights.  The first
-// and last layers (32 MACs per tap) and all weight gradients run on the CUDA cores; weight
-// gradients are reduced over a fixed set of blocks in a fixed order (deterministic).
+// Their data gradient is the same kernel run on the flipped, transposed weights, and their weight
+// gradients are GEMMs over the pixels on the same tensor cores.  The first and last layers (32 MACs
+// per tap) run on the CUDA cores.  Weight gradients are reduced over a fixed set of blocks in a fixed
+// order (deterministic).
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -296,7 +297,9 @@ __global__ void __launch_bounds__(256) k_conv_first(const float* __restrict__ x,
 // entries from shared memory.  Four lanes share a pixel, eight channels each (one 16-byte load, whole
 // lines per warp) with their 72 weights in registers as channel pairs; their nine partial sums are
 // added by exchanging halves, so that a lane ends with two or three of the nine.  Bound by FP32 issue
-// and by the activation stream (64 B per pixel).
+// and by the activation stream (64 B per pixel, 79 us at 8 x 1024^2).  The loads of four pixels are
+// issued before their sums: with one or two in flight the warps waited for memory (8 x 1024^2: 412 us,
+// with four 305).
 // DGRAD: the data gradient of layer 0, gin[p] = sum_{tap, co} w0[co][tap] g0[p - tap][co]: the same
 // sums with layer 0's weights, the taps flipped and no bias.
 constexpr int kLH = 16, kLW = 32;
@@ -322,43 +325,55 @@ __global__ void __launch_bounds__(256, 2) k_conv_last(const __nv_bfloat16* __res
     const int b = tile / tpi, ty = (tile % tpi) / tiles_x, tx = tile % tiles_x;
     const int y0 = ty * kLH, x0 = tx * kLW;
     __syncthreads();  // T of the previous tile consumed
-#pragma unroll 2
-    for (int i = threadIdx.x >> 2; i < (PX + 7) / 8 * 8; i += 64) {
-      const int gy = y0 - 1 + i / (kLW + 2), gx = x0 - 1 + i % (kLW + 2);
-      uint4 u = make_uint4(0, 0, 0, 0);
-      if (i < PX && gy >= 0 && gy < H && gx >= 0 && gx < W)
-        u = __ldg(reinterpret_cast<const uint4*>(a2 + (((size_t)b * H + gy) * W + gx) * kC) + q);
-      const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
-      float2 s[9];
+    // several pixels per lane quad and step, their loads issued first
+    constexpr int BATCH = 4;
+#pragma unroll 1
+    for (int i0 = threadIdx.x >> 2; (i0 & ~7) < PX; i0 += BATCH * 64) {
+      uint4 ub[BATCH];
 #pragma unroll
-      for (int t = 0; t < 9; ++t) s[t] = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const float2 a = __bfloat1622float2(h[c]);
-#pragma unroll
-        for (int t = 0; t < 9; ++t) s[t] = __ffma2_rn(w[c][t], a, s[t]);
-      }
-      float t[9];
-#pragma unroll
-      for (int k = 0; k < 9; ++k) t[k] = s[k].x + s[k].y;
-      // lanes differing in bit 0 share taps 0-3 / 4-7, then in bit 1 the pairs; tap 8 by all
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float give = b0 ? t[k] : t[k + 4];
-        t[k] = (b0 ? t[k + 4] : t[k]) + __shfl_xor_sync(0xffffffffu, give, 1);
+      for (int k = 0; k < BATCH; ++k) {
+        const int i = i0 + 64 * k, gy = y0 - 1 + i / (kLW + 2), gx = x0 - 1 + i % (kLW + 2);
+        ub[k] = make_uint4(0, 0, 0, 0);
+        if (i < PX && gy >= 0 && gy < H && gx >= 0 && gx < W)
+          ub[k] = __ldg(reinterpret_cast<const uint4*>(a2 + (((size_t)b * H + gy) * W + gx) * kC) + q);
       }
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const float give = b1 ? t[k] : t[k + 2];
-        t[k] = (b1 ? t[k + 2] : t[k]) + __shfl_xor_sync(0xffffffffu, give, 2);
-      }
-      t[8] += __shfl_xor_sync(0xffffffffu, t[8], 1);
-      t[8] += __shfl_xor_sync(0xffffffffu, t[8], 2);
-      if (i < PX) {
-        float* d = T[i] + (b0 ? 4 : 0) + (b1 ? 2 : 0);
-        d[0] = t[0];
-        d[1] = t[1];
-        if (q == 0) T[i][8] = t[8];
+      for (int k = 0; k < BATCH; ++k) {
+        const int i = i0 + 64 * k;
+        if ((i & ~7) >= PX) break;  // the same for the whole warp, which holds eight consecutive pixels
+        const uint4 u = ub[k];
+        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&u);
+        float2 s[9];
+#pragma unroll
+        for (int t = 0; t < 9; ++t) s[t] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const float2 a = __bfloat1622float2(h[c]);
+#pragma unroll
+          for (int t = 0; t < 9; ++t) s[t] = __ffma2_rn(w[c][t], a, s[t]);
+        }
+        float t[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) t[k] = s[k].x + s[k].y;
+        // lanes differing in bit 0 share taps 0-3 / 4-7, then in bit 1 the pairs; tap 8 by all
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const float give = b0 ? t[k] : t[k + 4];
+          t[k] = (b0 ? t[k + 4] : t[k]) + __shfl_xor_sync(0xffffffffu, give, 1);
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const float give = b1 ? t[k] : t[k + 2];
+          t[k] = (b1 ? t[k + 2] : t[k]) + __shfl_xor_sync(0xffffffffu, give, 2);
+        }
+        t[8] += __shfl_xor_sync(0xffffffffu, t[8], 1);
+        t[8] += __shfl_xor_sync(0xffffffffu, t[8], 2);
+        if (i < PX) {
+          float* d = T[i] + (b0 ? 4 : 0) + (b1 ? 2 : 0);
+          d[0] = t[0];
+          d[1] = t[1];
+          if (q == 0) T[i][8] = t[8];
+        }
       }
     }
     __syncthreads();
@@ -378,7 +393,8 @@ __global__ void __launch_bounds__(256, 2) k_conv_last(const __nv_bfloat16* __res
 
 // g2[p][ci] = (a2[p][ci] > 0) * sum_tap w3[ci][tap] gout[p - tap].  A block stages a 16 x 32 tile of
 // gout with a one-pixel halo; four lanes share a pixel, eight channels each with their weights in
-// registers, so the mask is read and the result written in whole lines.
+// registers, so the mask is read and the result written in whole lines.  Four masks are loaded before
+// their pixels are computed (8 x 1024^2: 397 -> 319 us).
 __global__ void __launch_bounds__(256, 2) k_last_dgrad(const float* __restrict__ gout, const __nv_bfloat16* __restrict__ a2,
                                                        int B, int H, int W, const float* __restrict__ master,
                                                        __nv_bfloat16* __restrict__ g2) {
@@ -404,30 +420,39 @@ __global__ void __launch_bounds__(256, 2) k_last_dgrad(const float* __restrict__
           (gy >= 0 && gy < H && gx >= 0 && gx < W) ? __ldg(gout + ((size_t)b * H + gy) * W + gx) : 0.f;
     }
     __syncthreads();
-#pragma unroll 2
-    for (int i = threadIdx.x >> 2; i < kLH * kLW; i += 64) {
-      const int ly = i / kLW, lx = i % kLW, gy = y0 + ly, gx = x0 + lx;
-      if (gy >= H || gx >= W) continue;
-      const size_t at = (((size_t)b * H + gy) * W + gx) * kC + 8 * q;
-      const uint4 mk = __ldg(reinterpret_cast<const uint4*>(a2 + at));
-      const __nv_bfloat162* mh = reinterpret_cast<const __nv_bfloat162*>(&mk);
-      float2 s[4];
+    constexpr int BATCH = 4;
+#pragma unroll 1
+    for (int i0 = threadIdx.x >> 2; i0 < kLH * kLW; i0 += BATCH * 64) {
+      uint4 mb[BATCH];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) s[c] = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int t = 0; t < 9; ++t) {
-        const float gv = gt[ly + 2 - t / 3][lx + 2 - t % 3];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) s[c] = __ffma2_rn(w[c][t], make_float2(gv, gv), s[c]);
+      for (int k = 0; k < BATCH; ++k) {
+        const int i = i0 + 64 * k, gy = y0 + i / kLW, gx = x0 + i % kLW;
+        mb[k] = make_uint4(0, 0, 0, 0);
+        if (gy < H && gx < W) mb[k] = __ldg(reinterpret_cast<const uint4*>(a2 + (((size_t)b * H + gy) * W + gx) * kC + 8 * q));
       }
-      uint4 o;
-      __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&o);
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const float2 a = __bfloat1622float2(mh[c]);
-        oh[c] = __floats2bfloat162_rn(a.x > 0.f ? s[c].x : 0.f, a.y > 0.f ? s[c].y : 0.f);
+      for (int k = 0; k < BATCH; ++k) {
+        const int i = i0 + 64 * k, ly = i / kLW, lx = i % kLW, gy = y0 + ly, gx = x0 + lx;
+        if (gy >= H || gx >= W) continue;
+        const __nv_bfloat162* mh = reinterpret_cast<const __nv_bfloat162*>(&mb[k]);
+        float2 s[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) s[c] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+          const float gv = gt[ly + 2 - t / 3][lx + 2 - t % 3];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) s[c] = __ffma2_rn(w[c][t], make_float2(gv, gv), s[c]);
+        }
+        uint4 o;
+        __nv_bfloat162* oh = reinterpret_cast<__nv_bfloat162*>(&o);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const float2 a = __bfloat1622float2(mh[c]);
+          oh[c] = __floats2bfloat162_rn(a.x > 0.f ? s[c].x : 0.f, a.y > 0.f ? s[c].y : 0.f);
+        }
+        *reinterpret_cast<uint4*>(g2 + (((size_t)b * H + gy) * W + gx) * kC + 8 * q) = o;
       }
-      *reinterpret_cast<uint4*>(g2 + at) = o;
     }
   }
 }
@@ -447,7 +472,7 @@ __global__ void __launch_bounds__(256, 2) k_last_dgrad(const float* __restrict__
 // than one FP32 chain per thread over all pixels.
 // Bound by the operand reads from shared memory (4 KB of A per MMA) and by the two activation
 // streams (128 B per pixel); the CUDA-core form this replaced read every pixel's nine neighbours
-// in every thread: 76 ms at 8 x 1024^2.
+// in every thread: 76 ms at 8 x 1024^2, now 0.55.
 constexpr int kGRows = 4;
 constexpr int kGRowB = 4 * kTM * 16;               // bytes of one staged row of g
 constexpr int kGInB = 6 * kChunkB;                 // one staged input row: four chunks, ones, zeros
@@ -581,7 +606,8 @@ __global__ void __launch_bounds__(128, 2) k_wgrad32(const __nv_bfloat16* __restr
 // channel pair (packed FP32 FMAs), the two half-warps walk the two halves of the row, and the nine
 // values of f slide along x, so a step costs one 4-byte load of h and three shared loads of f for
 // 18 sums.  Partial row layout: [0, 288) dW, then the bias.  The form this replaced read h once
-// per tap and pixel from 64 to 128 threads a block: 23.5 ms (first) and 36.9 ms (last) at 8 x 1024^2.
+// per tap and pixel from 64 to 128 threads a block: 23.5 ms (first) and 36.9 ms (last)
+// at 8 x 1024^2, now 0.23 and 0.23.
 constexpr int kEH = 8, kEW = 128;
 template <bool FIRST>
 __global__ void __launch_bounds__(256) k_wgrad_edge(const __nv_bfloat16* __restrict__ h, const float* __restrict__ f,
