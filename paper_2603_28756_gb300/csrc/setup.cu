@@ -7,9 +7,9 @@
 // The type-1 transform spreads the samples onto an oversampled periodic grid with the
 // "exponential of semicircle" kernel psi(u) = exp(beta (sqrt(1 - (2u/w)^2) - 1)) (Barnett,
 // Magland & af Klinteberg 2019), takes a 2D FFT and divides each output mode by the
-// kernel's Fourier transform.  K (4N grid, width 12) and R*g (5N/4 grid, width 14) run in
-// FP64, the FBP start (2N grid, width 10) in FP32.  K is spread with fixed-point integer atomics and R*g / FBP through a sorted sparse
-// matrix, so every result is bit-reproducible.
+// kernel's Fourier transform.  K (4N grid, width 12) runs in FP64, R*g (5N/4 grid, width 14) in
+// double-word FP32, the FBP start (2N grid, width 10) in FP32.  K is spread with fixed-point integer
+// atomics and R*g / FBP through a sorted sparse matrix, so every result is bit-reproducible.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -41,7 +41,7 @@ __device__ __forceinline__ void stockham_stage(const C* X, C* Y, int n, int Ls, 
     reg_dft<R, DIR, C>(a);
     const int o = (j - k) * R + k;
 #pragma unroll
-    for (int m = 0; m < R; ++m) Y[o + m * Ls] = a[m];
+    for (int m = 0; m < R; ++m) Y[o + m * Ls] = settle(a[m]);
   }
 }
 
@@ -64,9 +64,11 @@ __device__ __forceinline__ void load_row(const C* __restrict__ row, C* X, int n,
   }
 }
 
-// plan: the radices, one per 4-bit digit from the lowest (built by fft_plan)
+// plan: the radices, one per 4-bit digit from the lowest (built by fft_plan).  n / 8 threads: one
+// butterfly each in a radix-8 stage (256 threads left a second, nearly empty round of the 320
+// butterflies of a 2560-point row, and too few warps beside the two buffers).
 template <int DIR, class C>
-__global__ void __launch_bounds__(256) k_fft_rows(C* data, int n, unsigned plan, size_t stride, const C* __restrict__ tw) {
+__global__ void __launch_bounds__(640) k_fft_rows(C* data, int n, unsigned plan, size_t stride, const C* __restrict__ tw) {
   extern __shared__ unsigned char smraw[];
   C* X = reinterpret_cast<C*>(smraw);
   C* Y = X + n;
@@ -179,11 +181,12 @@ static int fft_rows(C* data, int n, int rows, int dir, const C* tw, cudaStream_t
     return TMBIR_OK;
   }
   const unsigned plan = fft_plan(n);
+  const int threads = std::min(((n + 7) / 8 + 31) / 32 * 32, 640);
   if (!plan) return set_error(TMBIR_ERR_SHAPE, "setup FFT length must be 2^a 3^b 5^c");
   if (dir < 0)
-    k_fft_rows<-1, C><<<rows, 256, smem, s>>>(data, n, plan, (size_t)n, tw);
+    k_fft_rows<-1, C><<<rows, threads, smem, s>>>(data, n, plan, (size_t)n, tw);
   else
-    k_fft_rows<1, C><<<rows, 256, smem, s>>>(data, n, plan, (size_t)n, tw);
+    k_fft_rows<1, C><<<rows, threads, smem, s>>>(data, n, plan, (size_t)n, tw);
   TMBIR_CHECK_LAUNCH();
   return TMBIR_OK;
 }
@@ -196,12 +199,13 @@ static int transpose(const C* in, C* out, int rows, int cols, int batch, cudaStr
   return TMBIR_OK;
 }
 
-// 2D FFT of `batch` n x n grids; result left transposed in `tmp` (tmp[b][kx][ky]).
+// 2D FFT of `batch` n x n grids; result left transposed in `tmp` (tmp[b][kx][ky]).  keep: of a single
+// grid, only kx < keep are transformed along y (0: all).
 template <class C>
-static int fft2_transposed(C* grid, C* tmp, int n, int batch, int dir, const C* tw, cudaStream_t s) {
+static int fft2_transposed(C* grid, C* tmp, int n, int batch, int dir, const C* tw, cudaStream_t s, int keep = 0) {
   if (int e = fft_rows(grid, n, n * batch, dir, tw, s)) return e;
   if (int e = transpose(grid, tmp, n, n, batch, s)) return e;
-  return fft_rows(tmp, n, n * batch, dir, tw, s);
+  return fft_rows(tmp, n, keep ? keep : n * batch, dir, tw, s);
 }
 
 // ---------------------------------------------------------------- spreading
@@ -480,53 +484,90 @@ __device__ __forceinline__ void gather_add(df w, df v, df& acc) {
   acc = df(s.hi, __fadd_rn(l, __fadd_rn(s.lo, e)));
 }
 __device__ __forceinline__ float gather_end(float acc) { return acc; }
-__device__ __forceinline__ df gather_end(df acc) { return two_sum(acc.hi, acc.lo); }
+__device__ __forceinline__ df gather_end(df acc) { return settle(acc); }
 
-// grid[b][cell] = sum_j wt[j] strengths[idx[j]][b], B slice pairs per launch (sample-major
-// strengths).  U entries per step with all their loads issued first (the index load and the
-// dependent strength loads are a latency chain); the accumulation order is that of one at a time.
-template <int B, class C>
-__global__ void k_csr_gather(const int* __restrict__ ptr, const int* __restrict__ idx, const double* __restrict__ wt,
-                             int ncells, const C* __restrict__ strengths, C* __restrict__ grid, int nb) {
+__device__ __forceinline__ float shfl_down(float v, int o) { return __shfl_down_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ df shfl_down(df v, int o) { return df(shfl_down(v.hi, o), shfl_down(v.lo, o)); }
+
+// acc += entries j0, j0 + step, ... < e of a row, U at a time with all their loads issued first (the
+// index load and the dependent strength loads are a latency chain), in that order
+template <int B, int U, class C>
+__device__ __forceinline__ void gather_row(int j0, int e, int step, const int* __restrict__ idx,
+                                           const double* __restrict__ wt, const C* __restrict__ strengths, C (&acc)[B]) {
   using S = real_t<C>;
-  constexpr int U = B >= 4 ? 2 : (B == 2 ? 4 : 8);
-  for (int cell = blockIdx.x * blockDim.x + threadIdx.x; cell < ncells; cell += gridDim.x * blockDim.x) {
-    C acc[B];
+  int j = j0;
+  for (; j + (U - 1) * step < e; j += U * step) {
+    S w[U];
+    C v[U][B];
 #pragma unroll
-    for (int b = 0; b < B; ++b) acc[b] = mkc((S)0, (S)0);
-    const int e = ptr[cell + 1];
-    int j = ptr[cell];
-    for (; j + U <= e; j += U) {
-      S w[U];
-      C v[U][B];
+    for (int u = 0; u < U; ++u) {
+      const C* sv = strengths + (size_t)idx[j + u * step] * B;
+      w[u] = load_wt<S>(wt, j + u * step);
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const C* sv = strengths + (size_t)idx[j + u] * B;
-        w[u] = load_wt<S>(wt, j + u);
-#pragma unroll
-        for (int b = 0; b < B; ++b) v[u][b] = sv[b];
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int b = 0; b < B; ++b) {
-          gather_add(w[u], v[u][b].x, acc[b].x);
-          gather_add(w[u], v[u][b].y, acc[b].y);
-        }
+      for (int b = 0; b < B; ++b) v[u][b] = sv[b];
     }
-    for (; j < e; ++j) {
-      const C* sv = strengths + (size_t)idx[j] * B;
-      const S w = load_wt<S>(wt, j);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
 #pragma unroll
       for (int b = 0; b < B; ++b) {
-        const C v = sv[b];
-        gather_add(w, v.x, acc[b].x);
-        gather_add(w, v.y, acc[b].y);
+        gather_add(w[u], v[u][b].x, acc[b].x);
+        gather_add(w[u], v[u][b].y, acc[b].y);
       }
+  }
+  for (; j < e; j += step) {
+    const C* sv = strengths + (size_t)idx[j] * B;
+    const S w = load_wt<S>(wt, j);
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      const C v = sv[b];
+      gather_add(w, v.x, acc[b].x);
+      gather_add(w, v.y, acc[b].y);
     }
+  }
+}
+
+// grid[b][cell] = sum_j wt[j] strengths[idx[j]][b], B slice pairs per launch (sample-major
+// strengths).  A thread sums the row of one cell; a row of more than kLongRow entries (near the
+// grid's centre they reach 11 per angle) is shared by the warp, each lane every 32nd entry, and the
+// lanes' sums are added in a fixed tree: one thread's chain through the longest row was the time of
+// the whole launch (1.2 ms at 4 x 512^2, 181 angles).
+constexpr int kLongRow = 96;
+template <int B, class C>
+__global__ void __launch_bounds__(256) k_csr_gather(const int* __restrict__ ptr, const int* __restrict__ idx,
+                                                    const double* __restrict__ wt, int ncells,
+                                                    const C* __restrict__ strengths, C* __restrict__ grid, int nb) {
+  using S = real_t<C>;
+  constexpr int U = B >= 4 ? 2 : (B == 2 ? 4 : 8);
+  const int cell = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
+  const int j0 = cell < ncells ? ptr[cell] : 0, e = cell < ncells ? ptr[cell + 1] : 0;
+  const bool is_long = e - j0 > kLongRow;
+  C acc[B];
+  auto put = [&](int at) {
 #pragma unroll
     for (int b = 0; b < B; ++b)
-      if (b < nb) grid[(size_t)b * ncells + cell] = mkc(gather_end(acc[b].x), gather_end(acc[b].y));
+      if (b < nb) grid[(size_t)b * ncells + at] = mkc(gather_end(acc[b].x), gather_end(acc[b].y));
+  };
+  if (cell < ncells && !is_long) {
+#pragma unroll
+    for (int b = 0; b < B; ++b) acc[b] = mkc((S)0, (S)0);
+    gather_row<B, U>(j0, e, 1, idx, wt, strengths, acc);
+    put(cell);
+  }
+  for (unsigned todo = __ballot_sync(0xffffffffu, is_long); todo; todo &= todo - 1) {
+    const int src = __ffs(todo) - 1;
+    const int b0 = __shfl_sync(0xffffffffu, j0, src), b1 = __shfl_sync(0xffffffffu, e, src);
+#pragma unroll
+    for (int b = 0; b < B; ++b) acc[b] = mkc((S)0, (S)0);
+    gather_row<B, U>(b0 + lane, b1, 32, idx, wt, strengths, acc);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+      for (int b = 0; b < B; ++b) {
+        acc[b].x = acc[b].x + shfl_down(acc[b].x, o);
+        acc[b].y = acc[b].y + shfl_down(acc[b].y, o);
+      }
+    }
+    if (lane == 0) put(cell - lane + src);
   }
 }
 // tmp[b][j][r] = grid[b][r][(j - N/2) mod nf] for the N kept x-modes j (column pruning)
@@ -575,18 +616,20 @@ __global__ void __launch_bounds__(256) k_deconv_pruned(const C* __restrict__ B, 
     if (c >= N || r >= N) continue;
     const C v = tile[threadIdx.x][i];
     const df f = inv_c[threadIdx.x] * inv_r[i];
-    out[((size_t)(2 * p) * N + r) * N + c] = (df(v.x) * f).hi;
-    if (2 * p + 1 < nb) out[((size_t)(2 * p + 1) * N + r) * N + c] = (df(v.y) * f).hi;
+    out[((size_t)(2 * p) * N + r) * N + c] = to_float(df(v.x) * f);
+    if (2 * p + 1 < nb) out[((size_t)(2 * p + 1) * N + r) * N + c] = to_float(df(v.y) * f);
   }
 }
 
-// K[(dy+N-1)(2N-1) + dx+N-1] = Re B[dx][dy] / (psi(dx) psi(dy)); B transposed ([kx][ky]).
+// K[(dy+N-1)(2N-1) + dx+N-1] = Re B[dx][dy] / (psi(dx) psi(dy)); B transposed ([kx][ky]), of which only
+// dx >= 0 is there: K(-d) = K(d), so the FP64 transforms of the other three quarters of the rows are
+// left out.
 __global__ void k_deconv_K(const double2* __restrict__ B, int nf, int N, const double* __restrict__ psi, double* K) {
   const int W = 2 * N - 1;
   for (int id = blockIdx.x * blockDim.x + threadIdx.x; id < W * W; id += gridDim.x * blockDim.x) {
     const int ix = id % W, iy = id / W;
     const int dx = ix - (N - 1), dy = iy - (N - 1);
-    const double2 v = B[(size_t)((dx + nf) % nf) * nf + (dy + nf) % nf];
+    const double2 v = dx < 0 ? B[(size_t)-dx * nf + (nf - dy) % nf] : B[(size_t)dx * nf + (dy + nf) % nf];
     K[id] = v.x / (psi[ix] * psi[iy]);
   }
 }
@@ -920,7 +963,7 @@ int build_kernel_spectrum(Ctx& c, int gi) {
   }
   k_fixed_to_complex<<<1024, 256, 0, s>>>(fixed_grid, grid, (size_t)nf * nf);
   TMBIR_CHECK_LAUNCH();
-  if (int e = fft2_transposed(grid, tmp, nf, 1, +1, tw, s)) return e;
+  if (int e = fft2_transposed(grid, tmp, nf, 1, +1, tw, s, N)) return e;
   k_deconv_K<<<1024, 256, 0, s>>>(tmp, nf, N, g.psiK, g.K);
   TMBIR_CHECK_LAUNCH();
   return circulant_spectrum(c, gi);
@@ -939,7 +982,7 @@ static int circulant_spectrum(Ctx& c, int gi) {
   double2* ct = grid + (size_t)M * M;
   k_circulant<<<1024, 256, 0, s>>>(g.K, N, cg);
   TMBIR_CHECK_LAUNCH();
-  if (int e = fft2_transposed(cg, ct, M, 1, -1, tw, s)) return e;
+  if (int e = fft2_transposed(cg, ct, M, 1, -1, tw, s, N + 1)) return e;  // the spectrum's v = 0 .. N
   k_chat_layout<<<1024, 256, 0, s>>>(ct, N, chat_split(N), g.chat);
   TMBIR_CHECK_LAUNCH();
   return TMBIR_OK;
