@@ -527,10 +527,12 @@ __device__ __forceinline__ void gather_row(int j0, int e, int step, const int* _
 }
 
 // grid[b][cell] = sum_j wt[j] strengths[idx[j]][b], B slice pairs per launch (sample-major
-// strengths).  A thread sums the row of one cell; a row of more than kLongRow entries (near the
-// grid's centre they reach 11 per angle) is shared by the warp, each lane every 32nd entry, and the
-// lanes' sums are added in a fixed tree: one thread's chain through the longest row was the time of
-// the whole launch (1.2 ms at 4 x 512^2, 181 angles).
+// strengths).  A thread sums the row of one cell; for R*g a row of more than kLongRow entries (near
+// the grid's centre they reach 11 per angle) is shared by the warp, each lane every 32nd entry, and
+// the lanes' sums are added in a fixed tree: one thread's chain through the longest row was the time
+// of the whole launch (4 x 512^2, 181 angles: 1.19 -> 0.60 ms).  The FP32 sums of the start keep one
+// thread's order: their chain is four times shorter per entry, and another order would move the
+// start by 4e-7 of its norm, which BF16 iterations after it amplify.
 constexpr int kLongRow = 96;
 template <int B, class C>
 __global__ void __launch_bounds__(256) k_csr_gather(const int* __restrict__ ptr, const int* __restrict__ idx,
@@ -540,7 +542,7 @@ __global__ void __launch_bounds__(256) k_csr_gather(const int* __restrict__ ptr,
   constexpr int U = B >= 4 ? 2 : (B == 2 ? 4 : 8);
   const int cell = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
   const int j0 = cell < ncells ? ptr[cell] : 0, e = cell < ncells ? ptr[cell + 1] : 0;
-  const bool is_long = e - j0 > kLongRow;
+  const bool is_long = std::is_same<C, dfc>::value && e - j0 > kLongRow;
   C acc[B];
   auto put = [&](int at) {
 #pragma unroll

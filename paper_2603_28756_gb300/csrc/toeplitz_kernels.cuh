@@ -160,6 +160,11 @@ __device__ __forceinline__ void block_partials(double (&acc)[kParts], double* re
   }
 }
 
+// the row passes' rotations keep the remainder of 1/sqrt(2) (twmul), except beside BF16 spectra, whose
+// rounding is 2^15 times larger
+template <int DIR, bool BF>
+constexpr int kRowDir = BF ? DIR : 2 * DIR;
+
 // ---------------------------------------------------------------- pass 1: rows, forward
 template <int N, bool BF>
 __global__ void __launch_bounds__(Geo<N>::THREADS) k_pass1(const __grid_constant__ GroupSet gs, StepArgs a) {
@@ -203,7 +208,7 @@ __global__ void __launch_bounds__(Geo<N>::THREADS) k_pass1(const __grid_constant
       v[i] = make_float2(0.f, 0.f);
     }
   });
-  F::template run<-2>(v, sm + (warp * G + grp) * F::SMEM, g.twN, t);
+  F::template run<kRowDir<-1, BF>>(v, sm + (warp * G + grp) * F::SMEM, g.twN, t);
 
   // split the packed transform: Y[v] = E[v] + w^v O[v], needs Z[v] and Z[N - v]
   float2 y[P];
@@ -363,7 +368,7 @@ __global__ void TMBIR_P3A_BOUNDS(Geo3a<N>::THREADS) k_pass3a(const __grid_consta
     q[i] = make_float2(e.x - o.y, e.y + o.x);
   });
   __syncthreads();
-  F::template run<2>(q, sm + (warp * G + grp) * F::SMEM, g.twN, t);
+  F::template run<kRowDir<1, BF>>(q, sm + (warp * G + grp) * F::SMEM, g.twN, t);
   // the first N/2 packed outputs are the N kept columns
   float2* out = reinterpret_cast<float2*>(kz + ((size_t)s * N + r0 + rl) * N);
   SFor<0, P / 2>::run([&](auto i_) {
@@ -495,7 +500,7 @@ __global__ void __launch_bounds__(GeoH<N>::THREADS) k_pass1_h(const __grid_const
     constexpr int i = decltype(i_)::value;
     v[i] = xs[t + T * i];
   });
-  F::template run<-2>(v, xs, g.twN, t);
+  F::template run<kRowDir<-1, BF>>(v, xs, g.twN, t);
   __syncthreads();  // every exchange buffer is free: the staged rows alias them
   float2* zrow = sm + rl * LDZ;
   SFor<0, P>::run([&](auto i_) {
@@ -660,7 +665,7 @@ __global__ void __launch_bounds__(GeoH3<N>::THREADS) k_pass3a_h(const __grid_con
   });
   __syncthreads();  // the staged rows are read: the exchange buffers alias them
   float2* xs = sm + unit * F::SMEM;
-  F::template run<2>(v, xs, g.twN, t);
+  F::template run<kRowDir<1, BF>>(v, xs, g.twN, t);
   __syncwarp();
   SFor<0, P>::run([&](auto i_) {
     constexpr int i = decltype(i_)::value;
