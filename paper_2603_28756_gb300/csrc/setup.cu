@@ -21,27 +21,52 @@ namespace tmbir {
 
 // ---------------------------------------------------------------- batched 1D FFT along rows
 // Stockham autosort in shared memory: one block per row, radix 8/4/2/3/5 stages, natural order
-// in and out.  tw[j] = exp(-2 pi i j / n).
+// in and out.  The L1/shared data pipe bounds it (16 x 2048^2: the rows of the FP32 start waited on
+// twiddles strided through memory and on 8-way bank conflicts), so that
+//   the twiddles lie stage by stage, tw[m Ls + k] = exp(-2 pi i k m / (Ls R)), k < Ls, 0 < m < R: a warp
+//   reads contiguous values, and the stages together need n of them;
+//   the buffers have one value of padding per 128 bytes (the first stage's stores are 8 apart);
+//   the first stage reads and the last one writes global memory.
+// R*g and the FBP start of 16 x 2048^2 together: 6.5 -> 5.6 ms; rows of 4 x 512^2: FP32 37 -> 25 us,
+// double-word 38 -> 34 us.
+
+// index i of a padded row buffer
+template <class C>
+__device__ __forceinline__ int padded(int i) {
+  return i + (i >> (sizeof(C) == 8 ? 4 : 3));
+}
+template <class C>
+constexpr size_t padded_bytes(size_t n) {
+  return (n + n / (128 / sizeof(C)) + 1) * sizeof(C);
+}
+// first: the input is `row`, else X; last: the output is `row`, else Y.  A stage that is both is a whole
+// transform of R points, in one thread.
 template <int R, int DIR, class C>
-__device__ __forceinline__ void stockham_stage(const C* X, C* Y, int n, int Ls, const C* __restrict__ tw) {
+__device__ __forceinline__ void stockham_stage(const C* X, C* Y, C* row, bool first, bool last, int n, int Ls,
+                                               const C* __restrict__ tw) {
   const int nb = n / R;
-  const int tstep = n / (Ls * R);
   for (int j = threadIdx.x; j < nb; j += blockDim.x) {
     const int k = j % Ls;  // Ls is a product of mixed radices
     C a[R];
 #pragma unroll
-    for (int m = 0; m < R; ++m) {
-      C v = X[j + m * nb];
-      if (m > 0 && k > 0) {
-        const C w = tw[(size_t)k * m * tstep];  // k m tstep < n
-        v = DIR < 0 ? cmul(v, w) : cmulc(v, w);
+    for (int m = 0; m < R; ++m) a[m] = first ? row[j + m * nb] : X[padded<C>(j + m * nb)];
+    if (!first) {
+#pragma unroll
+      for (int m = 1; m < R; ++m) {
+        const C w = tw[m * Ls + k];
+        a[m] = DIR < 0 ? cmul(a[m], w) : cmulc(a[m], w);
       }
-      a[m] = v;
     }
     reg_dft<R, DIR, C>(a);
     const int o = (j - k) * R + k;
 #pragma unroll
-    for (int m = 0; m < R; ++m) Y[o + m * Ls] = settle(a[m]);
+    for (int m = 0; m < R; ++m) {
+      const C v = settle(a[m]);
+      if (last)
+        row[o + m * Ls] = v;
+      else
+        Y[padded<C>(o + m * Ls)] = v;
+    }
   }
 }
 
@@ -71,19 +96,17 @@ template <int DIR, class C>
 __global__ void __launch_bounds__(640) k_fft_rows(C* data, int n, unsigned plan, size_t stride, const C* __restrict__ tw) {
   extern __shared__ unsigned char smraw[];
   C* X = reinterpret_cast<C*>(smraw);
-  C* Y = X + n;
+  C* Y = X + padded_bytes<C>(n) / sizeof(C);
   C* row = data + (size_t)blockIdx.x * stride;
-  load_row(row, X, n, [](int j) { return j; });
-  __syncthreads();
-  int Ls = 1;
-  for (; plan != 0; plan >>= 4) {
+  for (int Ls = 1; plan != 0; plan >>= 4) {
     const int R = (int)(plan & 15u);
+    const bool first = Ls == 1, last = plan < 16u;
     switch (R) {
-      case 8: stockham_stage<8, DIR>(X, Y, n, Ls, tw); break;
-      case 4: stockham_stage<4, DIR>(X, Y, n, Ls, tw); break;
-      case 2: stockham_stage<2, DIR>(X, Y, n, Ls, tw); break;
-      case 3: stockham_stage<3, DIR>(X, Y, n, Ls, tw); break;
-      default: stockham_stage<5, DIR>(X, Y, n, Ls, tw); break;
+      case 8: stockham_stage<8, DIR>(X, Y, row, first, last, n, Ls, tw); break;
+      case 4: stockham_stage<4, DIR>(X, Y, row, first, last, n, Ls, tw); break;
+      case 2: stockham_stage<2, DIR>(X, Y, row, first, last, n, Ls, tw); break;
+      case 3: stockham_stage<3, DIR>(X, Y, row, first, last, n, Ls, tw); break;
+      default: stockham_stage<5, DIR>(X, Y, row, first, last, n, Ls, tw); break;
     }
     Ls *= R;
     __syncthreads();
@@ -91,11 +114,11 @@ __global__ void __launch_bounds__(640) k_fft_rows(C* data, int n, unsigned plan,
     X = Y;
     Y = tmp;
   }
-  for (int j = threadIdx.x; j < n; j += blockDim.x) row[j] = X[j];
 }
 
 // In-place variant for rows whose two Stockham buffers do not fit in shared memory: the row
-// is loaded in bit-reversed order, then log2(n) radix-2 decimation-in-time stages.
+// is loaded in bit-reversed order, then log2(n) radix-2 decimation-in-time stages (twiddles stage by
+// stage, R = 2).
 template <int DIR, class C>
 __global__ void __launch_bounds__(1024) k_fft_rows_inplace(C* data, int n, int log2n, size_t stride,
                                                            const C* __restrict__ tw) {
@@ -104,11 +127,11 @@ __global__ void __launch_bounds__(1024) k_fft_rows_inplace(C* data, int n, int l
   C* row = data + (size_t)blockIdx.x * stride;
   load_row(row, X, n, [log2n](int j) { return (int)(__brev((unsigned)j) >> (32 - log2n)); });
   __syncthreads();
-  for (int half = 1, tstep = n / 2; half < n; half <<= 1, tstep >>= 1) {
+  for (int half = 1; half < n; half <<= 1) {
     for (int b = threadIdx.x; b < n / 2; b += blockDim.x) {
       const int k = b & (half - 1);
       const int i0 = 2 * (b - k) + k, i1 = i0 + half;
-      const C w = tw[(size_t)k * tstep];
+      const C w = tw[half + k];
       const C v = DIR < 0 ? cmul(X[i1], w) : cmulc(X[i1], w);
       const C u = X[i0];
       X[i0] = cadd(u, v);
@@ -158,25 +181,55 @@ static unsigned fft_plan(int n) {
   return (n == 1 && shift <= 32) ? plan : 0u;
 }
 
+// rows whose two buffers (without the padding, at most an eighth more) pass this run in place
+constexpr size_t kRowSmem = 200 * 1024;
+
+// the setup FFTs' twiddle table (n values, n up to 4N, at the front of the scratch):
+// tw[m Ls + k] of every stage of `plan`'s radices (0: radix 2 throughout, the in-place kernel)
+template <class C>
+__global__ void k_twiddle(C* tw, int n, unsigned plan) {
+  using S = real_t<C>;
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+    int Ls = 1, R = 2;
+    for (unsigned p = plan;; p >>= 4) {
+      R = plan ? (int)(p & 15u) : 2;
+      if (j < Ls * R) break;
+      Ls *= R;
+    }
+    const long long t = (long long)(j / Ls) * (j % Ls) * (n / (Ls * R));
+    double sv, cv;
+    sincospi(-2.0 * (double)t / n, &sv, &cv);
+    tw[j] = mkc((S)cv, (S)sv);
+  }
+}
+template <class C>
+static int twiddles(C* tw, int n, cudaStream_t s) {
+  k_twiddle<C><<<(n + 255) / 256, 256, 0, s>>>(tw, n, 2 * (size_t)n * sizeof(C) > kRowSmem ? 0u : fft_plan(n));
+  TMBIR_CHECK_LAUNCH();
+  return TMBIR_OK;
+}
+
 template <class C>
 static int fft_rows(C* data, int n, int rows, int dir, const C* tw, cudaStream_t s) {
-  const size_t smem = 2 * (size_t)n * sizeof(C);
+  const size_t smem = 2 * padded_bytes<C>(n);
   static bool attr_set = false;
   if (!attr_set) {
-    TMBIR_CUDA(cudaFuncSetAttribute(k_fft_rows<-1, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_fft_rows<1, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+    constexpr int kMax = (int)(2 * padded_bytes<C>(kRowSmem / (2 * sizeof(C))));
+    static_assert(kMax <= 227 * 1024, "two padded rows");
+    TMBIR_CUDA(cudaFuncSetAttribute(k_fft_rows<-1, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax));
+    TMBIR_CUDA(cudaFuncSetAttribute(k_fft_rows<1, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax));
     TMBIR_CUDA(cudaFuncSetAttribute(k_fft_rows_inplace<-1, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    200 * 1024));
+                                    kRowSmem));
     TMBIR_CUDA(cudaFuncSetAttribute(k_fft_rows_inplace<1, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    200 * 1024));
+                                    kRowSmem));
     attr_set = true;
   }
-  if (smem > 200 * 1024) {
-    if (smem / 2 > 200 * 1024 || (n & (n - 1)) != 0) return set_error(TMBIR_ERR_SHAPE, "setup FFT length too large");
+  if (const size_t one = (size_t)n * sizeof(C); 2 * one > kRowSmem) {
+    if (one > kRowSmem || (n & (n - 1)) != 0) return set_error(TMBIR_ERR_SHAPE, "setup FFT length too large");
     if (dir < 0)
-      k_fft_rows_inplace<-1, C><<<rows, 1024, smem / 2, s>>>(data, n, ilog2(n), (size_t)n, tw);
+      k_fft_rows_inplace<-1, C><<<rows, 1024, one, s>>>(data, n, ilog2(n), (size_t)n, tw);
     else
-      k_fft_rows_inplace<1, C><<<rows, 1024, smem / 2, s>>>(data, n, ilog2(n), (size_t)n, tw);
+      k_fft_rows_inplace<1, C><<<rows, 1024, one, s>>>(data, n, ilog2(n), (size_t)n, tw);
     TMBIR_CHECK_LAUNCH();
     return TMBIR_OK;
   }
@@ -897,17 +950,6 @@ size_t spread_nnz(const tmbir_group& g, int k) {
   return (size_t)g.n_angles * (g.n_det - 1) * kSpreadWidth[k] * kSpreadWidth[k];
 }
 
-// device twiddle tables for the setup FFTs (n up to 4N), carved from the front of the scratch
-template <class C>
-__global__ void k_twiddle(C* tw, int n) {
-  using S = real_t<C>;
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-    double sv, cv;
-    sincospi(-2.0 * j / n, &sv, &cv);
-    tw[j] = mkc((S)cv, (S)sv);
-  }
-}
-
 // K(d) = (1/n_det) sum_a w_a D(e_a . d) summed directly, D(t) = sin(pi (n_det - 1) e / n_det) /
 // sin(pi e / n_det) with e = t reduced to the nearest period of n_det, and n_det - 1 where the
 // denominator vanishes; cs holds (cos, sin) of every angle, wts the weights w_a (nullptr: 1)
@@ -953,8 +995,7 @@ int build_kernel_spectrum(Ctx& c, int gi) {
   double2* tw = reinterpret_cast<double2*>(c.scratch);
   double2* grid = tw + nf;
   double2* tmp = grid + (size_t)nf * nf;
-  k_twiddle<double2><<<(nf + 255) / 256, 256, 0, s>>>(tw, nf);
-  TMBIR_CHECK_LAUNCH();
+  if (int e = twiddles<double2>(tw, nf, s)) return e;
   unsigned long long* fixed_grid = reinterpret_cast<unsigned long long*>(tmp);
   TMBIR_CUDA(cudaMemsetAsync(fixed_grid, 0, sizeof(unsigned long long) * nf * nf, s));
   {
@@ -978,8 +1019,7 @@ static int circulant_spectrum(Ctx& c, int gi) {
   const int N = g.N, M = 2 * N;
   double2* tw = reinterpret_cast<double2*>(c.scratch);
   double2* grid = tw + 4 * (size_t)N;  // past the largest twiddle table
-  k_twiddle<double2><<<(M + 255) / 256, 256, 0, s>>>(tw, M);
-  TMBIR_CHECK_LAUNCH();
+  if (int e = twiddles<double2>(tw, M, s)) return e;
   double2* cg = grid;
   double2* ct = grid + (size_t)M * M;
   k_circulant<<<1024, 256, 0, s>>>(g.K, N, cg);
@@ -1063,8 +1103,7 @@ static int backproject_t(Ctx& c, int gi, const float* d_sino, float* d_out, bool
       k_prepare_rows<C><<<(int)std::min<size_t>(((size_t)nb * rows + 255) / 256, 152 * 16), 256, 0, s>>>(
           sino_b, (size_t)nb * rows, strengths);
     TMBIR_CHECK_LAUNCH();
-    k_twiddle<C><<<(nd + 255) / 256, 256, 0, s>>>(tw, nd);
-    TMBIR_CHECK_LAUNCH();
+    if (int e = twiddles<C>(tw, nd, s)) return e;
     if (int e = fft_rows(strengths, nd, nb * na, +1, tw, s)) return e;
     // slice pairs of the batch; the gather is instantiated for one, two and four (a sample's strengths
     // and the sums of the absent pairs cost the same as those of the others)
@@ -1082,8 +1121,7 @@ static int backproject_t(Ctx& c, int gi, const float* d_sino, float* d_out, bool
                 : np == 2 ? gather(std::integral_constant<int, 2>{})
                           : gather(std::integral_constant<int, 4>{}))
       return e;
-    k_twiddle<C><<<(nf + 255) / 256, 256, 0, s>>>(tw, nf);
-    TMBIR_CHECK_LAUNCH();
+    if (int e = twiddles<C>(tw, nf, s)) return e;
     // 2D transform of the pair grids with the output pruned to the N x N image modes
     if (int e = fft_rows(grid, nf, np * nf, -1, tw, s)) return e;
     {
@@ -1239,10 +1277,8 @@ int forward_project(Ctx& c, int gi, const float* d_x, float* d_sino, cudaStream_
   float2* grid = tw_d + nd;
   float2* tmp = grid + (size_t)PB * cells;
   float2* prow = tmp + (size_t)PB * cells;
-  k_twiddle<float2><<<(nf + 255) / 256, 256, 0, s>>>(tw_f, nf);
-  TMBIR_CHECK_LAUNCH();
-  k_twiddle<float2><<<(nd + 255) / 256, 256, 0, s>>>(tw_d, nd);
-  TMBIR_CHECK_LAUNCH();
+  if (int e = twiddles<float2>(tw_f, nf, s)) return e;
+  if (int e = twiddles<float2>(tw_d, nd, s)) return e;
   for (int b0 = 0; b0 < g.S; b0 += B) {
     const int nb = std::min(B, g.S - b0), np = (nb + 1) / 2;
     k_pad_deconv_pairs<<<1024, 256, 0, s>>>(d_x + g.img_off + (size_t)b0 * N * N, N, nf, nb, sp.psi, grid);
