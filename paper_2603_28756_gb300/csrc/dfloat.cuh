@@ -14,11 +14,10 @@
 // in FP32; a product keeps hi * hi exactly and adds the two cross products to its error.  Neither
 // renormalises the pair (three operations each): the low part then stays within a few units of the
 // high parts' last place, so that its own rounding is 2^-46 of the operands, and settle()
-// renormalises once per butterfly (R*g's
-// error stays at 2.5e-8 to 2.7e-8 of its norm).  The errors are bounded relative to the operands'
-// magnitudes, not to the result's, which is the bound an FFT or a dot product needs (their errors are
-// judged against the input's norm).  Every step uses the _rn intrinsics, which the compiler never
-// contracts into FMAs, so the transformations stay error-free.
+// renormalises once per butterfly (R*g's error stays at 2.5e-8 to 2.7e-8 of its norm).  The errors
+// are bounded relative to the operands' magnitudes, not to the result's, which is the bound an FFT or
+// a dot product needs (their errors are judged against the input's norm).  Every step uses the _rn
+// intrinsics, which the compiler never contracts into FMAs, so the transformations stay error-free.
 #pragma once
 #include <cuda_runtime.h>
 

@@ -583,7 +583,8 @@ __device__ __forceinline__ void gather_row(int j0, int e, int step, const int* _
 // strengths).  A thread sums the row of one cell; for R*g a row of more than kLongRow entries (near
 // the grid's centre they reach 11 per angle) is shared by the warp, each lane every 32nd entry, and
 // the lanes' sums are added in a fixed tree: one thread's chain through the longest row was the time
-// of the whole launch (4 x 512^2, 181 angles: 1.19 -> 0.60 ms).  The FP32 sums of the start keep one
+// of the whole launch (4 x 512^2, 181 angles: 1.19 -> 0.60 ms; 8 x 2048^2, 128 angles, with the
+// compensated sums: 1.80 -> 0.96 ms).  The FP32 sums of the start keep one
 // thread's order: their chain is four times shorter per entry, and another order would move the
 // start by 4e-7 of its norm, which BF16 iterations after it amplify.
 constexpr int kLongRow = 96;
@@ -647,7 +648,7 @@ __global__ void k_transpose_prune(const C* __restrict__ in, C* __restrict__ out,
 // and both sides are read and written along their contiguous index.  Grid: (N/32, N/32, pairs).
 // The factors 1 / psi are double-words (FP64 divisions, one per row and column of the tile), so that a
 // pixel takes two double-word products on the FP32 pipe instead of conversions and products on the
-// FP64 one, whose rate bound this kernel.
+// FP64 one, whose rate bound this kernel (8 x 2048^2, double-word: 435 -> 109 us).
 template <class C>
 __global__ void __launch_bounds__(256) k_deconv_pruned(const C* __restrict__ B, int nf, int N, int nb,
                                                        const double* __restrict__ psi, float scale,
@@ -723,8 +724,8 @@ __global__ void k_prepare_rows(const float* __restrict__ sino, size_t n, C* out)
 // uses it).  An output couples to the inputs of the other parity alone: with m = 2 i + a,
 //   out_1[i] = s_1[i] / 4 + sum_k s_0[k] G[i - k],  out_0[i] = s_0[i] / 4 + sum_k s_1[k] G[i - k - 1],
 // G[d] = h(2 d + 1).  A thread owns eight consecutive i of one parity, so that one input and one
-// new value of G serve eight products (two shared loads per product bound the direct form: 0.8 ms for
-// 1024 rows of 2048 bins).  G is stored with a gap every eight values: threads read it eight apart.
+// new value of G serve eight products (two shared loads per product bound the direct form: 0.82 ms for
+// 1024 rows of 2048 bins, now 0.16).  G is stored with a gap every eight values: threads read it eight apart.
 __global__ void __launch_bounds__(256) k_ramp_rows(const float* __restrict__ sino, int nd, size_t rows, float2* out) {
   extern __shared__ float rs[];
   const int half = nd / 2;
