@@ -131,9 +131,9 @@ typedef struct {
 
 /*
  * Create a context bound to a CUDA stream (cudaStream_t passed as void*; NULL = legacy default
- * stream).  On the device current at the call it also commits the fixed scratch arrays of
- * tmbir_normal_apply_static (67 MiB, held until the process exits) and caches their addresses;
- * fails with TMBIR_ERR_CUDA if that device cannot hold them.
+ * stream).  On the device current at the call it also commits the fixed scratch array of
+ * tmbir_normal_apply_static (64 MiB, held until the process exits) and caches its address;
+ * fails with TMBIR_ERR_CUDA if that device cannot hold it.
  */
 int tmbir_create(tmbir_ctx** out, void* stream);
 int tmbir_destroy(tmbir_ctx* ctx);
@@ -373,15 +373,16 @@ int tmbir_warm_start(tmbir_ctx* ctx, tmbir_cnn* net, const float* d_fbp, const f
 
 /*
  * tmbir_normal_apply without device scratch from the workspace: the same d_z = R*R d_x, with the
- * intermediate spectra and reduction partials in a fixed array inside the library.  The paper
+ * intermediate spectra in a fixed array inside the library.  The paper
  * has no counterpart; this entry point is for callers that cannot allocate device memory at the
  * time of the call (for example code running under a host application that owns the whole
  * device-memory budget, or a latency-critical loop where allocation is not allowed).
- *   - The array holds 8 Mi complex values (64 MiB) of spectra, (N+1) * N per slice, and the
- *     partial sums of 65536 blocks.  The groups run one after another in chunks of as many
- *     slices as fit (at most the context's spectrum chunk); a geometry whose pass 3b needs
- *     more than 65536 blocks is rejected with TMBIR_ERR_SHAPE; nothing is allocated on any
- *     path.
+ *   - The array holds 8 Mi complex values (64 MiB) of spectra, (N+1) * N per slice.  The groups
+ *     run one after another in chunks of as many slices as fit (at most the context's spectrum
+ *     chunk).  A geometry of more than 65536 blocks is rejected with TMBIR_ERR_SHAPE, counting
+ *     per group its bands of 4 rows by up to 512 columns times its slice chunks (about
+ *     1216 / bands of them, at most one per slice; after tmbir_autotune chunks of the chosen
+ *     slices per block).  Nothing is allocated on any path.
  *   - Every device that loads the library holds the array until the process exits.  The
  *     memory is committed when tmbir_create runs with that device current (it looks up the
  *     array's device address with cudaGetSymbolAddress, which loads the module holding it, and

@@ -85,3 +85,37 @@ def test_static_scratch_two_groups_with_chunks():
             err = float(torch.linalg.norm(a - b) / torch.linalg.norm(b))
             assert err < 1e-5, (N, err)
             off += n
+
+
+@pytest.mark.parametrize("N,S", [(64, 512), (256, 3)])
+def test_static_launches_what_the_workspace_path_does(N, S):
+    # the result is pass 3a's: a fourth kernel that only forms sums nobody reads cost 142 of 181 us at
+    # 512 slices of 64^2
+    ctx = tm.Context([tm.Group(N=N, angles=[0.0], n_slices=S)])
+    ctx.build_operator(torch.zeros(S * N, device="cuda"))
+    x = _dev(synth.random_image(np.random.default_rng(11), (S, N, N)))
+    counts = []
+    for apply in (ctx.normal_apply, ctx.normal_apply_static):
+        n0 = ctx.launch_count()
+        z = apply(x)
+        counts.append(ctx.launch_count() - n0)
+    torch.cuda.synchronize()
+    assert counts[0] == counts[1] == 3, counts
+    assert torch.equal(z, ctx.normal_apply(x))
+
+
+@pytest.mark.parametrize("extra,refused", [(0, False), (1, True)])
+def test_static_block_limit(extra, refused):
+    # 64^2: 16 bands, 76 slices in 76 chunks, so 1216 blocks a group; 53 groups and a slice chunk more
+    # or less stand on the two sides of the documented 65536
+    tail = 68 + extra  # 53 * 1216 + 16 * 68 = 65536
+    groups = [tm.Group(N=64, angles=[0.0], n_slices=76) for _ in range(53)] + [tm.Group(N=64, angles=[0.0], n_slices=tail)]
+    ctx = tm.Context(groups)
+    ctx.build_operator(torch.zeros(ctx.sino_numel(), device="cuda"))
+    x = torch.ones(ctx.image_numel(), device="cuda")
+    if refused:
+        with pytest.raises(tm.TmbirError) as e:
+            ctx.normal_apply_static(x)
+        assert e.value.code == -2
+    else:
+        assert torch.equal(ctx.normal_apply_static(x), ctx.normal_apply(x))
