@@ -1276,8 +1276,9 @@ int forward_project(Ctx& c, int gi, const float* d_x, float* d_sino, cudaStream_
   float2* tw_f = reinterpret_cast<float2*>(c.scratch);
   float2* tw_d = tw_f + nf;
   float2* grid = tw_d + nd;
-  float2* tmp = grid + (size_t)PB * cells;
-  float2* prow = tmp + (size_t)PB * cells;
+  const size_t pairs = (B + 1) / 2;  // as forward_scratch_bytes counts them, not PB
+  float2* tmp = grid + pairs * cells;
+  float2* prow = tmp + pairs * cells;
   if (int e = twiddles<float2>(tw_f, nf, s)) return e;
   if (int e = twiddles<float2>(tw_d, nd, s)) return e;
   for (int b0 = 0; b0 < g.S; b0 += B) {

@@ -110,3 +110,17 @@ def test_n2048_limited_angle_direct_gradient(orc):
         ref = (orc.normal_point(x64[z], K, r, c) - orc.adjoint_point(g[z], N, p.theta, r, c)
                + orc.prior_point(x64, pr, z, r, c))
         assert abs(G[z, r, c] - ref) <= 1e-5 * gscale
+
+
+# a batch of fewer slices than the largest uses as much scratch as its pairs need: 2560^2, whose
+# kernel is summed directly and leaves the smallest scratch beside the grids
+@pytest.mark.parametrize("N,S", [(2560, 1), (2560, 5), (2560, 9), (1536, 3)])
+def test_forward_scratch_of_small_batches(N, S):
+    ctx = tm.Context([tm.Group(N=N, angles=[0.0, math.pi / 2], n_slices=S)])
+    x = np.random.default_rng(N + S).standard_normal((S, N, N)).astype(np.float32)
+    Rx = host(ctx.forward(dev(x)), (S, 2, N))
+    # along the axes the bins are pixel columns and rows: their sums without the Nyquist term
+    ref = np.stack([x.sum(1, dtype=np.float64), x.sum(2, dtype=np.float64)], 1)
+    alt = (-1.0) ** np.arange(N)
+    ref -= (ref @ alt)[..., None] * alt / N
+    assert rel(Rx, ref) < 1e-5
