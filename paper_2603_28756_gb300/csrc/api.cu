@@ -39,6 +39,8 @@ PriorC make_prior(const tmbir_params& p) {
   c.l2_inv_csig = (float)std::log2(1.0 / (p.c * p.sigma));
   c.qp_l2_inv_csig = (float)((p.q - p.p) * std::log2(1.0 / (p.c * p.sigma)));
   c.l2_inv_sig = (float)std::log2(1.0 / p.sigma);
+  // |y| <= pair_lim keeps (d / (c sigma))^(q-p) of a difference, |d| <= 2 pair_lim, below 2^62 and d^2 below 2^126
+  c.pair_lim = (float)std::min(0.5 * p.c * p.sigma * std::exp2(std::min(62.0 / (p.q - p.p), 1000.0)), 0x1p62);
   return c;
 }
 

@@ -79,6 +79,7 @@ struct PriorC {
   float l2_inv_sig;      // log2(1 / sigma)
   int q_is_2;
   int nonneg;            // project each iterate onto x >= 0
+  float pair_lim;        // q = 2: up to this |y| a pair of differences may share a reciprocal (pairv)
 };
 
 // One geometry group as the kernels see it (device pointers into the workspace).

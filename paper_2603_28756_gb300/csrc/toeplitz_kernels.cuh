@@ -133,6 +133,12 @@ __device__ __forceinline__ float rcpa(float x) {
 
 // Packed FP32 pairs: one instruction computes both lanes of a float2 (sm_100 and later).
 __device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
+// the largest of three values, NaN if one of them is
+__device__ __forceinline__ float max_nan(float a, float b, float c) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
 __device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 f2mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 f2add(float2 a, float2 b) { return __fadd2_rn(a, b); }
@@ -755,11 +761,13 @@ struct GeoP {
 // grid, holds rows r0 - 1 + i (first halves) and r0 - 1 + i + R (second halves) at columns
 // c0 - 4 + 4 q .. + 3.  ld(row index 0 .. 2R + 1, q, which) gives the float4 of x (0) or x_prev (1).
 // A thread keeps its column and takes every fourth row; the two halo columns of all rows go to the
-// first threads.
+// first threads.  Returns the largest |y| of the thread's values, NaN if one of them is.
 template <int N, class Ld>
-__device__ __forceinline__ void fill_ring(float2* slot, float beta, Ld&& ld) {
+__device__ __forceinline__ float fill_ring(float2* slot, float beta, Ld&& ld) {
   using GP = GeoP<N>;
   constexpr int QB = GP::BC / 4;
+  float top = 0.f;
+  auto see = [&](float2 y) { top = max_nan(top, fabsf(y.x), fabsf(y.y)); };
   const float2 b2 = f2(beta);
   auto yv = [&](float2 x, float2 p) { return f2fma(b2, make_float2(x.x - p.x, x.y - p.y), x); };
   auto put = [&](int i, int q) {
@@ -771,6 +779,10 @@ __device__ __forceinline__ void fill_ring(float2* slot, float beta, Ld&& ld) {
     float4* d = reinterpret_cast<float4*>(slot + i * GP::LDR + 4 * q);
     d[0] = make_float4(y0.x, y0.y, y1.x, y1.y);
     d[1] = make_float4(y2.x, y2.y, y3.x, y3.y);
+    see(y0);
+    see(y1);
+    see(y2);
+    see(y3);
   };
   const int q = threadIdx.x % QB + 1, i0 = threadIdx.x / QB;
 #pragma unroll
@@ -779,12 +791,13 @@ __device__ __forceinline__ void fill_ring(float2* slot, float beta, Ld&& ld) {
   // (from the other end of the block, whose threads have fewer rows)
   const int e = GP::THREADS - 1 - threadIdx.x;
   if (e < 2 * (GP::R + 2)) put(e >> 1, (e & 1) * (QB + 1));
+  return top;
 }
 // from global memory (zero outside the image)
 template <int N>
-__device__ __forceinline__ void load_ring_p(float2* slot, const float* x, const float* xp, float beta,
-                                            size_t off_slice, int r0, int c0) {
-  fill_ring<N>(slot, beta, [&](int i, int q, int which) {
+__device__ __forceinline__ float load_ring_p(float2* slot, const float* x, const float* xp, float beta,
+                                             size_t off_slice, int r0, int c0) {
+  return fill_ring<N>(slot, beta, [&](int i, int q, int which) {
     const int rr = r0 - 1 + i, cc = c0 - 4 + 4 * q;
     if (rr < 0 || rr >= N || cc < 0 || cc >= N) return make_float4(0.f, 0.f, 0.f, 0.f);
     return __ldg(reinterpret_cast<const float4*>((which ? xp : x) + off_slice + (size_t)rr * N + cc));
@@ -825,9 +838,9 @@ struct Stager {
   }
 };
 template <int N>
-__device__ __forceinline__ void stage_to_ring(float2* slot, const float* stg, float beta) {
+__device__ __forceinline__ float stage_to_ring(float2* slot, const float* stg, float beta) {
   using GP = GeoP<N>;
-  fill_ring<N>(slot, beta, [&](int i, int q, int which) {
+  return fill_ring<N>(slot, beta, [&](int i, int q, int which) {
     return reinterpret_cast<const float4*>(stg + which * GP::STG + i * GP::LDR)[q];
   });
 }
@@ -861,26 +874,33 @@ __device__ __forceinline__ PairK pair_k(const PriorC& c) {
 // Unweighted pair value v = sigma^2 rho'(nb - y) of two pairs at once from n = -y, with the identity
 //   sigma^2 rho'(d) = d |d/sigma|^(q-2) r (p + (q - p) r), r = 1 / (1 + |d/(c sigma)|^(q-p)).
 // With PH, ph += sigma^2 rho(d) = d^2 |d/sigma|^(q-2) r (unweighted).  MX, MY: the first / second
-// half counts only when okx / oky.  For q = 2 the exponent is at most 1 and s is limited to 63 (a
-// difference of 10^19 times c sigma), so that the product of the two e stays finite; log2 0 = -inf
-// gives r = 1 there, and d = 0 ends both terms.  For q != 2 the logarithm is kept finite, since the
-// second exponential would meet it with a negative factor.
-template <bool Q2, bool PH, bool MX, bool MY>
+// half counts only when okx / oky.  For q = 2 the two halves share one reciprocal, which needs the
+// product of the two e to be finite; WIDE gives each its own, for slices with values past
+// PriorC::pair_lim (or not finite, which would spread from one half to the other).  The values are
+// looked at when they enter the ring: limiting the exponents here instead took two minima a pair (0.704
+// against 0.698 ms at 64 x 1024^2, 1.307 against 1.303 at 32 x 2048^2; a launch at 1 x 128^2 is 0.2 us
+// faster with them) and gave wrong gradients past the limit.  log2 0 = -inf
+// gives r = 1, and d = 0 ends both terms; WIDE takes 2 log2 |d|, whose range d^2 does not have.  For
+// q != 2 the logarithm is kept finite, since the second exponential would meet it with a negative factor.
+template <bool Q2, bool PH, bool MX, bool MY, bool WIDE>
 __device__ __forceinline__ float2 pairv(float2 n, float2 nb, const PairK& k, bool okx, bool oky, float2& ph) {
   float2 d = f2add(nb, n);
   if constexpr (MX) d.x = okx ? d.x : 0.f;
   if constexpr (MY) d.y = oky ? d.y : 0.f;
-  const float2 sq = Q2 ? f2mul(d, d) : f2fma(d, d, f2(1e-30f));
-  const float2 la = make_float2(lg2a(sq.x), lg2a(sq.y));
-  float2 s = f2fma(k.half_qp, la, k.qp_l2);
+  float2 la;
+  if constexpr (Q2 && WIDE) {
+    la = f2mul(make_float2(lg2a(fabsf(d.x)), lg2a(fabsf(d.y))), f2(2.f));
+  } else {
+    const float2 sq = Q2 ? f2mul(d, d) : f2fma(d, d, f2(1e-30f));
+    la = make_float2(lg2a(sq.x), lg2a(sq.y));
+  }
+  const float2 s = f2fma(k.half_qp, la, k.qp_l2);
+  const float2 e = f2add(make_float2(ex2a(s.x), ex2a(s.y)), k.one);
   float2 r;
-  if constexpr (Q2) {
-    s = make_float2(fminf(s.x, 63.f), fminf(s.y, 63.f));
-    const float2 e = f2add(make_float2(ex2a(s.x), ex2a(s.y)), k.one);
+  if constexpr (Q2 && !WIDE) {
     const float ri = rcpa(e.x * e.y);
     r = make_float2(ri * e.y, ri * e.x);
   } else {
-    const float2 e = f2add(make_float2(ex2a(s.x), ex2a(s.y)), k.one);
     r = make_float2(rcpa(e.x), rcpa(e.y));
   }
   float2 dr = f2mul(d, r);
@@ -961,14 +981,14 @@ __device__ __forceinline__ OuterItem outer_item(bool cross, const float2 (&w)[3]
   return it;
 }
 // the weighted value of the lane's outer pair, and its sums over the lanes of the same row
-template <int N, bool Q2, bool ROWE>
+template <int N, bool Q2, bool ROWE, bool WIDE>
 __device__ __forceinline__ void outer_sums(const float2* S0, const float2* T, const OuterItem& it, const PairK& k,
                                            float2& v, float2& v2, float2& v3) {
   constexpr int R = GeoP<N>::R;
   float2 unused = f2(0.f);
   const float2 sv = S0[it.src];
-  v = pairv<Q2, false, true, true>(make_float2(-sv.x, -sv.y), T[it.tgt], k, it.on && (!ROWE || it.okx),
-                                   it.on && (!ROWE || it.oky), unused);
+  v = pairv<Q2, false, true, true, WIDE>(make_float2(-sv.x, -sv.y), T[it.tgt], k, it.on && (!ROWE || it.okx),
+                                         it.on && (!ROWE || it.oky), unused);
   v = f2mul(f2(it.w), v);
   float2 a, b;
   a.x = __shfl_down_sync(0xffffffffu, v.x, R);
@@ -988,8 +1008,8 @@ __device__ __forceinline__ void outer_sums(const float2* S0, const float2* T, co
 // complete, with h = -(the prior gradient) and ph the unweighted sigma^2 rho sums by class of the
 // pairs whose target row the band owns.  w: class weights w / sigma^2 (face, edge, corner).  ROWE:
 // the block holds the image's first or last rows; COLE: the warp holds its first or last columns.
-// Elsewhere every neighbour lies inside the image and the boundary tests drop out.
-template <int N, bool Q2, bool PHI, bool PRE, bool ROWE, bool COLE, class Pre, class Fin>
+// Elsewhere every neighbour lies inside the image and the boundary tests drop out.  WIDE: see pairv.
+template <int N, bool Q2, bool PHI, bool PRE, bool ROWE, bool COLE, bool WIDE, class Pre, class Fin>
 __device__ __forceinline__ void band_step(const float2* S0, const float2* S1, bool have1, const BandB& bb,
                                           const OuterItem& it, const OuterItem& itx, int ic, float2* cr, float2* edge,
                                           const float2* xin, float2* xout, const PairK& k, const float2 (&w)[3],
@@ -1006,12 +1026,12 @@ __device__ __forceinline__ void band_step(const float2* S0, const float2* S1, bo
   {
     float2 v, v2, v3;
     if constexpr (!PRE) {
-      outer_sums<N, Q2, ROWE>(S0, S0, it, k, v, v2, v3);
+      outer_sums<N, Q2, ROWE, WIDE>(S0, S0, it, k, v, v2, v3);
       if (lane < R) edge[lane] = v2;
       if (lane >= 2 * R && lane < 3 * R) edge[lane - R] = v;
     }
     if (have1 && (warp == 0 || warp == GP::WPB - 1)) {
-      outer_sums<N, Q2, ROWE>(S0, S1, itx, k, v, v2, v3);
+      outer_sums<N, Q2, ROWE, WIDE>(S0, S1, itx, k, v, v2, v3);
       if (lane < R) edge[2 * R + lane] = v3;
     }
   }
@@ -1044,8 +1064,8 @@ __device__ __forceinline__ void band_step(const float2* S0, const float2* S1, bo
     constexpr int DX = decltype(DX_)::value;
     constexpr bool C = COLE && DX != 0;
     const bool okc = DX < 0 ? bb.okL : bb.okR;
-    return pairv<Q2, decltype(PH_)::value, ROWE || C, ROWE || C>(n, nb, k, (!ROWE || mx) && (!C || okc),
-                                                                 (!ROWE || my) && (!C || okc), p);
+    return pairv<Q2, decltype(PH_)::value, ROWE || C, ROWE || C, WIDE>(n, nb, k, (!ROWE || mx) && (!C || okc),
+                                                                       (!ROWE || my) && (!C || okc), p);
   };
   using Lf = std::integral_constant<int, -1>;
   using Ce = std::integral_constant<int, 0>;
@@ -1150,6 +1170,8 @@ __global__ void __launch_bounds__(GeoP<N>::THREADS, 512 / GeoP<N>::THREADS)
   constexpr bool UPDATE = MODE == (int)Pass3Mode::Step || MODE == (int)Pass3Mode::Iterate;
   extern __shared__ float2 sm[];
   __shared__ double red[GP::WPB * kParts];
+  __shared__ std::conditional_t<GP::WPB == 2, uint16_t, uint32_t> past_lim[2];  // a byte per warp and ring slot
+  static_assert(GP::WPB == 2 || GP::WPB == 4, "a byte per warp");
   int bid_;
   const int gi_ = gs.template pick<MULTI>(bid_);
   const GroupDev& g = gs.g[MULTI ? gi_ : 0];
@@ -1228,9 +1250,17 @@ __global__ void __launch_bounds__(GeoP<N>::THREADS, 512 / GeoP<N>::THREADS)
     // shares[parity]: [side][warp + 1][row]; the places beyond the block's warps stay zero
     for (int i = threadIdx.x; i < 2 * GP::XCH; i += GP::THREADS) xch[i] = f2(0.f);
     float2 ph[3] = {f2(0.f), f2(0.f), f2(0.f)};
-    load_ring_p<N>(ring + (z0 & 1) * GP::RING, x, xp, beta, (size_t)z0 * N2, r0, c0);
+    // every warp notes whether its part of a ring slot holds values past the limit of the shared
+    // reciprocal; the block's answer is the same wherever the slice is held, in any division into chunks
+    auto note = [&](int z, float top) {
+      if constexpr (Q2) {
+        const bool past = __any_sync(0xffffffffu, !(top <= pc.pair_lim));
+        if ((threadIdx.x & 31) == 0) reinterpret_cast<bool*>(&past_lim[z & 1])[warp] = past;
+      }
+    };
+    note(z0, load_ring_p<N>(ring + (z0 & 1) * GP::RING, x, xp, beta, (size_t)z0 * N2, r0, c0));
     if (z0 > 0) {
-      load_ring_p<N>(ring + ((z0 - 1) & 1) * GP::RING, x, xp, beta, (size_t)(z0 - 1) * N2, r0, c0);
+      note(z0 - 1, load_ring_p<N>(ring + ((z0 - 1) & 1) * GP::RING, x, xp, beta, (size_t)(z0 - 1) * N2, r0, c0));
     } else {
 #pragma unroll
       for (int t = 0; t < R; ++t) cr[t * GP::THREADS] = f2(0.f);
@@ -1247,18 +1277,22 @@ __global__ void __launch_bounds__(GeoP<N>::THREADS, 512 / GeoP<N>::THREADS)
       const float2* s1 = ring + (z0 & 1) * GP::RING;
       float2* xo0 = xch + (z0 & 1) * GP::XCH;
       const float2* xi0 = xo0;  // not read
-      if (rowe || cole)
-        band_step<N, Q2, PHI, true, true, true>(s0, s1, true, bb, it, itx, ic, cr, edge, xi0, xo0, pk, w, ph, none, fin0);
+      if (Q2 && (past_lim[0] | past_lim[1]))
+        band_step<N, Q2, PHI, true, true, true, true>(s0, s1, true, bb, it, itx, ic, cr, edge, xi0, xo0, pk, w, ph, none, fin0);
+      else if (rowe || cole)
+        band_step<N, Q2, PHI, true, true, true, false>(s0, s1, true, bb, it, itx, ic, cr, edge, xi0, xo0, pk, w, ph, none, fin0);
       else
-        band_step<N, Q2, PHI, true, false, false>(s0, s1, true, bb, it, itx, ic, cr, edge, xi0, xo0, pk, w, ph, none, fin0);
+        band_step<N, Q2, PHI, true, false, false, false>(s0, s1, true, bb, it, itx, ic, cr, edge, xi0, xo0, pk, w, ph, none, fin0);
     }
     for (int z = z0; z < z1; ++z) {
       // every thread has finished slice z - 1, so its ring slot takes slice z + 1 from the
       // staging area; then the staging area takes slice z + 2 while slice z is worked on
       tc05::cp_async_wait_all();
       __syncthreads();
-      if (z + 1 < S) stage_to_ring<N>(ring + ((z + 1) & 1) * GP::RING, stg, beta);
-      __syncthreads();
+      if (z + 1 < S) {
+        note(z + 1, stage_to_ring<N>(ring + ((z + 1) & 1) * GP::RING, stg, beta));
+        __syncthreads();
+      }
       if (z + 1 < z1 && z + 2 < S) stager.issue((size_t)(z + 2) * N2);
       float2 acc[kParts];
 #pragma unroll
@@ -1305,10 +1339,12 @@ __global__ void __launch_bounds__(GeoP<N>::THREADS, 512 / GeoP<N>::THREADS)
       const float2* s1 = ring + ((z + 1) & 1) * GP::RING;
       const float2* xi = xch + (z & 1) * GP::XCH;        // what slice z - 1 handed over
       float2* xo = xch + ((z + 1) & 1) * GP::XCH;
-      if (rowe || cole)
-        band_step<N, Q2, PHI, false, true, true>(s0, s1, z + 1 < S, bb, it, itx, ic, cr, edge, xi, xo, pk, w, ph, pre, fin);
+      if (Q2 && (past_lim[z & 1] | (z + 1 < S ? past_lim[(z + 1) & 1] : 0)))
+        band_step<N, Q2, PHI, false, true, true, true>(s0, s1, z + 1 < S, bb, it, itx, ic, cr, edge, xi, xo, pk, w, ph, pre, fin);
+      else if (rowe || cole)
+        band_step<N, Q2, PHI, false, true, true, false>(s0, s1, z + 1 < S, bb, it, itx, ic, cr, edge, xi, xo, pk, w, ph, pre, fin);
       else
-        band_step<N, Q2, PHI, false, false, false>(s0, s1, z + 1 < S, bb, it, itx, ic, cr, edge, xi, xo, pk, w, ph, pre, fin);
+        band_step<N, Q2, PHI, false, false, false, false>(s0, s1, z + 1 < S, bb, it, itx, ic, cr, edge, xi, xo, pk, w, ph, pre, fin);
       if constexpr (PHI) {
 #pragma unroll
         for (int j = 0; j < 3; ++j) {

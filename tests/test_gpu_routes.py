@@ -102,3 +102,47 @@ def test_prior_bands(orc, N, S, p, scale):
     G0 = host(ctx.gradient(dev(x), zero, tm.Params(**prm, lam=0.0)), x.shape)
     ref = orc.prior(x.astype(np.float64), orc.Prior(**prm, lam=lam))[0]
     assert rel(G - G0, ref) < 1e-5
+
+
+def _prior_gradient(x, prm, lam):
+    S, N = x.shape[0], x.shape[1]
+    ctx = tm.Context([tm.Group(N=N, angles=list(synth.angles(4)), n_slices=S)])
+    ctx.build_operator(torch.zeros(S * 4 * N, device="cuda"))
+    zero = torch.zeros(S * N * N, device="cuda")
+    G = host(ctx.gradient(dev(x), zero, tm.Params(**prm, lam=lam, L=1.0)), x.shape)
+    return G - host(ctx.gradient(dev(x), zero, tm.Params(**prm, lam=0.0, L=1.0)), x.shape)
+
+
+# pass 3b: differences of up to 2^66 times c sigma, and around 2^62 times (where the two halves of a pair
+# stop sharing a reciprocal), everywhere and in every second band only.  The exponent of
+# r = 1 / (1 + 2^s) has an error of about 2^-24 s, s <= 66: 4e-6 of the pair's value
+@pytest.mark.parametrize("N,p,sigma,scale", [(64, 1.0, 1e-18, 1.0), (512, 1.0, 1e-18, 1.0), (512, 1.0, 2.2e-17, 1.0),
+                                             (512, 1.2, 1e-18, 1e4), (128, 1.2, 1e-18, 1e4)])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_prior_at_huge_differences(orc, N, p, sigma, scale, mixed):
+    S, R = 2, 8 if N >= 512 else 4
+    x = synth.random_image(np.random.default_rng(N), (S, N, N), scale).astype(np.float32)
+    r = np.arange(N)
+    small = (r // R) % 2 == 1 if mixed else np.zeros(N, bool)
+    x[:, small] *= np.float32(1e-12)
+    prm = dict(p=p, q=2.0, c=0.01, sigma=sigma)
+    lam = 1e12 * sigma  # the data term's rounding does not count
+    G = _prior_gradient(x, prm, lam)
+    ref = orc.prior(x.astype(np.float64), orc.Prior(**prm, lam=lam))[0]
+    assert rel(G[:, ~small], ref[:, ~small]) < 1e-5
+    if mixed:  # the rows whose neighbours are all small
+        inner = small & (r % R > 0) & (r % R < R - 1)
+        assert rel(G[:, inner], ref[:, inner]) < 1e-5
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_prior_keeps_a_bad_voxel_to_its_neighbours(bad):
+    # the data term spreads it over its slice; in the slices before and after only the prior reads it
+    S, N, r, c = 3, 512, 37, 131
+    x = synth.random_image(np.random.default_rng(3), (S, N, N)).astype(np.float32)
+    x[1, r, c] = bad
+    G = _prior_gradient(x, dict(p=1.2, q=2.0, c=0.01, sigma=0.1), 1.0)
+    want = np.zeros((N, N), bool)
+    want[r - 1:r + 2, c - 1:c + 2] = True
+    for z in (0, 2):
+        assert np.array_equal(~np.isfinite(G[z]), want)
