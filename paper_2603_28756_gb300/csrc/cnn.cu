@@ -699,15 +699,54 @@ __global__ void __launch_bounds__(256) k_wgrad_edge(const __nv_bfloat16* __restr
     }
   }
 }
+enum class Layer { First, Hidden, Last };
+
+// One block's share of weight i's sum in k_wgrad32 (Hidden: h = g) or k_wgrad_edge, product by product
+// and without those outside the image.
+template <Layer L>
+__device__ __noinline__ float wgrad_inside(const __nv_bfloat16* h, const void* other, int B, int H, int W, int block,
+                                           int nblocks, int i) {
+  constexpr int TH = L == Layer::Hidden ? kGRows : kEH, TW = L == Layer::Hidden ? kTM : kEW;
+  const int tap = i % 9, dy = tap / 3 - 1, dx = tap % 3 - 1, ci = i / 9 % kC, c = L == Layer::Hidden ? i / (9 * kC) : ci;
+  const int tiles_x = (W + TW - 1) / TW, tiles_y = (H + TH - 1) / TH;
+  float s = 0.f;
+  for (int tile = block; tile < B * tiles_y * tiles_x; tile += nblocks) {
+    const int x0 = tile % tiles_x * TW, y0 = tile / tiles_x % tiles_y * TH;
+    const size_t plane = (size_t)(tile / (tiles_x * tiles_y)) * H;
+    for (int q = 0; q < TH * TW; ++q) {
+      const int y = y0 + q / TW, hx = x0 + q % TW;  // Hidden: y is the row of the layer's input
+      const int hy = L == Layer::Hidden ? y - dy : y, oy = L == Layer::Hidden ? y : (L == Layer::First ? y + dy : y - dy);
+      const int ox = L == Layer::Last ? hx - dx : hx + dx;
+      if (hy < 0 || hy >= H || hx >= W || oy < 0 || oy >= H || ox < 0 || ox >= W) continue;
+      const size_t o = (plane + oy) * W + ox;
+      const float f = L == Layer::Hidden ? __bfloat162float(static_cast<const __nv_bfloat16*>(other)[o * kC + ci])
+                                         : static_cast<const float*>(other)[o];
+      s = fmaf(__bfloat162float(h[((plane + hy) * W + hx) * kC + c]), f, s);
+    }
+  }
+  return s;
+}
+
 // dst[i] += sum over blocks of part[b][i], i < n, in FP64: eight threads per element take every
-// eighth block, then their sums in order
+// eighth block, then their sums in order.  The blocks multiply infinities and NaN beside the border by
+// the zeros staged outside the image, which makes NaN of sums that such a value is not part of: where
+// a weight's sum is not finite, its blocks' shares are formed again without those products.
+template <Layer L>
 __global__ void __launch_bounds__(256) k_reduce_parts(const float* __restrict__ part, int nblocks, int n,
-                                                      float* __restrict__ dst) {
+                                                      float* __restrict__ dst, const __nv_bfloat16* h, const void* other,
+                                                      int B, int H, int W) {
   __shared__ double sh[8][32];
   const int i = blockIdx.x * 32 + (threadIdx.x & 31), r = threadIdx.x >> 5;
   double s = 0.0;
   if (i < n)
     for (int b = r; b < nblocks; b += 8) s += part[(size_t)b * kPartRow + i];
+  if (i < (L == Layer::Hidden ? kW1 : kW0) && !isfinite(s)) {
+    s = 0.0;
+    for (int b = r; b < nblocks; b += 8) {
+      const float v = part[(size_t)b * kPartRow + i];
+      s += isfinite(v) ? v : wgrad_inside<L>(h, other, B, H, W, b, nblocks, i);
+    }
+  }
   sh[r][threadIdx.x & 31] = s;
   __syncthreads();
   if (r == 0 && i < n) {
@@ -870,7 +909,8 @@ static int wgrad32(CnnNet& n, int B, const __nv_bfloat16* g, const __nv_bfloat16
   const int blocks = std::min(tiles, kWgradBlocks);
   k_wgrad32<<<blocks, 128, kGradSmem, n.stream>>>(g, in, B, n.H, n.W, n.wpart, n.err);
   TMBIR_CHECK_LAUNCH();
-  k_reduce_parts<<<(kPartRow + 31) / 32, 256, 0, n.stream>>>(n.wpart, blocks, kPartRow, n.grad + off);
+  k_reduce_parts<Layer::Hidden><<<(kPartRow + 31) / 32, 256, 0, n.stream>>>(n.wpart, blocks, kPartRow, n.grad + off, g, in,
+                                                                            B, n.H, n.W);
   TMBIR_CHECK_LAUNCH();
   return TMBIR_OK;
 }
@@ -884,7 +924,8 @@ static int net_backward(CnnNet& n, int B, float* gin) {
   // layer 3
   k_wgrad_edge<false><<<eblocks, 256, 0, n.stream>>>(n.a2, n.gout, B, n.H, n.W, n.wpart);
   TMBIR_CHECK_LAUNCH();
-  k_reduce_parts<<<(kW3 + kB3 + 31) / 32, 256, 0, n.stream>>>(n.wpart, eblocks, kW3 + kB3, n.grad + kOff3);
+  k_reduce_parts<Layer::Last><<<(kW3 + kB3 + 31) / 32, 256, 0, n.stream>>>(n.wpart, eblocks, kW3 + kB3, n.grad + kOff3, n.a2,
+                                                                           n.gout, B, n.H, n.W);
   TMBIR_CHECK_LAUNCH();
   k_last_dgrad<<<blocks, 256, 0, n.stream>>>(n.gout, n.a2, B, n.H, n.W, n.master, n.g2);
   TMBIR_CHECK_LAUNCH();
@@ -898,7 +939,8 @@ static int net_backward(CnnNet& n, int B, float* gin) {
   // layer 0
   k_wgrad_edge<true><<<eblocks, 256, 0, n.stream>>>(g0, n.xin, B, n.H, n.W, n.wpart);
   TMBIR_CHECK_LAUNCH();
-  k_reduce_parts<<<(kW0 + kB0 + 31) / 32, 256, 0, n.stream>>>(n.wpart, eblocks, kW0 + kB0, n.grad + kOff0);
+  k_reduce_parts<Layer::First><<<(kW0 + kB0 + 31) / 32, 256, 0, n.stream>>>(n.wpart, eblocks, kW0 + kB0, n.grad + kOff0, g0,
+                                                                            n.xin, B, n.H, n.W);
   TMBIR_CHECK_LAUNCH();
   if (gin) {
     k_conv_last<true><<<blocks, 256, 0, n.stream>>>(g0, B, n.H, n.W, n.master, gin);

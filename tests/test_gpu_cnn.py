@@ -179,3 +179,25 @@ def test_trained_network_improves_the_start():
         sb = ctx.reconstruct(b, atg, tm.Params(**PRIOR, max_iter=20))
         assert sb.objective < sa.objective
     assert min(gains) > 1.5
+
+
+# values that are not finite, beside the border, beside a tile's edge and inside: exactly the gradients
+# that such a value is part of are not finite
+@pytest.mark.parametrize("where,pos,value", [("gout", (0, 0), math.nan), ("gout", (7, 199), math.inf),
+                                             ("gout", (10, 127), math.inf), ("x", (0, 0), math.inf),
+                                             ("x", (10, 199), math.inf), ("x", (5, 128), -math.inf)])
+def test_backward_not_finite(orc, where, pos, value):
+    B, H, W = 1, 11, 200
+    rng = np.random.default_rng(6)
+    p = robust_params(orc, 3)
+    x = rng.uniform(-0.5, 0.5, (B, H, W)).astype(np.float32)
+    gout = rng.standard_normal((B, H, W)).astype(np.float32)
+    (gout if where == "gout" else x)[(0,) + pos] = value
+    net = tm.CNN(H, W, max_batch=B)
+    net.set_weights(p)
+    gp, gin = net.net_backward(dev(x), dev(gout), B)
+    torch.cuda.synchronize()
+    rgp, rgin = orc.cnn_backward(x.astype(np.float64), p, gout.astype(np.float64))
+    assert 0 < np.isfinite(rgp).sum() < rgp.size
+    assert np.array_equal(np.isfinite(gp), np.isfinite(rgp))
+    assert np.array_equal(np.isfinite(gin.cpu().numpy().reshape(rgin.shape)), np.isfinite(rgin))
