@@ -170,6 +170,11 @@ __device__ __forceinline__ void block_partials(double (&acc)[kParts], double* re
 // rounding is 2^15 times larger
 template <int DIR, bool BF>
 constexpr int kRowDir = BF ? DIR : 2 * DIR;
+// and pass 2's at 1536, whose columns rotate by odd multiples of pi/4 more often than in the four radix
+// stages that the 512-point split replaced: without it R*R's error there is 2.63e-7 (4 slices of noise, 64
+// angles), with it 2.53e-7, with the stages 2.58e-7.  8 x 1536^2: 143 -> 148 us
+template <int DIR, int N, bool BF>
+constexpr int kColDir = !BF && N == 1536 ? 2 * DIR : DIR;
 
 // ---------------------------------------------------------------- pass 1: rows, forward
 template <int N, bool BF>
@@ -402,7 +407,7 @@ __global__ void TMBIR_P3A_BOUNDS(Geo3a<N>::THREADS) k_pass3a(const __grid_consta
 // layouts save: twiddles come from tables that are contiguous in m (W^m, W^2m, W^4m, W^8m; the others
 // are one product of two of these), the kernel spectrum is stored per j, and for J = 4 a staged row
 // keeps the four residues of v apart (stride-4 accesses would meet in four banks).  Measured per
-// launch, pass 1 / 2 / 3a: 6 x 2560^2 177 / 369 / 179 us, 8 x 1536^2 92 / 144 / 96 us (632 / 1215 /
+// launch, pass 1 / 2 / 3a: 6 x 2560^2 177 / 369 / 179 us, 8 x 1536^2 92 / 148 / 96 us (632 / 1215 /
 // 570 and 188 / 448 / 212 us with the four-stage block-wide Stockham transform, five round trips with a
 // block barrier each, that this replaced); 32 x 2048^2 540 / 932 / 582 us (707 / 1026 / 690 us with
 // 1024-point transforms of one warp).
@@ -566,10 +571,10 @@ __global__ void __launch_bounds__(GeoH<N>::THREADS2) k_pass2_h(const __grid_cons
       tw_powers<0>(g, m, w);
       SFor<0, J>::run([&](auto q_) {
         constexpr int q = decltype(q_)::value;
-        o[q] = twmul<q, J2, -1>(c[k][q]);
+        o[q] = twmul<q, J2, kColDir<-1, N, BF>>(c[k][q]);
       });
-      reg_dft<J, -1, float2>(c[k]);
-      reg_dft<J, -1, float2>(o);
+      reg_dft<J, kColDir<-1, N, BF>, float2>(c[k]);
+      reg_dft<J, kColDir<-1, N, BF>, float2>(o);
       SFor<0, J>::run([&](auto i_) {
         constexpr int i = decltype(i_)::value;
         sm[2 * i * F::SMEM + m] = i ? cmul(c[k][i], w[2 * i]) : c[k][i];
@@ -585,7 +590,7 @@ __global__ void __launch_bounds__(GeoH<N>::THREADS2) k_pass2_h(const __grid_cons
     constexpr int i = decltype(i_)::value;
     v[i] = xs[t + T * i];
   });
-  F::template run<-1>(v, xs, g.twN, t);
+  F::template run<kColDir<-1, N, BF>>(v, xs, g.twN, t);
   // v[i] = X[2J k + j], k = t + 16 i
   const float* cc = g.chat + (size_t)vcol * 2 * N + j * H;
   SFor<0, P>::run([&](auto i_) {
@@ -593,7 +598,7 @@ __global__ void __launch_bounds__(GeoH<N>::THREADS2) k_pass2_h(const __grid_cons
     const float f = __ldg(&cc[t + T * i]);
     v[i] = make_float2(v[i].x * f, v[i].y * f);
   });
-  F::template run<1>(v, xs, g.twN, t);
+  F::template run<kColDir<1, N, BF>>(v, xs, g.twN, t);
   __syncwarp();  // the transform's last exchange reads are done
   SFor<0, P>::run([&](auto i_) {
     constexpr int i = decltype(i_)::value;
@@ -609,11 +614,11 @@ __global__ void __launch_bounds__(GeoH<N>::THREADS2) k_pass2_h(const __grid_cons
       if constexpr (i > 0) e[i] = cmulc(e[i], w[2 * i]);
       o[i] = cmulc(sm[(2 * i + 1) * F::SMEM + m], w[2 * i + 1]);
     });
-    reg_dft<J, 1, float2>(e);
-    reg_dft<J, 1, float2>(o);
+    reg_dft<J, kColDir<1, N, BF>, float2>(e);
+    reg_dft<J, kColDir<1, N, BF>, float2>(o);
     SFor<0, J>::run([&](auto q_) {
       constexpr int q = decltype(q_)::value;
-      IO::st(p, m + q * H, cadd(e[q], twmul<q, J2, 1>(o[q])));
+      IO::st(p, m + q * H, cadd(e[q], twmul<q, J2, kColDir<1, N, BF>>(o[q])));
     });
   }
 }

@@ -146,3 +146,24 @@ def test_prior_keeps_a_bad_voxel_to_its_neighbours(bad):
     want[r - 1:r + 2, c - 1:c + 2] = True
     for z in (0, 2):
         assert np.array_equal(~np.isfinite(G[z]), want)
+
+
+def test_operator_error_at_1536():
+    # the transforms of this side came with 2.58e-7 from their first form (four radix stages) on these
+    # inputs, its error against 64 bits; any other form has to stay there
+    N, S, na = 1536, 4, 64
+    ctx = tm.Context([tm.Group(N=N, angles=[math.pi * a / na for a in range(na)], n_slices=S)])
+    ctx.build_operator(torch.zeros(S * na * N, device="cuda"))
+    K = ctx.kernel(0).reshape(2 * N - 1, 2 * N - 1)
+    torch.cuda.synchronize()
+    C = torch.zeros(2 * N, 2 * N, device="cuda", dtype=torch.float64)
+    i = torch.arange(-(N - 1), N, device="cuda") % (2 * N)
+    C[i[:, None], i[None, :]] = K
+    spec = torch.fft.rfft2(C).real
+    errs = []
+    for seed in (0, 1):
+        x = torch.randn(S, N, N, device="cuda", generator=torch.Generator(device="cuda").manual_seed(seed))
+        z = ctx.normal_apply(x.reshape(-1)).reshape(S, N, N).double()
+        ref = torch.fft.irfft2(torch.fft.rfft2(x.double(), s=(2 * N, 2 * N)) * spec, s=(2 * N, 2 * N))[:, :N, :N]
+        errs.append(float((z - ref).norm() / ref.norm()))
+    assert np.mean(errs) < 2.58e-7, errs
