@@ -897,24 +897,25 @@ void nufft_psi_table(int nmodes, int nfine, int w, double beta, std::vector<doub
   gauss_legendre(4 * w + 40, x, wt);
   const int off = (nmodes % 2 == 1) ? (nmodes - 1) / 2 : nmodes / 2;
   out.assign(nmodes, 0.0);
-  // per node, cos(d theta) by rotation, restarted from the library's sine and cosine every 32 modes (the
-  // rotations add about 32 units of roundoff), for d >= 0: the table is even in d
+  // per node, cos(d theta) for d >= 0 (the table is even in d) with d = 32 a + b as the product of the library's
+  // values at 32 a theta and at b theta.  The smallest value of the widest table is 1/630 of the largest and its error,
+  // against 40 digits, 5e-14 of it at 2048 (7e-14 with one library cosine per mode, 16e-14 by rotation)
+  double cb[32], sb[32];
   for (size_t q = 0; q < x.size(); ++q) {
     const double t = 1.0 - x[q] * x[q];
     const double f = 0.5 * w * wt[q] * (t > 0 ? exp(beta * (sqrt(t) - 1.0)) : 0.0);
     const double theta = 2.0 * M_PI * (0.5 * w * x[q]) / nfine;
-    const double cr = cos(theta), sr = sin(theta);
-    double c = 1.0, s = 0.0;
-    for (int d = 0; d <= off; ++d) {
-      if (d % 32 == 0) {
-        c = cos(d * theta);
-        s = sin(d * theta);
+    for (int i = 0; i < 32; ++i) {
+      cb[i] = cos(i * theta);
+      sb[i] = sin(i * theta);
+    }
+    for (int d0 = 0; d0 <= off; d0 += 32) {
+      const double ca = f * cos(d0 * theta), sa = f * sin(d0 * theta);
+      for (int d = d0; d <= std::min(off, d0 + 31); ++d) {
+        const double v = ca * cb[d - d0] - sa * sb[d - d0];
+        out[off - d] += v;
+        if (d > 0 && off + d < nmodes) out[off + d] += v;
       }
-      out[off - d] += f * c;
-      if (d > 0 && off + d < nmodes) out[off + d] += f * c;
-      const double cn = c * cr - s * sr;
-      s = s * cr + c * sr;
-      c = cn;
     }
   }
 }
