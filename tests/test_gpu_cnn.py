@@ -201,3 +201,25 @@ def test_backward_not_finite(orc, where, pos, value):
     assert 0 < np.isfinite(rgp).sum() < rgp.size
     assert np.array_equal(np.isfinite(gp), np.isfinite(rgp))
     assert np.array_equal(np.isfinite(gin.cpu().numpy().reshape(rgin.shape)), np.isfinite(rgin))
+
+
+# more tiles than blocks (456 of the convolutions, 304 of the weight gradients), so that blocks stage, multiply
+# and store several: 616 and 620 tiles of 4 x 128 pixels, 308 and 312 of 8 x 128, the last of a row and of a
+# column partial
+@pytest.mark.parametrize("B,H,W", [(2, 1230, 35), (2, 620, 131)])
+def test_several_tiles_per_block(orc, B, H, W):
+    # ReLU decisions as in test_backward_matches_oracle: the pre-activations' BF16 error is below 0.03
+    rng = np.random.default_rng(4)
+    p = robust_params(orc, 3)
+    x = rng.uniform(-0.5, 0.5, (B, H, W)).astype(np.float32)
+    gout = rng.standard_normal((B, H, W)).astype(np.float32)
+    net = tm.CNN(H, W, max_batch=B)
+    net.set_weights(p)
+    out = net.net_forward(dev(x), B)
+    torch.cuda.synchronize()
+    ref = orc.cnn_forward(x.astype(np.float64), p)
+    assert rel(out.cpu().numpy().reshape(ref.shape), ref) < 2e-2
+    check_backward(orc, p, x, gout, 2e-2)
+    runs = [net.net_backward(dev(x), dev(gout), B) for _ in range(2)]
+    torch.cuda.synchronize()
+    assert np.array_equal(runs[0][0], runs[1][0]) and torch.equal(runs[0][1], runs[1][1])

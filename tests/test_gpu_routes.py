@@ -167,3 +167,32 @@ def test_operator_error_at_1536():
         ref = torch.fft.irfft2(torch.fft.rfft2(x.double(), s=(2 * N, 2 * N)) * spec, s=(2 * N, 2 * N))[:, :N, :N]
         errs.append(float((z - ref).norm() / ref.norm()))
     assert np.mean(errs) < 2.58e-7, errs
+
+
+# the general exponent in the bands of four and of eight rows, with several column blocks (pairs across a
+# block's outer columns) and chunks of slices
+@pytest.mark.parametrize("N,S,p,q", [(256, 2, 1.1, 1.8), (512, 3, 1.1, 1.8), (512, 2, 1.5, 3.0), (1024, 5, 1.2, 1.8)])
+def test_prior_bands_general_q(orc, N, S, p, q):
+    x = synth.random_image(np.random.default_rng(N + S), (S, N, N))
+    prm = dict(p=p, q=q, c=0.01, sigma=0.1)
+    G = _prior_gradient(x, prm, 1e12)
+    ref = orc.prior(x.astype(np.float64), orc.Prior(**prm, lam=1e12))[0]
+    assert rel(G, ref) < 1e-5
+
+
+# R*g beside the bound that its FP32 storage sets (2.5e-8 of the norm): several hundred angles, whose rows at
+# the grid's centre are shared by a warp, and the corner pixels, whose deconvolution factors are the largest
+# and where the spreading kernel's own error, about 1e-7, is too
+def test_atg_error_and_corners(orc):
+    na = 400
+    for N in (128, 1024):
+        p = synth.volume(S=1, N=N, n_angles=na, n_ellipsoids=4, seed=N)
+        g = p.sino.astype(np.float64)
+        ctx = tm.Context([tm.Group(N=N, angles=list(p.theta), n_slices=1)])
+        atg = host(ctx.build_operator(dev(p.sino)), (N, N))
+        rms = np.sqrt(np.mean(atg ** 2))
+        if N == 128:
+            assert rel(atg, orc.adjoint(g, N, p.theta)[0]) < 5e-8
+        at = [0, 1, 2, 3, N - 4, N - 3, N - 2, N - 1]
+        err = max(abs(atg[r, c] - orc.adjoint_point(g[0], N, p.theta, r, c)) for r in at for c in at)
+        assert err < 2.5e-7 * rms, (N, err / rms)
