@@ -121,12 +121,13 @@ __global__ void __launch_bounds__(640) k_fft_rows(C* data, int n, unsigned plan,
   stage(std::false_type{}, std::true_type{});
 }
 
-// In-place variant for rows whose two Stockham buffers do not fit in shared memory: the row
-// is loaded in bit-reversed order, then log2(n) radix-2 decimation-in-time stages (twiddles stage by
+// In-place variant for rows whose two Stockham buffers do not fit in shared memory (FP64 only: K's rows of
+// 8192 at 2048): the row is loaded in bit-reversed order, then log2(n) radix-2 decimation-in-time stages (twiddles stage by
 // stage, R = 2).
-template <int DIR, class C>
-__global__ void __launch_bounds__(1024) k_fft_rows_inplace(C* data, int n, int log2n, size_t stride,
-                                                           const C* __restrict__ tw) {
+template <int DIR>
+__global__ void __launch_bounds__(1024) k_fft_rows_inplace(double2* data, int n, int log2n, size_t stride,
+                                                           const double2* __restrict__ tw) {
+  using C = double2;
   extern __shared__ unsigned char smraw[];
   C* X = reinterpret_cast<C*>(smraw);
   C* row = data + (size_t)blockIdx.x * stride;
@@ -223,20 +224,23 @@ static int fft_rows(C* data, int n, int rows, int dir, const C* tw, cudaStream_t
     static_assert(kMax <= 227 * 1024, "two padded rows");
     TMBIR_CUDA(cudaFuncSetAttribute(k_fft_rows<-1, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax));
     TMBIR_CUDA(cudaFuncSetAttribute(k_fft_rows<1, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMax));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_fft_rows_inplace<-1, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    kRowSmem));
-    TMBIR_CUDA(cudaFuncSetAttribute(k_fft_rows_inplace<1, C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    kRowSmem));
+    if constexpr (std::is_same<C, double2>::value) {
+      TMBIR_CUDA(cudaFuncSetAttribute(k_fft_rows_inplace<-1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmem));
+      TMBIR_CUDA(cudaFuncSetAttribute(k_fft_rows_inplace<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRowSmem));
+    }
     attr_set = true;
   }
   if (const size_t one = (size_t)n * sizeof(C); 2 * one > kRowSmem) {
-    if (one > kRowSmem || (n & (n - 1)) != 0) return set_error(TMBIR_ERR_SHAPE, "setup FFT length too large");
-    if (dir < 0)
-      k_fft_rows_inplace<-1, C><<<rows, 1024, one, s>>>(data, n, ilog2(n), (size_t)n, tw);
-    else
-      k_fft_rows_inplace<1, C><<<rows, 1024, one, s>>>(data, n, ilog2(n), (size_t)n, tw);
-    TMBIR_CHECK_LAUNCH();
-    return TMBIR_OK;
+    if constexpr (std::is_same<C, double2>::value) {
+      if (one > kRowSmem || (n & (n - 1)) != 0) return set_error(TMBIR_ERR_SHAPE, "setup FFT length too large");
+      if (dir < 0)
+        k_fft_rows_inplace<-1><<<rows, 1024, one, s>>>(data, n, ilog2(n), (size_t)n, tw);
+      else
+        k_fft_rows_inplace<1><<<rows, 1024, one, s>>>(data, n, ilog2(n), (size_t)n, tw);
+      TMBIR_CHECK_LAUNCH();
+      return TMBIR_OK;
+    }
+    return set_error(TMBIR_ERR_SHAPE, "setup FFT length too large");
   }
   const unsigned plan = fft_plan(n);
   const int threads = std::min(((n + 7) / 8 + 31) / 32 * 32, 640);

@@ -143,29 +143,6 @@ __device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) { return _
 __device__ __forceinline__ float2 f2mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 f2add(float2 a, float2 b) { return __fadd2_rn(a, b); }
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Block reduction of kParts values to partials[block]: fixed order, FP64.
-template <int W>
-__device__ __forceinline__ void block_partials(double (&acc)[kParts], double* red, double* out) {
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int j = 0; j < kParts; ++j) {
-    double v = warp_sum(acc[j]);
-    if (lane == 0) red[warp * kParts + j] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < kParts) {
-    double s = 0.0;
-    for (int w = 0; w < W; ++w) s += red[w * kParts + threadIdx.x];
-    out[threadIdx.x] = s;
-  }
-}
-
 // the row passes' rotations keep the remainder of 1/sqrt(2) (twmul), except beside BF16 spectra, whose
 // rounding is 2^15 times larger
 template <int DIR, bool BF>
