@@ -26,8 +26,6 @@ PriorC make_prior(const tmbir_params& p) {
   c.p = (float)p.p;
   c.q = (float)p.q;
   c.qp = (float)(p.q - p.p);
-  c.inv_csig = (float)(1.0 / (p.c * p.sigma));
-  c.inv_sig = (float)(1.0 / p.sigma);
   c.inv_sig2 = (float)(1.0 / (p.sigma * p.sigma));
   c.lam = (float)p.lambda;
   const double total = 6.0 + 12.0 / std::sqrt(2.0) + 8.0 / std::sqrt(3.0);
@@ -36,7 +34,6 @@ PriorC make_prior(const tmbir_params& p) {
   c.wc = (float)(1.0 / std::sqrt(3.0) / total);
   c.q_is_2 = p.q == 2.0 ? 1 : 0;
   c.nonneg = p.nonneg ? 1 : 0;
-  c.l2_inv_csig = (float)std::log2(1.0 / (p.c * p.sigma));
   c.qp_l2_inv_csig = (float)((p.q - p.p) * std::log2(1.0 / (p.c * p.sigma)));
   c.l2_inv_sig = (float)std::log2(1.0 / p.sigma);
   // |y| <= pair_lim keeps (d / (c sigma))^(q-p) of a difference, |d| <= 2 pair_lim, below 2^62 and d^2 below 2^126

@@ -69,12 +69,9 @@ inline size_t state_header_bytes(int n_groups) {
 // qGGMRF constants in the form the kernels use.
 struct PriorC {
   float p, q, qp;        // exponents and q - p
-  float inv_csig;        // 1 / (c sigma)
-  float inv_sig;         // 1 / sigma
   float inv_sig2;        // 1 / sigma^2
   float lam;             // lambda
   float wf, we, wc;      // face / edge / corner neighbour weights (sum of the 26 is 1)
-  float l2_inv_csig;     // log2(1 / (c sigma))
   float qp_l2_inv_csig;  // (q - p) log2(1 / (c sigma))
   float l2_inv_sig;      // log2(1 / sigma)
   int q_is_2;
