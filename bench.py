@@ -442,7 +442,7 @@ def time_to_gap_hier(tm, H, sino, F_ref, F0, stream, barrier, world, step_ms, st
     forms["chosen"] = {"ms": step_ms, "finest_iterations": step_stats[-1].iterations,
                        "level_iterations": [s.iterations for s in step_stats], "gap_reached": step_stats[-1].gap,
                        "reached": step_stats[-1].gap <= GAP, "used_cnn": H.used_cnn,
-                       "form": "the bench step: levels N/4, N/2, N (R*g in FP32 at the coarse levels, FP64 at N), "
+                       "form": "the bench step: levels N/4, N/2, N (R*g in FP32 at the coarse levels, double-word FP32 at N), "
                                "CNN-refined FBP start at N/4 (FBP fallback), "
                                f"BF16 spectra with FP32 refinement from gap {REFINE_GAP:g}, device-driven graph loops"}
     forms["single_slice"] = single_slice_form(tm, w, H.theta, sino, stream, barrier, world)
@@ -536,9 +536,11 @@ def pass_bytes(N):
     return [8.0 + 8.0 * B, 16.0 * B, 8.0 * B + 4.0, 4.0 + 4 + 8 + 4]
 
 
-# special-function operations per voxel of pass 3b: 13 neighbour pairs (each unordered pair of the
-# 26-neighbourhood once) x (log2, exp2, reciprocal)
-SFU_OPS_PER_VOXEL = 13 * 3
+# special-function work per voxel of pass 3b in units of one exp2: 13 neighbour pairs (each unordered pair
+# of the 26-neighbourhood once) x (a log2, which issues at half exp2's rate; an exp2; half a reciprocal,
+# shared by two pairs, at half the rate).  The measured rate is exp2's: its chains of log2, exp2 and a
+# reciprocal that the compiler folds into the exp2 count three operations in the time of three exp2.
+SFU_OPS_PER_VOXEL = 13 * 4
 
 
 def roofline_of(pt, iters, S, N, workload, sfu_rate=None):
@@ -572,7 +574,7 @@ def roofline_of(pt, iters, S, N, workload, sfu_rate=None):
         sf = per[name]["sfu"]
         if SFU_OPS_PER_VOXEL / sfu_rate > bpv[top] / (peak * 1e9):
             roof.update({"bound": "alu", "achieved": sf["achieved_gops"], "peak": sf["peak_gops"], "unit": "Gop/s",
-                         "frac": sf["frac"], "peak_source": "measured: tmbir_sfu_rate (log2/exp2/reciprocal chains)",
+                         "frac": sf["frac"], "peak_source": "measured: tmbir_sfu_rate (log2/exp2 chains, in units of exp2)",
                          "hbm": {"achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak}})
     return roof
 
@@ -653,8 +655,7 @@ def run_ours(args, tm, w, prob, stream, rank, world, local, barrier, extra):
         extra["F_ref"] = {"value": F_ref, "F0": F0, "finest_iterations": REF_ITERS,
                           "change_last_half_in_gap_units": (log[REF_ITERS // 2 - 1][0] - F_ref) / (F0 - F_ref),
                           "s": time.perf_counter() - t0}
-        # launch shapes of every level by timing (pass-3b slices per block, spectrum chunk, rows
-        # per block of the row passes where a side has variants)
+        # launch shapes of every level by timing (pass-3b slices per block, spectrum chunk)
         extra["autotune"] = [{"N": c.groups[0].N, "pass3_slices_per_block": c.autotune(c._lv["x"], c._lv["atg"],
                                                                                        tm_params()),
                               "spectrum_chunk": c.spec_chunks} for c in H.ctxs]

@@ -177,9 +177,9 @@ int tmbir_set_angle_weights(tmbir_ctx* ctx, int group, const double* h_w);
  * [slice][row][col]; 1/2 g.g per group; lambda_max(R*R) by 100 power steps (kept in the
  * workspace).  d_sino is [slice][angle][bin] for all groups back to back.  K, its spectrum and
  * the reductions in FP64; R*g (the type-1 NUFFT of Eq. 4 on a 1.25x grid) in double-word FP32
- * arithmetic (hi + lo pairs of FP32, a 48-bit significand: FP64-class accuracy, about 1e-10
- * relative before the FP32 store) on the FP32 pipe, whose rate on GB300 is far above the FP64
- * pipe's.
+ * arithmetic (hi + lo pairs of FP32, a 48-bit significand; 6e-9 to 8e-9 relative L2 before the
+ * FP32 store, the spreading kernel's own error) on the FP32 pipe, whose rate on GB300 is far above
+ * the FP64 pipe's.
  */
 int tmbir_build_operator(tmbir_ctx* ctx, const float* d_sino, float* d_atg);
 

@@ -308,7 +308,7 @@ class Context:
         _check(_lib.tmbir_set_angle_weights(self._h, int(group), w))
 
     def build_operator(self, sino, atg=None, fp64: bool = True):
-        """K, its spectrum, lambda_max, 1/2 g.g and R*g (FP64, or FP32 with fp64=False)."""
+        """K, its spectrum, lambda_max, 1/2 g.g and R*g (double-word FP32, or FP32 with fp64=False)."""
         atg = self._empty(self.image_numel()) if atg is None else atg
         self._pre()
         fn = _lib.tmbir_build_operator if fp64 else _lib.tmbir_build_operator_fp32
@@ -611,7 +611,7 @@ def reconstruct_levels(N: int, angles, n_slices: int, sino, levels: int, params,
     coarser levels iterate; the contexts must then have distinct streams (created here when
     `ctxs` is None).  Without it all levels share one stream and run one after another.  With
     coarse_setup_fp32 the levels below the finest build their R*g in FP32
-    (tmbir_build_operator_fp32); the finest level's is FP64 either way.
+    (tmbir_build_operator_fp32); the finest level's is the double-word one either way.
     Returns the finest image, the level contexts and the per-level Stats.
     """
     import torch

@@ -540,7 +540,7 @@ int tmbir_build_operator_fp32(tmbir_ctx* ctx, const float* d_sino, float* d_atg)
   return TMBIR_OK;
 }
 
-// build_operator and fbp in one call: R*g (FP64) on the context stream while the FBP start
+// build_operator and fbp in one call: R*g (double-word FP32) on the context stream while the FBP start
 // (FP32, its own scratch) runs on a second stream, joined before the call returns its work.
 int tmbir_build_operator_fbp(tmbir_ctx* ctx, const float* d_sino, float* d_atg, float* d_x0) {
   TMBIR_TRACE("tmbir_build_operator_fbp");

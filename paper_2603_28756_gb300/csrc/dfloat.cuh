@@ -4,19 +4,23 @@
 // operation is accurate to about 2^-44 of its operands' magnitude (FP64 carries 2^-53).  The
 // transforms that use it (the NUFFT adjoint of Eq. 4: the sparse gather onto the spreading grid,
 // the 2D grid FFT, the deconvolution) then run on the FP32 pipe, whose rate on GB300 is
-// sixty-four times the FP64 pipe's; their result is stored in FP32, whose 2^-24 is far above the
-// double-word error even after the deconvolution's amplification (about 5e5 at the image
-// corners on the 1.25x grid).
+// sixty-four times the FP64 pipe's; their result is stored in FP32.  At the image corners the
+// deconvolution amplifies by 4e5 (1.25x grid), and 4e5 * 2^-44 is half of FP32's 2^-24, so the bound alone
+// leaves no margin there; measured against 64 bits, the corners' largest error is 1.2e-7 of the image's rms
+// (64^2 to 2560^2, 30 to 1000 angles), which is the spreading kernel's own error: it was the same with
+// every operation renormalised and the deconvolution in FP64.
 //
 // The building blocks are the error-free transformations of floating-point arithmetic: Knuth's
 // TwoSum (the exact rounding error of a sum) and the FMA-based TwoProduct (the exact rounding error
 // of a product, fma(a, b, -ab)).  A sum adds the high parts by TwoSum and the low parts and the error
 // in FP32; a product keeps hi * hi exactly and adds the two cross products to its error.  Neither
-// renormalises the pair (three operations each): the low part then stays within a few units of the
-// high parts' last place, so that its own rounding is 2^-46 of the operands, and settle()
-// renormalises once per butterfly (R*g's error stays at 2.5e-8 to 2.7e-8 of its norm).  The errors
-// are bounded relative to the operands' magnitudes, not to the result's, which is the bound an FFT or
-// a dot product needs (their errors are judged against the input's norm).  Every step uses the _rn
+// renormalises the pair (three operations each).  The low part then stays within a few units in the last
+// place of the largest operand since settle() last renormalised (once per butterfly, once per row of
+// the gather), and its own rounding within 2^-46 of that operand; it is not bounded by the high part,
+// which a cancellation can make as small as it likes.  So the errors are bounded relative to the
+// operands' magnitudes, not to the result's, which is the bound an FFT or a dot product needs (their
+// errors are judged against the input's norm): R*g's error is 2.6e-8 to 2.7e-8 of its norm, of which FP32
+// storage alone makes 2.5e-8 to 2.6e-8.  Every step uses the _rn
 // intrinsics, which the compiler never contracts into FMAs, so the transformations stay error-free.
 #pragma once
 #include <cuda_runtime.h>

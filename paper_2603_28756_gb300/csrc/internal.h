@@ -99,13 +99,13 @@ struct GroupDev {
   const double* wts;   // [na] per-angle weights of the data term (nullptr: all 1)
   double* lam_max;     // device scalar
   double* gtg;         // device scalar (1/2 g.g of the group)
-  // sparse spreading operators (geometry only): sp[0] for the FP32 paths, sp[1] for R*g in FP64
+  // sparse spreading operators (geometry only): sp[0] for the FP32 paths, sp[1] for R*g
   struct Spread {
     int nf;            // periodic grid side
     double* psi;       // [N] deconvolution factors (the kernel's Fourier transform at the image modes)
     int* ptr;          // [nf^2 + 1] rows of grid cells
     int* idx;          // [nnz] strength index a * n_det + (k mod n_det)
-    double* wt;        // [nnz] kernel weight
+    double* wt;        // [nnz] kernel weight (sp[1]: as an (hi, lo) pair of FP32 in the double's place)
   } sp[2];
   float* kz;           // [S][N][N] K (*) y between passes 3a and 3b
   int zc;              // slices each pass-3 block marches through (0: the default rule)
@@ -150,11 +150,11 @@ inline int spec_chunk(const GroupDev& g) { return g.sc > 0 && g.sc < g.S ? g.sc 
 // relative error of R* about 1e-9 / 1e-8):
 //   0, the FP32 paths (FBP start, forward and adjoint projections): a 2N x 2N grid, width 10,
 //      beta 2.30 per unit width;
-//   1, R*g in FP64: a 5N/4 x 5N/4 grid (2^a 3^b 5^c for every supported side), width 14,
-//      beta = 0.97 pi (1 - 1/(2 * 1.25)) per unit width.  The smaller grid cuts the FP64 grid
-//      FFTs, which dominate the setup, to 0.37x for 1.96x the sparse gather; dividing by the
-//      kernel's Fourier transform amplifies rounding towards the image corners (up to ~5e5 at
-//      1.25, 13 at 2), harmless in FP64 but not in FP32, hence two configurations.
+//   1, R*g in double-word FP32: a 5N/4 x 5N/4 grid (2^a 3^b 5^c for every supported side), width 14,
+//      beta = 0.97 pi (1 - 1/(2 * 1.25)) per unit width.  The smaller grid cuts the grid FFTs to
+//      0.37x for 1.96x the sparse gather; dividing by the kernel's Fourier transform amplifies
+//      rounding towards the image corners (up to 4e5 at 1.25, 13 at 2), which 48 bits bear
+//      (dfloat.cuh) but not 24, hence two configurations.
 constexpr int kSpreadWidth[2] = {10, 14};
 inline int spread_grid(int k, int N) { return k ? N * 5 / 4 : 2 * N; }
 inline double spread_beta(int k) { return k ? 0.97 * 3.14159265358979323846 * (1.0 - 1.0 / 2.5) * 14 : 2.30 * 10; }

@@ -27,8 +27,8 @@ namespace tmbir {
 //   reads contiguous values, and the stages together need n of them;
 //   the buffers have one value of padding per 128 bytes (the first stage's stores are 8 apart);
 //   the first stage reads and the last one writes global memory.
-// R*g and the FBP start of 16 x 2048^2 together: 6.5 -> 5.6 ms; rows of 4 x 512^2: FP32 37 -> 25 us,
-// double-word 38 -> 34 us.
+// R*g and the FBP start of 16 x 2048^2 together: 6.5 -> 5.6 ms, and 5.36 with the first and last stage known
+// at compile time (stockham_stage).
 
 // index i of a padded row buffer
 template <class C>
@@ -316,8 +316,8 @@ __global__ void k_fixed_to_complex(const unsigned long long* __restrict__ in, do
 }
 
 // ---------------------------------------------------------------- sparse spreading operator
-// The polar sample positions depend on the geometry only, so the spreading onto the 2N x 2N
-// grid of R*g and of the FBP start is stored once as a sparse matrix in compressed rows, one
+// The polar sample positions depend on the geometry only, so the spreading onto the grids of the FBP
+// start (2N x 2N) and of R*g (5N/4 x 5N/4) is stored once, as a sparse matrix each in compressed rows, one
 // row per grid cell: the strength index a * n_det + (k mod n_det) of every contributing
 // sample and its kernel weight psi(x) psi(y).  Entries of a row are sorted by strength index,
 // so every later gather sums in a fixed order (deterministic) and needs no atomics.
@@ -594,8 +594,8 @@ __device__ __forceinline__ void gather_row(int j0, int e, int step, const int* _
 // the lanes' sums are added in a fixed tree: one thread's chain through the longest row was the time
 // of the whole launch (4 x 512^2, 181 angles: 1.19 -> 0.60 ms; 8 x 2048^2, 128 angles, with the
 // compensated sums: 1.80 -> 0.96 ms).  The FP32 sums of the start keep one
-// thread's order: their chain is four times shorter per entry, and another order would move the
-// start by 4e-7 of its norm, which BF16 iterations after it amplify.
+// thread's order (4 x 512^2: 0.32 ms, 0.23 with shared rows): another order would move the start by 4e-7
+// of its norm, which BF16 iterations after it amplify.
 constexpr int kLongRow = 96;
 template <int B, class C>
 __global__ void __launch_bounds__(256) k_csr_gather(const int* __restrict__ ptr, const int* __restrict__ idx,

@@ -10,7 +10,8 @@
 //   pass 2  columns: per column v, FFT of length 2N of the N nonzero rows, multiply by the
 //                    real kernel spectrum, inverse FFT, keep the first N rows (the crop).
 //                    The length-2N transforms are split into their even and odd halves, two
-//                    length-N transforms each, so the zero padding and the crop cost nothing.
+//                    length-N transforms each (above 1024 into 2N/512 of 512 points), so the
+//                    zero padding and the crop cost nothing.
 //   pass 3a rows:    inverse real FFT of each row, keep the first N columns -> K (*) y.
 //   pass 3b stencil: per voxel G = K(*)y - R*g + lambda grad Phi(y) (each neighbour pair of the
 //                    26-neighbourhood evaluated once), x_{k+1} = y - G/L, and the partial sums
@@ -380,7 +381,8 @@ __global__ void TMBIR_P3A_BOUNDS(Geo3a<N>::THREADS) k_pass3a(const __grid_consta
 // A shared-memory round trip carries the values between the J-point DFTs (threads along m) and the
 // group FFTs (one per j), and one more is inside each group FFT.
 //
-// Bound by the shared-memory / L1 data pipe (75 % busy in all three), so its wavefronts are what the
+// Bound by the shared-memory / L1 data pipe (72, 69 and 50 % busy in passes 1, 2 and 3a at 2048; 3a, one
+// block per SM, also waits for its gather), so its wavefronts are what the
 // layouts save: twiddles come from tables that are contiguous in m (W^m, W^2m, W^4m, W^8m; the others
 // are one product of two of these), the kernel spectrum is stored per j, and for J = 4 a staged row
 // keeps the four residues of v apart (stride-4 accesses would meet in four banks).  Measured per
@@ -410,9 +412,11 @@ struct GeoH {
 };
 
 // Pass 3a gathers eight rows (64-byte segments of the column-major spectrum, half the load
-// wavefronts of four): 582 against 647 us at 32 x 2048^2, 96 against 112 us at 8 x 1536^2, except at
-// 2560, where eight rows leave one block per SM (190 against 179 us); pass 1, whose stores need no
-// registers while they are in flight, keeps four and more blocks per SM (540 against 636 us at 2048).
+// wavefronts of four): 582 against 647 us at 32 x 2048^2, 96 against 112 us at 8 x 1536^2.  Not at 2560:
+// 40 group FFTs are a block of 640 threads and 169 KB, the only one of its SM, which measured 190 us
+// against 179 with two blocks of 320 threads and four rows (at 2048 eight rows are one block of 512 threads
+// as well, and still win).  Pass 1, whose stores need no registers while they are in flight, keeps four
+// rows and three blocks per SM (540 against 636 us at 2048).
 template <int N>
 using GeoH3 = GeoH<N, N == 2560 ? 4 : 8>;
 
@@ -717,7 +721,8 @@ __global__ void __launch_bounds__(GeoH3<N>::THREADS) k_pass3a_h(const __grid_con
 // log2, 32 exp2 and 16 reciprocals per clock and SM), the FMA pipe about 25.  The two halves share
 // one reciprocal (r_x = e_y / (e_x e_y)); with one each the kernel ran at the unit's rate (40 cycles a
 // pair).  Measured at 32 x 2048^2: 1.64 ms with neighbouring columns in a pair, 1.36 with the two
-// bands, 1.29 with the shared reciprocal and eight-row bands; at 64 x 1024^2 0.87, 0.77 and 0.69 ms.
+// bands, 1.30 with the shared reciprocal and eight-row bands; at 64 x 1024^2 0.87, 0.77 and 0.70 ms.
+// At 8 x 2048^2 62 % of the issue slots, the FMA pipe 47 % and the unit 58 % (32 cycles per packed pair).
 template <int N>
 struct GeoP {
   static_assert(N % 64 == 0, "a warp owns 32 columns, a block at least two warps");
