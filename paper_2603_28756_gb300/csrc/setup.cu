@@ -27,8 +27,8 @@ namespace tmbir {
 //   reads contiguous values, and the stages together need n of them;
 //   the buffers have one value of padding per 128 bytes (the first stage's stores are 8 apart);
 //   the first stage reads and the last one writes global memory.
-// R*g and the FBP start of 16 x 2048^2 together: 6.5 -> 5.6 ms, and 5.36 with the first and last stage known
-// at compile time (stockham_stage).
+// R*g and the FBP start of 16 x 2048^2 together: 6.5 -> 5.6 ms, and 5.36 with the first stage known at
+// compile time (stockham_stage).
 
 // index i of a padded row buffer
 template <class C>
@@ -39,11 +39,15 @@ template <class C>
 constexpr size_t padded_bytes(size_t n) {
   return (n + n / (128 / sizeof(C)) + 1) * sizeof(C);
 }
-// FIRST: the input is `row`, else X; LAST: the output is `row`, else Y.  As arguments instead of template
-// parameters they left rows of 64 to 512 points slower than whole-row copies in and out would (512 rows of
-// 128 points: 6.3 us, with template parameters 4.6; 4096 rows of 2048: 23.7 and 19.2).
-template <int R, int DIR, bool FIRST, bool LAST, class C>
-__device__ __forceinline__ void stockham_stage(const C* X, C* Y, C* row, int n, int Ls, const C* __restrict__ tw) {
+// FIRST: the input is `row`, else X; last (a bool or an integral_constant): the output is `row`, else Y.
+// With FIRST as an argument a thread's loads were not issued together, and rows of 64 to 512 points were
+// slower than with whole-row copies in and out (512 rows of 128 points: 6.3 us, so 4.6; 4096 rows of 2048: 23.7
+// and 19.2).  `last` is known at compile time in FP32 (adjoint of 512 x 64^2: 4.98 ms, so 4.91) and an argument
+// otherwise, which leaves a double-word row 48 registers instead of 80 and so two blocks of a 3200-point
+// row per SM (R*g of 1 x 2560^2: 930 us, so 824; 512 x 64^2: 9.77 ms and 9.65).
+template <int R, int DIR, bool FIRST, class Last, class C>
+__device__ __forceinline__ void stockham_stage(const C* X, C* Y, C* row, Last last, int n, int Ls,
+                                               const C* __restrict__ tw) {
   const int nb = n / R;
   for (int j = threadIdx.x; j < nb; j += blockDim.x) {
     const int k = j % Ls;  // Ls is a product of mixed radices
@@ -62,7 +66,7 @@ __device__ __forceinline__ void stockham_stage(const C* X, C* Y, C* row, int n, 
 #pragma unroll
     for (int m = 0; m < R; ++m) {
       const C v = settle(a[m]);
-      if constexpr (LAST)
+      if (last)
         row[o + m * Ls] = v;
       else
         Y[padded<C>(o + m * Ls)] = v;
@@ -99,15 +103,15 @@ __global__ void __launch_bounds__(640) k_fft_rows(C* data, int n, unsigned plan,
   C* Y = X + padded_bytes<C>(n) / sizeof(C);
   C* row = data + (size_t)blockIdx.x * stride;
   int Ls = 1;
-  auto stage = [&](auto first_, auto last_) {
-    constexpr bool F = decltype(first_)::value, L = decltype(last_)::value;
+  auto stage = [&](auto first, auto last) {
+    constexpr bool F = decltype(first)::value;
     const int R = (int)(plan & 15u);
     switch (R) {
-      case 8: stockham_stage<8, DIR, F, L>(X, Y, row, n, Ls, tw); break;
-      case 4: stockham_stage<4, DIR, F, L>(X, Y, row, n, Ls, tw); break;
-      case 2: stockham_stage<2, DIR, F, L>(X, Y, row, n, Ls, tw); break;
-      case 3: stockham_stage<3, DIR, F, L>(X, Y, row, n, Ls, tw); break;
-      default: stockham_stage<5, DIR, F, L>(X, Y, row, n, Ls, tw); break;
+      case 8: stockham_stage<8, DIR, F>(X, Y, row, last, n, Ls, tw); break;
+      case 4: stockham_stage<4, DIR, F>(X, Y, row, last, n, Ls, tw); break;
+      case 2: stockham_stage<2, DIR, F>(X, Y, row, last, n, Ls, tw); break;
+      case 3: stockham_stage<3, DIR, F>(X, Y, row, last, n, Ls, tw); break;
+      default: stockham_stage<5, DIR, F>(X, Y, row, last, n, Ls, tw); break;
     }
     Ls *= R;
     plan >>= 4;
@@ -116,9 +120,14 @@ __global__ void __launch_bounds__(640) k_fft_rows(C* data, int n, unsigned plan,
     X = Y;
     Y = tmp;
   };
-  stage(std::true_type{}, std::false_type{});
-  while (plan >= 16u) stage(std::false_type{}, std::false_type{});
-  stage(std::false_type{}, std::true_type{});
+  if constexpr (std::is_same<C, float2>::value) {
+    stage(std::true_type{}, std::false_type{});
+    while (plan >= 16u) stage(std::false_type{}, std::false_type{});
+    stage(std::false_type{}, std::true_type{});
+  } else {
+    stage(std::true_type{}, plan < 16u);
+    while (plan != 0) stage(std::false_type{}, plan < 16u);
+  }
 }
 
 // In-place variant for rows whose two Stockham buffers do not fit in shared memory (FP64 only: K's rows of
